@@ -1,0 +1,174 @@
+// Select-and-sort of one row by one CTA: the kk best of n scored keys, in (score descending, index ascending) order.
+#pragma once
+
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "lt_common.cuh"
+
+namespace lt {
+
+// ---------------------------------------------------------------------------------------------
+// Distribution sort.  The scores are mapped monotonically to kFineBins bins over their own range, so that a bin of
+// the part that matters holds a handful of keys; one histogram and its prefix sum give every bin its place in the
+// output, every key up to the bin that holds the kk-th one is dropped into its bin's slots, and a key's final rank
+// is its bin's start plus the number of larger keys (full 64-bit keys: score, then index) in the same bin.  Two
+// shared-memory atomics and a few comparisons per key and seven barriers per row: latency-bound, which is why the
+// keys of a row are held in registers between the sweeps and three CTAs share an SM.  It replaces a least-significant-
+// digit radix sort (three to four passes of match.any ranking, ~40 barriers) preceded by a histogram select.  One B200, final
+// select of the whole chunk: 4096 rows of 2048 out of 3.4 k candidates 431 -> 137 us, out of 4.2 k 425 -> 153 us, 8192
+// rows 736 -> 235 us, one row 23 -> 13 us; 1024 rows with heavy-tailed scores 216 -> 48 us, of tie-ridden ones 187 -> 45 us.
+//
+// Two mappings are tried: equal-width bins in the score (bell-shaped tails, whole rows around zero), and equal-width bins in
+// the score's ordered bit pattern (heavy tails: the width then grows with the score).  Rows that crowd into few
+// bins under both - mass ties above all - are left to the caller: the function then returns false, on every
+// thread, without having written anything.
+//
+//   load(i)   score bits and index of the i-th key, i < n; called for i >= kFineBatch * kThreads only, several times
+//   c         the first kFineBatch * kThreads keys, key j * kThreads + tid in c[j] (anything past n)
+//   keys      key_cap 64-bit slots, bins: kFineBins counters (both shared memory)
+// ---------------------------------------------------------------------------------------------
+constexpr int kFineBins = 4096;
+constexpr int kFineBatch = 8;
+
+template <int kThreads, class Load>
+__device__ __forceinline__ bool fine_select_sort(const Load& load, uint2 (&c)[kFineBatch], unsigned int n, int kk, int topk,
+                                                 uint64_t* keys, unsigned int key_cap, unsigned int* bins, int32_t* out_idx,
+                                                 float* out_score, int n_keys, Control* ctl) {
+  constexpr int kWarps = kThreads / 32;
+  constexpr int kBinsPerThread = kFineBins / kThreads;
+  static_assert(kWarps <= 32 && kBinsPerThread % 4 == 0, "one warp combines the warps' results; bins are swept in 16-byte pieces");
+  __shared__ unsigned int s_min[kWarps], s_max[kWarps], s_sum[kWarps], s_cost[kWarps];
+  __shared__ unsigned int s_keep, s_last_bin;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const unsigned int batches = (n + kFineBatch * kThreads - 1) / (kFineBatch * kThreads);
+  // visits every key of this thread; the first batch comes from registers
+  auto sweep = [&](auto&& visit) {
+#pragma unroll
+    for (int j = 0; j < kFineBatch; ++j)
+      if (j * kThreads + tid < n) visit(c[j]);
+    for (unsigned int b = 1; b < batches; ++b) {
+      uint2 e[kFineBatch];
+#pragma unroll
+      for (int j = 0; j < kFineBatch; ++j) {
+        const unsigned int i = (b * kFineBatch + j) * kThreads + tid;
+        if (i < n) e[j] = load(i);
+      }
+#pragma unroll
+      for (int j = 0; j < kFineBatch; ++j)
+        if ((b * kFineBatch + j) * kThreads + tid < n) visit(e[j]);
+    }
+  };
+
+  // range of the scores, in ordered bit patterns
+  unsigned int kmin = 0xffffffffu, kmax = 0u;
+  sweep([&](uint2 e) {
+    const unsigned int k = score_to_key(e.x);
+    kmin = min(kmin, k);
+    kmax = max(kmax, k);
+  });
+  kmin = __reduce_min_sync(0xffffffffu, kmin);
+  kmax = __reduce_max_sync(0xffffffffu, kmax);
+  if (lane == 0) {
+    s_min[warp] = kmin;
+    s_max[warp] = kmax;
+  }
+  uint4* bins4 = reinterpret_cast<uint4*>(bins);
+  for (int attempt = 0; attempt < 2; ++attempt) {
+    for (int i = tid; i < kFineBins / 4; i += kThreads) bins4[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    if (attempt == 0) {
+      kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? s_min[lane] : 0xffffffffu);
+      kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? s_max[lane] : 0u);
+    }
+    const float fmax = __uint_as_float(key_to_score_bits(kmax)), fmin = __uint_as_float(key_to_score_bits(kmin));
+    const float fscale = static_cast<float>(kFineBins) / (fmax - fmin);
+    const unsigned int span = kmax - kmin;
+    const unsigned int kscale = span >= kFineBins ? static_cast<unsigned int>((static_cast<unsigned long long>(kFineBins) << 32) / (static_cast<unsigned long long>(span) + 1ull)) : 0u;
+    // bin 0 holds the best keys; both maps are monotone (a difference, a product and a conversion round monotonically)
+    auto bin_of_key = [&](unsigned int k) -> unsigned int {
+      if (attempt == 0) {
+        const float d = (fmax - __uint_as_float(key_to_score_bits(k))) * fscale;
+        return d < static_cast<float>(kFineBins - 1) ? static_cast<unsigned int>(d) : (d == d ? kFineBins - 1 : 0u);
+      }
+      return kscale != 0u ? __umulhi(kmax - k, kscale) : min(kmax - k, static_cast<unsigned int>(kFineBins - 1));
+    };
+    sweep([&](uint2 e) { atomicAdd(&bins[bin_of_key(score_to_key(e.x))], 1u); });
+    __syncthreads();
+    // starts of the bins, and the number of comparisons the bins up to the kk-th key will take
+    unsigned int cnt[kBinsPerThread], mine = 0;
+#pragma unroll
+    for (int j = 0; j < kBinsPerThread / 4; ++j) {
+      const uint4 v = bins4[tid * (kBinsPerThread / 4) + j];
+      cnt[4 * j] = v.x;
+      cnt[4 * j + 1] = v.y;
+      cnt[4 * j + 2] = v.z;
+      cnt[4 * j + 3] = v.w;
+      mine += v.x + v.y + v.z + v.w;
+    }
+    unsigned int incl = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned int o = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= d) incl += o;
+    }
+    if (lane == 31) s_sum[warp] = incl;
+    __syncthreads();
+    const unsigned int before = __reduce_add_sync(0xffffffffu, lane < warp ? s_sum[lane] : 0u);
+    unsigned int run = before + incl - mine;
+    unsigned int cost = 0;
+#pragma unroll
+    for (int j = 0; j < kBinsPerThread; ++j) {
+      const unsigned int m = cnt[j];
+      cnt[j] = run;
+      if (run < static_cast<unsigned int>(kk)) {
+        cost += min(m, 16383u) * min(m, 16383u);  // the sum stays below 2^32 for the largest capacity (12 * LT_MAX_TOPK keys)
+        if (run + m >= static_cast<unsigned int>(kk)) {  // exactly one bin
+          s_keep = run + m;
+          s_last_bin = tid * kBinsPerThread + j;
+        }
+      }
+      run += m;
+    }
+#pragma unroll
+    for (int j = 0; j < kBinsPerThread / 4; ++j)
+      bins4[tid * (kBinsPerThread / 4) + j] = make_uint4(cnt[4 * j], cnt[4 * j + 1], cnt[4 * j + 2], cnt[4 * j + 3]);
+    cost = __reduce_add_sync(0xffffffffu, cost);
+    if (lane == 0) s_cost[warp] = cost;
+    __syncthreads();
+    const unsigned int keep = s_keep, last_bin = s_last_bin;
+    cost = __reduce_add_sync(0xffffffffu, lane < kWarps ? s_cost[lane] : 0u);
+    // comparisons past a few dozen per key cost more than the caller's sort
+    if (keep > key_cap || cost > 48u * keep + 65536u) {
+      __syncthreads();  // everybody has read the verdict before the bins are cleared or the caller reuses them
+      continue;
+    }
+    // every kept key to the next free slot of its bin; bins[b] ends as the end of bin b
+    sweep([&](uint2 e) {
+      const unsigned int k = score_to_key(e.x);
+      const unsigned int b = bin_of_key(k);
+      if (b <= last_bin) keys[atomicAdd(&bins[b], 1u)] = (static_cast<uint64_t>(k) << 32) | (0xffffffffu - e.y);
+    });
+    __syncthreads();
+    for (unsigned int i = tid; i < keep; i += kThreads) {
+      const uint64_t key = keys[i];
+      const unsigned int b = bin_of_key(static_cast<unsigned int>(key >> 32));
+      unsigned int rank = b > 0u ? bins[b - 1] : 0u;
+      const unsigned int end = bins[b];
+      for (unsigned int j = rank; j < end; ++j) rank += keys[j] > key ? 1u : 0u;
+      if (rank < static_cast<unsigned int>(kk)) {
+        const bool have = LT_IN_BOUNDS(key_index(key) >= 0 && key_index(key) < n_keys, ctl);  // never publish an index outside the keys
+        out_idx[rank] = have ? key_index(key) : -1;
+        if (out_score != nullptr) out_score[rank] = have ? key_score(key) : -INFINITY;
+      }
+    }
+    for (int j = kk + tid; j < topk; j += kThreads) {
+      out_idx[j] = -1;
+      if (out_score != nullptr) out_score[j] = -INFINITY;
+    }
+    return true;
+  }
+  return false;
+}
+
+}  // namespace lt

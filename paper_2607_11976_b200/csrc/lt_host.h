@@ -155,6 +155,7 @@ struct SelectRowsParams {
   int rows_per_block;
   const unsigned char* row_flag;
   Control* ctl;
+  unsigned int sel_slots;  // set by the launch: a power of two >= topk
 };
 cudaError_t launch_select_rows(const SelectRowsParams& p, cudaStream_t stream);
 

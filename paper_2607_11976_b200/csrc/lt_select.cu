@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include "lt_common.cuh"
+#include "lt_fine_select.cuh"
 #include "lt_host.h"
 
 namespace lt {
@@ -15,6 +16,7 @@ namespace lt {
 namespace {
 
 constexpr int kSelThreads = 1024;
+constexpr int kSelDirect = 8192;  // rows up to this length are sorted without a select (one batch of registers)
 constexpr int kSelBatch = 8;  // independent row loads in flight per thread of the full-row select
 constexpr int kSelCap = 2 * LT_MAX_TOPK;  // 64-bit keys the final select can sort in shared memory
 
@@ -120,152 +122,15 @@ __global__ void __launch_bounds__(256) sample_stats_kernel(const float* __restri
 }
 
 // ---------------------------------------------------------------------------------------------
-// Stable LSD radix sort of src[0 .. n) by the high word of the keys (the score), descending, 8 bits per pass,
-// between src and a second buffer alt of n keys; n <= kRadixSortMax, called by every thread of a CTA of
-// kRadixThreads threads.  Warp w owns the contiguous slice [w, w + 1) * 32 * rounds of the input; within a warp
-// `match.any` groups the lanes of equal digit, so a key's place is (keys of smaller digits) + (keys of its digit in
-// lower warps) + (keys of its digit earlier in its own warp): the order of equal digits is kept, which is what
-// makes least-significant-digit-first passes a sort.  A pass in which every key has the same digit (the leading
-// bytes of a row's top scores mostly agree) moves nothing and is skipped.  The bitonic network this replaces costs
-// ~3.3 k instructions per thread for 2048 keys, four of these passes ~0.7 k.
-// Returns the buffer holding the result.  *sorted is false when two neighbours with equal scores ended in the
-// wrong index order: the low words took no part, the caller then has to sort the full keys.
-// ---------------------------------------------------------------------------------------------
-constexpr int kRadixThreads = 512;
-constexpr int kRadixSortMax = 4096;
-__device__ __forceinline__ uint64_t* radix_sort_by_score_desc(uint64_t* src, uint64_t* alt, int n, bool* sorted) {
-  constexpr int kWarps = kRadixThreads / 32;
-  constexpr int kMaxRounds = kRadixSortMax / kRadixThreads;
-  __shared__ unsigned int cnt[kWarps][256];
-  __shared__ unsigned int base[256];
-  __shared__ int s_skip, s_unsorted;
-  __shared__ unsigned int s_and, s_or;  // bits every score word has / some score word has (known after pass 0)
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int rounds = (n + kRadixThreads - 1) / kRadixThreads;
-  const int first = warp * 32 * rounds;
-  if (tid == 0) {
-    s_and = 0xffffffffu;
-    s_or = 0u;
-  }
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 32 + 8 * pass;
-    // a byte that is the same in every score word (usually the leading one) needs no pass at all
-    if (pass > 0 && (((s_and ^ s_or) >> (8 * pass)) & 255u) == 0u) continue;
-    for (int i = tid; i < kWarps * 256; i += kRadixThreads) (&cnt[0][0])[i] = 0u;
-    __syncthreads();
-    uint64_t key[kMaxRounds];
-    unsigned int loc[kMaxRounds];
-    unsigned int all_bits = 0xffffffffu, any_bits = 0u;
-#pragma unroll
-    for (int r = 0; r < kMaxRounds; ++r) {
-      if (r < rounds) {
-        const int i = first + r * 32 + lane;
-        const bool valid = i < n;
-        key[r] = valid ? src[i] : 0ull;
-        // digit 0 = largest byte, so that ascending places are descending scores; idle lanes get digits of their own
-        const unsigned int d = valid ? 255u - (static_cast<unsigned int>(key[r] >> shift) & 255u) : 256u + lane;
-        const unsigned int peers = __match_any_sync(0xffffffffu, d);
-        const unsigned int rank = __popc(peers & ((1u << lane) - 1u));
-        const unsigned int before = valid ? cnt[warp][d] : 0u;
-        __syncwarp();
-        if (valid && rank == 0) cnt[warp][d] = before + __popc(peers);
-        __syncwarp();
-        loc[r] = before + rank;
-        if (valid) {
-          all_bits &= static_cast<unsigned int>(key[r] >> 32);
-          any_bits |= static_cast<unsigned int>(key[r] >> 32);
-        }
-      }
-    }
-    if (pass == 0) {
-      all_bits = __reduce_and_sync(0xffffffffu, all_bits);
-      any_bits = __reduce_or_sync(0xffffffffu, any_bits);
-      if (lane == 0) {
-        atomicAnd(&s_and, all_bits);
-        atomicOr(&s_or, any_bits);
-      }
-    }
-    __syncthreads();
-    if (tid < 256) {
-      unsigned int run = 0;
-#pragma unroll
-      for (int w = 0; w < kWarps; ++w) {
-        const unsigned int c = cnt[w][tid];
-        cnt[w][tid] = run;
-        run += c;
-      }
-      base[tid] = run;  // keys with this digit
-    }
-    __syncthreads();
-    if (tid < 32) {
-      unsigned int c[8], mine = 0;
-      bool all_in_one = false;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        c[j] = base[lane * 8 + j];
-        mine += c[j];
-        all_in_one = all_in_one || c[j] == static_cast<unsigned int>(n);
-      }
-      unsigned int incl = mine;
-#pragma unroll
-      for (int dd = 1; dd < 32; dd <<= 1) {
-        const unsigned int o = __shfl_up_sync(0xffffffffu, incl, dd);
-        if (lane >= dd) incl += o;
-      }
-      unsigned int run = incl - mine;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        base[lane * 8 + j] = run;
-        run += c[j];
-      }
-      const bool skip = __any_sync(0xffffffffu, all_in_one);
-      if (lane == 0) s_skip = skip ? 1 : 0;
-    }
-    __syncthreads();
-    if (s_skip) continue;  // uniform: nothing would move
-#pragma unroll
-    for (int r = 0; r < kMaxRounds; ++r) {
-      if (r < rounds) {
-        const int i = first + r * 32 + lane;
-        if (i < n) {
-          const unsigned int d = 255u - (static_cast<unsigned int>(key[r] >> shift) & 255u);
-          alt[base[d] + cnt[warp][d] + loc[r]] = key[r];
-        }
-      }
-    }
-    __syncthreads();
-    uint64_t* t = src;
-    src = alt;
-    alt = t;
-  }
-  if (tid == 0) s_unsorted = 0;
-  __syncthreads();
-  bool bad = false;
-  for (int i = tid; i + 1 < n; i += kRadixThreads) {
-    const uint64_t a = src[i], b = src[i + 1];
-    bad = bad || ((a >> 32) == (b >> 32) && a < b);
-  }
-  if (bad) s_unsorted = 1;
-  __syncthreads();
-  *sorted = s_unsorted == 0;
-  return src;
-}
-
-// ---------------------------------------------------------------------------------------------
-// sort the first `count` keys of sel[] (shared) and write the row's outputs.  alt: an optional second buffer of
-// kRadixSortMax keys; with it (and a CTA of kRadixThreads threads) rows of 512 .. kRadixSortMax keys are sorted
-// by the radix passes above, and by the bitonic network only if equal scores were left in the wrong order.
+// Bitonic sort of the first `count` keys of sel[] (shared, room for next_pow2(count)), then the row's outputs.  For rows
+// the distribution sort gives up on.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void sort_and_write(uint64_t* sel, int count, int topk, int32_t* out_idx, float* out_score,
-                                               int n_keys, Control* ctl, uint64_t* alt = nullptr) {
-  bool sorted = false;
-  if (alt != nullptr && count >= 512 && count <= kRadixSortMax) sel = radix_sort_by_score_desc(sel, alt, count, &sorted);
-  if (!sorted) {
-    const int n = next_pow2(count < 2 ? 2 : count);
-    for (int i = count + threadIdx.x; i < n; i += blockDim.x) sel[i] = 0ull;
-    __syncthreads();
-    bitonic_sort_desc(sel, n, threadIdx.x, blockDim.x);
-  }
+                                               int n_keys, Control* ctl) {
+  const int n = next_pow2(count < 2 ? 2 : count);
+  for (int i = count + threadIdx.x; i < n; i += blockDim.x) sel[i] = 0ull;
+  __syncthreads();
+  bitonic_sort_desc(sel, n, threadIdx.x, blockDim.x);
   for (int j = threadIdx.x; j < topk; j += blockDim.x) {
     bool have = j < count;
     if (have && !LT_IN_BOUNDS(key_index(sel[j]) >= 0 && key_index(sel[j]) < n_keys, ctl)) have = false;  // never publish an index outside the keys
@@ -364,35 +229,57 @@ __device__ __forceinline__ void keep_top_keys(uint64_t* sel, int count, int keep
 }
 
 // ---------------------------------------------------------------------------------------------
-// final select over one row's candidate buffer (paper Sec. 3.2 "Top-k Selection"): the final
-// threshold bin is the highest bin whose cumulative count from the top reaches k; every candidate
-// at or above its lower edge is pulled into shared memory (the bins above hold fewer than k of
-// them), sorted by (score desc, index asc), and the first k are written out.
+// final select over one row's candidate buffer (paper Sec. 3.2 "Top-k Selection").  Every candidate buffer that did not
+// overflow holds the row's whole top-k, so the distribution sort takes all of its candidates.  The rows it gives up
+// on go the longer way: the final threshold bin is the highest bin whose cumulative count from the top reaches k;
+// every candidate at or above its lower edge is pulled into shared memory (the bins above hold fewer than k of
+// them), cut to k by a radix select, sorted, and written out.
 // ---------------------------------------------------------------------------------------------
 constexpr int kFinalThreads = 512;
-static_assert(kFinalThreads == kRadixThreads, "the radix sort is written for the final select's CTA size");
 
-__global__ void __launch_bounds__(kFinalThreads) final_select_kernel(const FinalSelectParams p, int sel_cap) {
-  extern __shared__ uint64_t sel[];  // sel_cap keys
+__global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const FinalSelectParams p, int sel_cap) {
+  extern __shared__ __align__(16) uint64_t sel[];  // sel_cap keys; the distribution sort's bins are the last of them
   __shared__ unsigned int hist[kBins];
   __shared__ int s_tb;
   __shared__ unsigned int s_count;
   const int t = blockIdx.x;
   const int lane = threadIdx.x & 31;
+  const uint2* cand = p.cand + static_cast<size_t>(t) * p.cap;
+  // The candidates are fetched without waiting for their number: most rows have between 1 and 2 topk of them.
+  uint2 first[kFineBatch];
+  const int ahead = min(p.cap, 2 * p.topk);
+#pragma unroll
+  for (int j = 0; j < kFineBatch; ++j) {
+    const int i = j * kFinalThreads + threadIdx.x;
+    if (i < ahead) first[j] = __ldcs(cand + i);
+  }
   const unsigned int tail = p.tail[t];
   const int vis = visible_keys(t, p.N, p.causal_offset);
   const int kk = p.topk < vis ? p.topk : vis;
-  bool redo = tail > static_cast<unsigned int>(p.cap);
+  bool redo = tail > static_cast<unsigned int>(p.cap) || tail < static_cast<unsigned int>(kk);
   if (threadIdx.x == 0) {
     atomicMax(&p.ctl->max_survivors, static_cast<int>(tail > 0x7fffffffu ? 0x7fffffffu : tail));
     atomicAdd(&p.ctl->tot_survivors, static_cast<int>(tail > 0x000fffffu ? 0x000fffffu : tail));
-    if (redo) atomicAdd(&p.ctl->overflow_rows, 1);
+    if (tail > static_cast<unsigned int>(p.cap)) atomicAdd(&p.ctl->overflow_rows, 1);
+  }
+  int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
+  float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
+  if (!redo && kk > 0) {
+#pragma unroll
+    for (int j = 0; j < kFineBatch; ++j) {
+      const int i = j * kFinalThreads + threadIdx.x;
+      if (i >= ahead && i < static_cast<int>(tail)) first[j] = __ldcs(cand + i);
+    }
+    constexpr int kBinSlots = kFineBins * 4 / 8;
+    if (fine_select_sort<kFinalThreads>([&](unsigned int i) { return __ldcs(cand + i); }, first, tail, kk, p.topk, sel,
+                                        static_cast<unsigned int>(sel_cap - kBinSlots),
+                                        reinterpret_cast<unsigned int*>(sel + sel_cap - kBinSlots), out_idx, out_score, p.N, p.ctl))
+      return;
   }
   if (!redo) {
     // candidates are fetched eight rounds at a time so that the loads of a batch overlap; the first batch is
     // issued before the histogram work, which does not depend on it
     constexpr int kBatch = 8;
-    const uint2* cand = p.cand + static_cast<size_t>(t) * p.cap;
     const unsigned int rounds = (tail + kFinalThreads - 1) / kFinalThreads;
     uint2 c[kBatch];
 #pragma unroll
@@ -543,34 +430,13 @@ __global__ void __launch_bounds__(kFinalThreads) final_select_kernel(const Final
     if (count > static_cast<unsigned int>(sel_cap) || count < static_cast<unsigned int>(kk)) redo = true;
     if (!redo) {
       int n_keep = static_cast<int>(count);
-      int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
-      float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
-      // the upper half of sel[] is a second buffer for the radix sort whenever the keys fit the lower one
-      uint64_t* alt = sel_cap >= 2 * kRadixSortMax ? sel + kRadixSortMax : nullptr;
-      uint64_t* keys = sel;
-      if (alt != nullptr && n_keep >= 512 && n_keep <= kRadixSortMax) {
-        // The usual row: a few hundred candidates more than outputs (the threshold bin is included whole).  Sorting
-        // all of them by score and writing the first kk is cheaper than selecting the kk-th key first.
-        bool sorted;
-        keys = radix_sort_by_score_desc(sel, alt, n_keep, &sorted);
-        if (sorted) {
-          for (int j = threadIdx.x; j < p.topk; j += kFinalThreads) {
-            bool have = j < kk;
-            if (have && !LT_IN_BOUNDS(key_index(keys[j]) >= 0 && key_index(keys[j]) < p.N, p.ctl)) have = false;
-            out_idx[j] = have ? key_index(keys[j]) : -1;
-            if (out_score != nullptr) out_score[j] = have ? key_score(keys[j]) : -INFINITY;
-          }
-          return;
-        }
-        alt = nullptr;  // equal scores in the wrong index order: the full-key path below, on wherever the keys are now
-      }
       if (n_keep > kk && kk > 0) {
         // More candidates than outputs.  The packed keys are distinct (the index is part of them), so the kk-th
         // largest key is unique: find it by a radix select in shared memory and keep exactly the keys at or above it.
-        keep_top_keys(keys, n_keep, kk, hist, &s_count);
+        keep_top_keys(sel, n_keep, kk, hist, &s_count);
         n_keep = kk;
       }
-      sort_and_write(keys, n_keep, p.topk, out_idx, out_score, p.N, p.ctl, keys == sel ? alt : nullptr);
+      sort_and_write(sel, n_keep, p.topk, out_idx, out_score, p.N, p.ctl);
       return;
     }
   }
@@ -586,11 +452,14 @@ __global__ void __launch_bounds__(kFinalThreads) final_select_kernel(const Final
 }
 
 // ---------------------------------------------------------------------------------------------
-// full-row exact select: 4-pass MSB radix select for the k-th key, ordered collection of ties
-// (lowest indices first), bitonic sort of the k winners.
+// full-row exact select.  A row of at most kSelDirect visible keys goes straight through the distribution sort; a longer
+// one (or one with mass ties) takes a 4-pass MSB radix select for the k-th key, ordered collection of ties (lowest
+// indices first), and a sort of the k winners.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRowsParams p) {
-  extern __shared__ uint64_t sel[];  // LT_MAX_TOPK keys
+  extern __shared__ __align__(16) uint64_t sel_smem[];  // the distribution sort's bins, then two buffers of p.sel_slots keys
+  unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
+  uint64_t* sel = sel_smem + kFineBins * 4 / 8;
   __shared__ unsigned int hist[256];
   __shared__ unsigned int s_prefix, s_remaining, s_gt;
   __shared__ unsigned int warp_cnt[32];
@@ -611,8 +480,24 @@ __global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRo
   float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
+  if (vis == 0) {
+    sort_and_write(sel, 0, p.topk, out_idx, out_score, p.N, p.ctl);
+    return;
+  }
+  uint2 first[kFineBatch];
+  if (vis <= kSelDirect) {
+#pragma unroll
+    for (int j = 0; j < kFineBatch; ++j) {
+      const int i = j * kSelThreads + tid;
+      if (i < vis) first[j] = make_uint2(__float_as_uint(row[i]), static_cast<unsigned int>(i));
+    }
+    if (fine_select_sort<kSelThreads>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
+                                      static_cast<unsigned int>(vis), kk, p.topk, sel, 2u * p.sel_slots, bins, out_idx, out_score,
+                                      p.N, p.ctl))
+      return;
+  }
   if (vis <= p.topk) {
-    // every visible key is selected
+    // every visible key is selected, and they did not spread over the bins
     for (int i = tid; i < vis; i += kSelThreads) sel[i] = pack_key(row[i], i);
     __syncthreads();
     sort_and_write(sel, vis, p.topk, out_idx, out_score, p.N, p.ctl);
@@ -741,6 +626,14 @@ __global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRo
    }
   }
   __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kFineBatch; ++j) {  // kFineBatch * kSelThreads == LT_MAX_TOPK: all winners are in registers
+    const int i = j * kSelThreads + tid;
+    if (i < kk) first[j] = make_uint2(key_to_score_bits(static_cast<unsigned int>(sel[i] >> 32)), static_cast<unsigned int>(key_index(sel[i])));
+  }
+  if (fine_select_sort<kSelThreads>([&](unsigned int) { return make_uint2(0u, 0u); }, first, static_cast<unsigned int>(kk), kk, p.topk,
+                                    sel + p.sel_slots, p.sel_slots, bins, out_idx, out_score, p.N, p.ctl))
+    return;
   sort_and_write(sel, kk, p.topk, out_idx, out_score, p.N, p.ctl);
 }
 
@@ -789,11 +682,13 @@ cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream)
   return cudaGetLastError();
 }
 
-cudaError_t launch_select_rows(const SelectRowsParams& p, cudaStream_t stream) {
-  const int smem = LT_MAX_TOPK * sizeof(uint64_t);
+cudaError_t launch_select_rows(const SelectRowsParams& params, cudaStream_t stream) {
+  SelectRowsParams p = params;
+  if (p.n_blocks <= 0) return cudaSuccess;
+  p.sel_slots = static_cast<unsigned int>(next_pow2(p.topk < 2048 ? 2048 : p.topk));
+  const int smem = kFineBins * 4 + 2 * static_cast<int>(p.sel_slots) * static_cast<int>(sizeof(uint64_t));
   cudaError_t e = cudaFuncSetAttribute(select_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  if (p.n_blocks <= 0) return cudaSuccess;
   select_rows_kernel<<<p.n_blocks, kSelThreads, smem, stream>>>(p);
   return cudaGetLastError();
 }
