@@ -242,14 +242,15 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid) {
   const long long want = (n_blocks <= 2 ? 1ll : 2ll) * grid;
   while (seg > 16 && static_cast<long long>(n_blocks) * ((n_tiles + seg - 1) / seg) < want) seg >>= 1;
   // Work items are dealt to the persistent CTAs round-robin, so the launch lasts as long as the CTA with the
-  // most items: among the sizes from the one above down to 16 tiles, take the shortest such critical path (in key
+  // most items: among the sizes from the one above down to one tile, take the shortest such critical path (in key
   // tiles, plus a few tiles' worth of per-item start-up: the query block of an item is as large as four key tiles).
   // Matters for short chunks: 128 rows over 8192 tiles are 512 items of 256 tiles (4 rounds on 148 CTAs, the last
-  // one half empty) or 592 items of 222 tiles.
+  // one half empty) or 592 items of 222 tiles.  Also for the sample phase, whose 64 tiles x 10 blocks (77 rows) are 40 items
+  // of 16 tiles or 130 of 5: one round either way, 29 or 15 us.
   constexpr int kItemOverheadTiles = 4;
   long long best_cost = -1;
   int best = seg;
-  for (int s = seg; s >= 16; --s) {
+  for (int s = seg; s >= 1; --s) {
     const long long items = static_cast<long long>(n_blocks) * ((n_tiles + s - 1) / s);
     const long long rounds = (items + grid - 1) / grid;
     const long long cost = rounds * ((s < n_tiles ? s : n_tiles) + kItemOverheadTiles);
