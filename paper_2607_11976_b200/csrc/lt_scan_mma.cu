@@ -43,7 +43,6 @@ constexpr int kD = 128;
 constexpr int kBlockQ = 8;                  // query rows resident per CTA
 constexpr int kUnitQ = 4;                   // query rows per UMMA (N = 4 * 64 = 256 columns)
 constexpr int kUnits = kBlockQ / kUnitQ;    // UMMAs per key tile = TMEM halves
-constexpr int kUmmaN = kUnitQ * kH;         // 256
 constexpr int kTmemCols = 512;              // two accumulators of 256 fp32 columns
 constexpr int kFirstEpiWarp = 3;
 constexpr int kEpiWarps = 16;
@@ -54,13 +53,26 @@ constexpr int kQTile = 256 * 128;           // bytes: 256 rows x 128-byte rows (
 constexpr int kStageLen = 64;               // entries of one per-warp staging list
 constexpr int kUnitWBytes = kUnitQ * kH * 4;  // bytes between the weights of query g and query 4 + g
 
-template <bool kFp8>
+// kU: units of four queries per key tile.  kUQ: queries a unit really has.  A chunk of more than four rows runs with
+// kU = 2, kUQ = 4: unit u of every tile goes to TMEM half u, warpgroup g finishes query g of it.  A chunk of at most four
+// rows (decode, verification of drafted tokens) has one unit per tile of kUQ = 1, 2 or 4 queries: its UMMAs are 64 kUQ
+// columns wide, the TMEM holds 512 / (64 kUQ) accumulators that consecutive tiles rotate through, and the four
+// warpgroups take 4 / kUQ tiles at a time (warpgroup g: query g % kUQ of the tiles whose number is g / kUQ modulo
+// 4 / kUQ).  One accumulator that is issued, drained and issued again (as it was) leaves both the tensor pipe and the
+// epilogue waiting for the other: 1 / 4 rows over 2^20 fp8 keys 59 / 64 us; now SCANKEEP us, with 21 us the time of
+// reading the keys.
+template <bool kFp8, int kU, int kUQ>
 struct Cfg {
+  static_assert((kU == 2 && kUQ == 4) || (kU == 1 && (kUQ == 1 || kUQ == 2 || kUQ == 4)), "see above");
   static constexpr int kHalves = kFp8 ? 1 : 2;           // 128-byte row pieces along D
   static constexpr int kElemsPerRow128 = kFp8 ? 128 : 64;  // elements in a 128-byte row
-  static constexpr int kStages = kFp8 ? 6 : 2;           // K-tile ring depth
+  static constexpr int kStages = kU == 2 ? (kFp8 ? 6 : 2) : (kFp8 ? 8 : 4);  // K-tile ring depth: what the query block leaves
   static constexpr int kKBlocks = kFp8 ? 4 : 8;          // UMMA K-steps per tile (K = 32 fp8 / 16 bf16 = 32 bytes)
-  static constexpr int kQBytes = kUnits * kHalves * kQTile;
+  static constexpr int kN = kUQ * kH;                    // UMMA columns of a unit
+  static constexpr int kAccs = kTmemCols / kN;           // accumulators in TMEM
+  static constexpr int kShare = kUnitQ / kUQ;            // tiles the four warpgroups work on together
+  static constexpr int kDrainers = 4 * kUQ;              // warps that read one accumulator
+  static constexpr int kQBytes = kU * kHalves * kQTile;
   static constexpr int kStageBytes = kHalves * kSwizzleTile;
   static constexpr int kSmemTiles = kQBytes + kStages * kStageBytes;
 };
@@ -77,8 +89,8 @@ struct SmemTail {
   uint64_t bar_empty[8];
   uint64_t bar_q_full;
   uint64_t bar_q_empty;
-  uint64_t bar_tmem_full[2];
-  uint64_t bar_tmem_empty[2];
+  uint64_t bar_tmem_full[8];
+  uint64_t bar_tmem_empty[8];
   uint32_t tmem_base;
   int abort_flag;     // [0] raised by a wait that ran out; every role unwinds on it
   int wait_limit_us;  // [1] bound of every wait (read by mbar_wait through the flag's address)
@@ -87,9 +99,9 @@ struct SmemTail {
   uint2 stage[kEpiWarps][kUnits][kStageLen];  // per warp and unit: (score bits, key index) of survivors
 };
 
-template <bool kFp8>
+template <bool kFp8, int kU, int kUQ>
 constexpr int smem_bytes() {
-  return 1024 + Cfg<kFp8>::kSmemTiles + static_cast<int>(sizeof(SmemTail));
+  return 1024 + Cfg<kFp8, kU, kUQ>::kSmemTiles + static_cast<int>(sizeof(SmemTail));
 }
 
 struct Item {
@@ -232,12 +244,10 @@ __device__ __forceinline__ void flush_stage(const uint2* list, int count, const 
   __syncwarp();
 }
 
-// kU: units in use.  A chunk of at most kUnitQ rows (a decode step, a tail of a few tokens) has no row for the second
-// unit: its launch issues, loads and finishes unit 0 only, which halves the tensor and the epilogue work per key tile.
-template <bool kFp8, int kMode, bool kPaged, int kU = kUnits>
+template <bool kFp8, int kMode, bool kPaged, int kU = kUnits, int kUQ = kUnitQ>
 __global__ void __launch_bounds__(kThreads, 1)
 scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScanParams p) {
-  using C = Cfg<kFp8>;
+  using C = Cfg<kFp8, kU, kUQ>;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t pad = (1024u - (raw_addr & 1023u)) & 1023u;
@@ -259,9 +269,9 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     }
     mbar_init(smem_u32(&st->bar_q_full), 1);
     mbar_init(smem_u32(&st->bar_q_empty), 1);
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < C::kAccs; ++i) {
       mbar_init(smem_u32(&st->bar_tmem_full[i]), 1);
-      mbar_init(smem_u32(&st->bar_tmem_empty[i]), kEpiWarps);
+      mbar_init(smem_u32(&st->bar_tmem_empty[i]), C::kDrainers);
     }
     st->abort_flag = 0;
     st->wait_limit_us = static_cast<int>(p.wait_limit_us);
@@ -348,10 +358,11 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   } else if (warp == 1) {
     // ------------------------------------------------------------------ UMMA issuer
     if (lane == 0) {
-      constexpr uint32_t idesc = make_idesc(kFp8, kUmmaN);
+      constexpr uint32_t idesc = make_idesc(kFp8, C::kN);
       int stage = 0;
       uint32_t phase = 0;
-      uint32_t acc_phase = 0;  // flips once per key tile: each TMEM half is filled once per tile
+      uint32_t acc_phase = 0;  // two units: flips once per key tile, each TMEM half is filled once per tile
+      uint32_t useq = 0;       // one unit: tiles issued so far
       uint32_t n_done = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
@@ -364,7 +375,9 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           ok = mbar_wait<40>(smem_u32(&st->bar_full[stage]), phase, abort_flag);
           if (!ok) break;
           for (int u = 0; u < kU; ++u) {
-            ok = mbar_wait<40>(smem_u32(&st->bar_tmem_empty[u]), acc_phase ^ 1, abort_flag);
+            const uint32_t acc = kU == 2 ? static_cast<uint32_t>(u) : useq % C::kAccs;
+            const uint32_t par = kU == 2 ? acc_phase ^ 1 : ((useq / C::kAccs) & 1) ^ 1;
+            ok = mbar_wait<40>(smem_u32(&st->bar_tmem_empty[acc]), par, abort_flag);
             if (!ok) break;
             tc_fence_after();
 #pragma unroll
@@ -373,11 +386,12 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
               const int step = kFp8 ? kb : (kb & 3);
               uint64_t a = make_smem_desc_sw128(k_base + stage * C::kStageBytes + hf * kSwizzleTile) + (step * 32 >> 4);
               uint64_t b = make_smem_desc_sw128(q_base + (u * C::kHalves + hf) * kQTile) + (step * 32 >> 4);
-              tc_mma<kFp8>(tmem_base + u * kUmmaN, a, b, idesc, kb > 0 ? 1u : 0u);
+              tc_mma<kFp8>(tmem_base + acc * C::kN, a, b, idesc, kb > 0 ? 1u : 0u);
             }
-            tc_commit(smem_u32(&st->bar_tmem_full[u]));
+            tc_commit(smem_u32(&st->bar_tmem_full[acc]));
           }
           acc_phase ^= 1;
+          ++useq;
           tc_commit(smem_u32(&st->bar_empty[stage]));
           if (++stage == C::kStages) {
             stage = 0;
@@ -395,11 +409,13 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       const int e = threadIdx.x - kFirstEpiWarp * 32;  // epilogue thread number (valid for epilogue warps)
       const int ew = warp - kFirstEpiWarp;             // epilogue warp number
       const int quarter = warp & 3;                    // TMEM lane quarter this warp may read
-      const int g = ew >> 2;                           // warpgroup 0..3: queries g (unit 0) and 4 + g (unit 1)
+      const int g = (ew >> 2) % kUQ;                   // warpgroup 0..3: queries g (unit 0) and 4 + g (unit 1)
+      const uint32_t turn = static_cast<uint32_t>((ew >> 2) / kUQ);  // one unit: which of kShare consecutive tiles it takes
       const int key_in_tile = quarter * 32 + lane;
       const uint32_t tcol = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(g * kH);
       const uint32_t w_addr = smem_u32(st->w) + g * kH * 4;
       uint32_t acc_phase = 0;
+      uint32_t useq = 0;  // one unit: tiles gone through so far
       int seq = 0;
       for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         Item it;
@@ -508,16 +524,18 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         const bool has_scale = p.k_scale != nullptr;
         bool ok = true;
         float ks_next = 1.f;
+        // with one unit per tile, the first tile of the item that is this warpgroup's turn
+        const int tile_first = kU == 2 ? it.tile_lo : it.tile_lo + static_cast<int>((turn - useq) % C::kShare);
         {
-          const int s0 = it.tile_lo * kTileKeys + key_in_tile;
-          if (has_scale && s0 < p.n_keys) ks_next = __ldg(p.k_scale + scale_index<kPaged>(p, s0));
+          const int s0 = tile_first * kTileKeys + key_in_tile;
+          if (has_scale && tile_first < it.tile_hi && s0 < p.n_keys) ks_next = __ldg(p.k_scale + scale_index<kPaged>(p, s0));
         }
-        for (int tile = it.tile_lo; tile < it.tile_hi && ok; ++tile) {
+        for (int tile = tile_first; tile < it.tile_hi && ok; tile += C::kShare) {
           const int s = tile * kTileKeys + key_in_tile;
           const float ks = ks_next;
           {
-            const int s1 = s + kTileKeys;
-            if (has_scale && tile + 1 < it.tile_hi && s1 < p.n_keys)
+            const int s1 = s + C::kShare * kTileKeys;
+            if (has_scale && tile + C::kShare < it.tile_hi && s1 < p.n_keys)
               ks_next = __ldg(p.k_scale + scale_index<kPaged>(p, s1));
           }
           // keys of this tile that some row of the block may not see (diagonal or ragged last tile)
@@ -527,19 +545,21 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             const int r = u * kUnitQ + g;
             float thr = 0.f;
             if (kMode == kModeFilter) thr = *reinterpret_cast<volatile float*>(&st->thr[r]);
-            ok = mbar_wait(smem_u32(&st->bar_tmem_full[u]), acc_phase, abort_flag);
+            const uint32_t tseq = useq + static_cast<uint32_t>(tile - it.tile_lo);
+            const uint32_t ab = kU == 2 ? static_cast<uint32_t>(u) : tseq % C::kAccs;
+            ok = mbar_wait(smem_u32(&st->bar_tmem_full[ab]), kU == 2 ? acc_phase : (tseq / C::kAccs) & 1, abort_flag);
             tc_fence_after();
             // the 64 columns of this query: both loads in flight, one wait.  The loads are issued even
             // after a failed wait (they then fetch values nobody uses): keeping them unconditional
             // keeps the 64 destination registers free of copies.
             uint32_t va[32], vb[32];
-            tmem_ld32(tcol + u * kUmmaN, va);
-            tmem_ld32(tcol + u * kUmmaN + 32, vb);
+            tmem_ld32(tcol + ab * C::kN, va);
+            tmem_ld32(tcol + ab * C::kN + 32, vb);
             tmem_ld_wait();
             // this warp's columns of half u are in registers: hand the half back to the UMMA warp
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&st->bar_tmem_empty[u]));
+            if (lane == 0) mbar_arrive(smem_u32(&st->bar_tmem_empty[ab]));
             Acc8 acc;
             if (u == 0) {
               head_sum32<kFp8, true, 0>(va, w_addr, acc);
@@ -576,6 +596,7 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           }
           acc_phase ^= 1;
         }
+        useq += static_cast<uint32_t>(it.tile_hi - it.tile_lo);
         if (kMode == kModeFilter) {
 #pragma unroll
           for (int u = 0; u < kU; ++u)
@@ -641,24 +662,28 @@ bool make_map(CUtensorMap* map, bool fp8, const void* base, uint64_t rows, uint6
   return r == CUDA_SUCCESS;
 }
 
-template <bool kFp8, int kMode, bool kPaged, int kU>
+template <bool kFp8, int kMode, bool kPaged, int kU, int kUQ>
 cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const ScanParams& p, int grid, cudaStream_t stream) {
-  constexpr int bytes = smem_bytes<kFp8>();
-  cudaError_t e = cudaFuncSetAttribute(scan_kernel<kFp8, kMode, kPaged, kU>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  constexpr int bytes = smem_bytes<kFp8, kU, kUQ>();
+  cudaError_t e = cudaFuncSetAttribute(scan_kernel<kFp8, kMode, kPaged, kU, kUQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  scan_kernel<kFp8, kMode, kPaged, kU><<<grid, kThreads, bytes, stream>>>(tq, tk, p);
+  scan_kernel<kFp8, kMode, kPaged, kU, kUQ><<<grid, kThreads, bytes, stream>>>(tq, tk, p);
   return cudaGetLastError();
 }
 // the paged variant is a separate instantiation so that the dense kernels carry none of its address arithmetic; the
-// one-unit variant exists for the fused scan of a chunk of at most kUnitQ rows
+// one-unit variants serve chunks of at most kUnitQ rows (see Cfg)
+template <bool kFp8, int kMode, bool kPaged>
+cudaError_t launch_paged(const CUtensorMap& tq, const CUtensorMap& tk, const ScanParams& p, int grid, cudaStream_t stream) {
+  const int rows = p.fb_list == nullptr ? p.row_end - p.row_begin : kBlockQ;
+  if (rows > kUnitQ) return launch_one<kFp8, kMode, kPaged, kUnits, kUnitQ>(tq, tk, p, grid, stream);
+  if (rows > 2) return launch_one<kFp8, kMode, kPaged, 1, 4>(tq, tk, p, grid, stream);
+  if (rows == 2) return launch_one<kFp8, kMode, kPaged, 1, 2>(tq, tk, p, grid, stream);
+  return launch_one<kFp8, kMode, kPaged, 1, 1>(tq, tk, p, grid, stream);
+}
 template <bool kFp8, int kMode>
 cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const ScanParams& p, int grid, cudaStream_t stream) {
-  if (kMode == kModeFilter && p.fb_list == nullptr && p.row_end - p.row_begin <= kUnitQ) {
-    return p.page_table != nullptr ? launch_one<kFp8, kModeFilter, true, 1>(tq, tk, p, grid, stream)
-                                   : launch_one<kFp8, kModeFilter, false, 1>(tq, tk, p, grid, stream);
-  }
-  return p.page_table != nullptr ? launch_one<kFp8, kMode, true, kUnits>(tq, tk, p, grid, stream)
-                                 : launch_one<kFp8, kMode, false, kUnits>(tq, tk, p, grid, stream);
+  return p.page_table != nullptr ? launch_paged<kFp8, kMode, true>(tq, tk, p, grid, stream)
+                                 : launch_paged<kFp8, kMode, false>(tq, tk, p, grid, stream);
 }
 
 }  // namespace
