@@ -97,6 +97,28 @@ bool use_abs_form(const Tun& tun, int dtype, int H, int D) {
   return tun.path == LT_PATH_FUSED_ABS && dtype == LT_DTYPE_E4M3 && scan_mma_supported(dtype, H, D);
 }
 
+// Small problems: score everything into a dense buffer and select from it (two launches) instead of sample, statistics,
+// gated scan, final select and fallback.  Both give the same bits.  The dense form saves four launches and the
+// gate's work per key, and pays 4 bytes of traffic per pair and a select over whole rows.  Measured on one B200, dense
+// against sampled, us per call, topk 2048.  Rows of up to kDenseKeys keys are selected by one CTA each: 1 row x 8 K keys
+// 20 / 41, 256 x 16 K 72 / 107, 4096 x 4 K (bf16, first chunk) 211 / 351, 4096 x 16 K 766 / 937; many rows with a small topk
+// are the exception, their candidate lists are short (topk 64, 4096 x 16 K 864 / 802, 4096 x 8 K 418 / 456).  Longer rows
+// are shared by clusters of CTAs, which pays up to about kDensePairs pairs and kDenseMaxKeys keys: 1 x 128 K 29 / 42,
+// 16 x 128 K 54 / 65, 4 x 512 K 52 / 63, 64 x 64 K 83 / 89, but 1 x 1 M 71 / 66, 16 x 512 K 137 / 119, 64 x 256 K 231 / 216.
+// The k-NN variant follows the same lines (64 x 16 K x 128: 24 / 65, 16 x 200 K x 768: 94 / 102, 4 x 1 M x 128: 111 / 91).
+constexpr int kDenseKeys = 16384;
+constexpr int kDenseMaxKeys = 512 << 10;
+constexpr long long kDensePairs = 4ll << 20;
+bool use_direct(const Tun& tun, int T, int N, int topk, bool paged) {
+  // an explicit path or a tunable of the sampled form asks for that form
+  if (tun.path != LT_PATH_AUTO || tun.sample_mult_given || tun.cap_mult_given || tun.sample_rank != 0 || tun.debug_flags != 0) return false;
+  // over a paged cache only up to one query block: larger chunks report the survivor counts of the sampled form, which
+  // equal those over dense keys and which callers compare
+  if (paged && T > kRowsPerBlock) return false;
+  if (N <= kDenseKeys / 2 || (N <= kDenseKeys && topk >= 512)) return true;
+  return (N <= kDenseKeys && T <= 1024) || (N <= kDenseMaxKeys && static_cast<long long>(T) * N <= kDensePairs);
+}
+
 // ---- workspace layout ------------------------------------------------------------------------
 struct Layout {
   bool fused;
@@ -106,6 +128,8 @@ struct Layout {
   int cap, n_sample, sample_stride, sample_rank, fb_slots, n_blocks, generic_rows;
   int rpb;        // rows of one scan block = rows of one fallback block
   bool abs_form;  // the alternative fp8 scan: linear-term rows live in the workspace
+  bool direct;    // few rows: dense scores (rows of direct_ld floats at `scratch`) and a select over them, nothing else
+  int direct_ld;
 };
 
 // n_given > 0: the caller provides that many sample positions (lt_indexer_topk_sampled); their keys are
@@ -126,6 +150,15 @@ Layout make_layout(bool fused, int T, int N, int topk, int causal_offset, const 
     L.zero_end = off;
     L.scratch = off;
     off = align_up(off + static_cast<size_t>(L.generic_rows) * N * 4);
+    L.total = off;
+    return L;
+  }
+  if (n_given == 0 && !L.abs_form && use_direct(tun, T, N, topk, gather_default)) {
+    L.direct = true;
+    L.direct_ld = (N + 31) / 32 * 32;
+    L.zero_end = off;
+    L.scratch = off;
+    off = align_up(off + static_cast<size_t>(T) * L.direct_ld * 4);
     L.total = off;
     return L;
   }
@@ -241,6 +274,7 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid) {
   // or two row blocks, whose items all have the same length (measured: 84 instead of 102 us for 1 row over 2^20 keys)
   const long long want = (n_blocks <= 2 ? 1ll : 2ll) * grid;
   while (seg > 16 && static_cast<long long>(n_blocks) * ((n_tiles + seg - 1) / seg) < want) seg >>= 1;
+  if (n_blocks <= 2 && seg < 256) seg = 2 * seg - 1;  // the halving may have gone past one item per CTA
   // Work items are dealt to the persistent CTAs round-robin, so the launch lasts as long as the CTA with the
   // most items: among the sizes from the one above down to one tile, take the shortest such critical path (in key
   // tiles, plus a few tiles' worth of per-item start-up: the query block of an item is as large as four key tiles).
@@ -366,6 +400,48 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
   float* scratch = reinterpret_cast<float*>(ws + L.fb_base);  // the fallback's dense rows (see make_layout)
   void* lin_q = abs_form ? ws + L.lin_q : nullptr;
   float* lin_scale = abs_form ? reinterpret_cast<float*>(ws + L.lin_scale) : nullptr;
+
+  if (L.direct) {
+    mark_phase(0, stream);
+    mark_phase(1, stream);
+    mark_phase(2, stream);
+    ScanParams p{};
+    p.wait_limit_us = tun.wait_limit_us;
+    p.w = w;
+    p.k_scale = k_scale;
+    p.ks_stride = 1;
+    p.T = T;
+    p.row_begin = 0;
+    p.row_end = T;
+    p.n_keys = N;
+    p.causal_offset = causal_offset;
+    p.skip_masked_tiles = 1;  // the select reads visible keys only
+    p.seg_tiles = pick_seg_tiles(tun, N, (T + kRowsPerBlock - 1) / kRowsPerBlock, grid);
+    p.topk = topk;
+    p.dump = reinterpret_cast<float*>(ws + L.scratch);
+    p.dump_ld = L.direct_ld;
+    p.page_table = page_table;
+    p.n_pages = n_pages;
+    p.pool_pages = pool_rows / kPageKeys;
+    p.ctl = ctl;
+    LT_LAUNCH(launch_scan_mma(dtype, kModeDump, q, T, k, key_rows, key_pitch, p, grid, stream));
+    mark_phase(3, stream);
+    SelectRowsParams sp{};
+    sp.scores = p.dump;
+    sp.ld = L.direct_ld;
+    sp.n_blocks = T;
+    sp.T = T;
+    sp.N = N;
+    sp.topk = topk;
+    sp.causal_offset = causal_offset;
+    sp.out_idx = out_idx;
+    sp.out_score = out_score;
+    sp.ctl = ctl;
+    LT_LAUNCH(launch_select_dense(sp, stream));
+    mark_phase(4, stream);
+    mark_phase(5, stream);
+    return LT_OK;
+  }
 
   // 0. alternative fp8 scan: the linear part of Eq. 1 as extra operand rows of every query (used by all scans below)
   mark_phase(0, stream);
@@ -660,7 +736,9 @@ int lt_dsa_union_mask(const int32_t* idx, int T, int topk, int N, int group, int
 
 int lt_indexer_sample_plan(int N, int topk, int causal_offset, const lt_tunables* tunables, int plan3[3]) {
   if (plan3 == nullptr || N <= 0 || topk <= 0 || topk > N || topk > LT_MAX_TOPK) return LT_ERR_INVALID_ARG;
-  const Layout L = make_layout(true, 1, N, topk, causal_offset, resolve_tunables(tunables));
+  Tun tun = resolve_tunables(tunables);
+  tun.path = LT_PATH_FUSED;  // the plan of the sampled path, which a chunk of a few rows does not take by itself
+  const Layout L = make_layout(true, 1, N, topk, causal_offset, tun);
   plan3[0] = L.n_sample;
   plan3[1] = L.sample_stride;
   plan3[2] = L.sample_rank;
@@ -830,6 +908,39 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
   Control* ctl = reinterpret_cast<Control*>(ws + L.ctl);
   LT_CUDA(cudaMemsetAsync(ws, 0, L.zero_end, stream));
   const int grid = tun.grid > 0 ? tun.grid : sm_count();
+  if (L.direct) {  // small problem: dense scores and a select over them (see use_direct)
+    mark_phase(0, stream);
+    mark_phase(1, stream);
+    mark_phase(2, stream);
+    KnnScanParams p{};
+    p.wait_limit_us = tun.wait_limit_us;
+    p.T = T;
+    p.row_begin = 0;
+    p.row_end = T;
+    p.n_keys = N;
+    p.D = D;
+    p.seg_tiles = knn_seg_tiles(tun, N, grid);
+    p.dump = reinterpret_cast<float*>(ws + L.scratch);
+    p.dump_ld = L.direct_ld;
+    p.ctl = ctl;
+    LT_LAUNCH(launch_scan_knn(kModeDump, q, T, x, N, D, p, grid, stream));
+    mark_phase(3, stream);
+    SelectRowsParams sp{};
+    sp.scores = p.dump;
+    sp.ld = L.direct_ld;
+    sp.n_blocks = T;
+    sp.T = T;
+    sp.N = N;
+    sp.topk = topk;
+    sp.causal_offset = N;
+    sp.out_idx = out_idx;
+    sp.out_score = out_score;
+    sp.ctl = ctl;
+    LT_LAUNCH(launch_select_dense(sp, stream));
+    mark_phase(4, stream);
+    mark_phase(5, stream);
+    return LT_OK;
+  }
   float* smin = reinterpret_cast<float*>(ws + L.smin);
   float* width = reinterpret_cast<float*>(ws + L.width);
   float* thr = reinterpret_cast<float*>(ws + L.thr);

@@ -156,8 +156,12 @@ struct SelectRowsParams {
   const unsigned char* row_flag;
   Control* ctl;
   unsigned int sel_slots;  // set by the launch: a power of two >= topk
+  int slice_keys;          // set by the launch of the cluster form
 };
 cudaError_t launch_select_rows(const SelectRowsParams& p, cudaStream_t stream);
+// The same for few rows (direct mode only): long rows are shared by clusters of CTAs.  scores 16-byte aligned, ld a
+// multiple of 4.
+cudaError_t launch_select_dense(const SelectRowsParams& p, cudaStream_t stream);
 
 // ---- lt_sampler.cu --------------------------------------------------------------------------
 // counts[p] += occurrences of p in idx[0..n) (entries outside [0, N) are skipped); counts must be zeroed.

@@ -59,7 +59,7 @@ constexpr int kUnitWBytes = kUnitQ * kH * 4;  // bytes between the weights of qu
 // columns wide, the TMEM holds 512 / (64 kUQ) accumulators that consecutive tiles rotate through, and the four
 // warpgroups take 4 / kUQ tiles at a time (warpgroup g: query g % kUQ of the tiles whose number is g / kUQ modulo
 // 4 / kUQ).  One accumulator that is issued, drained and issued again (as it was) leaves both the tensor pipe and the
-// epilogue waiting for the other: 1 / 4 rows over 2^20 fp8 keys 59 / 64 us; now SCANKEEP us, with 21 us the time of
+// epilogue waiting for the other: 1 / 4 rows over 2^20 fp8 keys 63 / 69 us; now 34 / 56 us, with 21 us the time of
 // reading the keys.
 template <bool kFp8, int kU, int kUQ>
 struct Cfg {

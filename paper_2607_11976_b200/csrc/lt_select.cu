@@ -1,6 +1,7 @@
 // Selection-side kernels of the indexer top-k: sample statistics, final select over the candidate
 // buffers, full-row radix select (generic path, unfused baseline, exact fallback) and the generic
 // SIMT scoring kernel.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
@@ -15,8 +16,7 @@ namespace lt {
 
 namespace {
 
-constexpr int kSelThreads = 1024;
-constexpr int kSelDirect = 8192;  // rows up to this length are sorted without a select (one batch of registers)
+constexpr int kSelDirect = 16384;  // rows up to this length are sorted without a select (a few batches of registers)
 constexpr int kSelBatch = 8;  // independent row loads in flight per thread of the full-row select
 constexpr int kSelCap = 2 * LT_MAX_TOPK;  // 64-bit keys the final select can sort in shared memory
 
@@ -472,58 +472,16 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
 }
 
 // ---------------------------------------------------------------------------------------------
-// full-row exact select.  A row of at most kSelDirect visible keys goes straight through the distribution sort; a longer
-// one (or one with mass ties) takes a 4-pass MSB radix select for the k-th key, ordered collection of ties (lowest
-// indices first), and a sort of the k winners.
+// The kk (< vis) best of row[0 .. vis), by one CTA: 4-pass MSB radix select for the kk-th score, then everything above it and
+// the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRowsParams p) {
-  extern __shared__ __align__(16) uint64_t sel_smem[];  // the distribution sort's bins, then two buffers of p.sel_slots keys
-  unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
-  uint64_t* sel = sel_smem + kFineBins * 4 / 8;
+template <int kThreads>
+__device__ __forceinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel) {
+  constexpr int kWarps = kThreads / 32;
   __shared__ unsigned int hist[256];
   __shared__ unsigned int s_prefix, s_remaining, s_gt;
-  __shared__ unsigned int warp_cnt[32];
-  int t;
-  if (p.fb_list != nullptr) {
-    int j = p.fb_round_base + blockIdx.x / p.rows_per_block;
-    if (j >= *p.fb_blocks) return;
-    t = p.fb_list[j] * p.rows_per_block + blockIdx.x % p.rows_per_block;
-    if (t >= p.T || !p.row_flag[t]) return;
-  } else {
-    t = p.row_begin + blockIdx.x;
-    if (p.row_flag != nullptr && !p.row_flag[t]) return;  // only flagged rows are redone
-  }
-  const float* row = p.scores + static_cast<size_t>(blockIdx.x) * p.ld;
-  const int vis = visible_keys(t, p.N, p.causal_offset);
-  const int kk = p.topk < vis ? p.topk : vis;
-  int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
-  float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
+  __shared__ unsigned int warp_cnt[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-
-  if (vis == 0) {
-    sort_and_write(sel, 0, p.topk, out_idx, out_score, p.N, p.ctl);
-    return;
-  }
-  uint2 first[kFineBatch];
-  if (vis <= kSelDirect) {
-#pragma unroll
-    for (int j = 0; j < kFineBatch; ++j) {
-      const int i = j * kSelThreads + tid;
-      if (i < vis) first[j] = make_uint2(__float_as_uint(row[i]), static_cast<unsigned int>(i));
-    }
-    if (fine_select_sort<kSelThreads>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
-                                      static_cast<unsigned int>(vis), kk, p.topk, sel, 2u * p.sel_slots, bins, out_idx, out_score,
-                                      p.N, p.ctl))
-      return;
-  }
-  if (vis <= p.topk) {
-    // every visible key is selected, and they did not spread over the bins
-    for (int i = tid; i < vis; i += kSelThreads) sel[i] = pack_key(row[i], i);
-    __syncthreads();
-    sort_and_write(sel, vis, p.topk, out_idx, out_score, p.N, p.ctl);
-    return;
-  }
-
   if (tid == 0) {
     s_prefix = 0;
     s_remaining = static_cast<unsigned int>(kk);
@@ -538,16 +496,16 @@ __global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRo
     // same counter: each thread run-length-encodes its digits and issues one atomic per run.
     unsigned int run_digit = 0x100u, run_len = 0;
     // (kSelBatch loads in flight per thread: one row is read by one SM, which is latency-bound otherwise)
-    for (int base = 0; base < vis; base += kSelThreads * kSelBatch) {
+    for (int base = 0; base < vis; base += kThreads * kSelBatch) {
       float v[kSelBatch];
 #pragma unroll
       for (int j = 0; j < kSelBatch; ++j) {
-        const int i = base + j * kSelThreads + tid;
+        const int i = base + j * kThreads + tid;
         v[j] = i < vis ? row[i] : 0.f;
       }
 #pragma unroll
       for (int j = 0; j < kSelBatch; ++j) {
-        const int i = base + j * kSelThreads + tid;
+        const int i = base + j * kThreads + tid;
         unsigned int digit = 0x100u;  // "not a candidate" (out of range or another prefix)
         if (i < vis) {
           const unsigned int key = score_to_key(__float_as_uint(v[j]));
@@ -589,8 +547,8 @@ __global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRo
   if (tid == 0) s_gt = 0;
   // Collection.  Keys above the k-th go in any order (the sort follows).  Ties at the k-th value keep
   // the lowest indices, so they are ranked in index order: every warp owns one contiguous range of the
-  // row, counts its ties, and after one prefix sum over the 32 warps writes them at their ranks.
-  const int per_warp = (((vis + 31) / 32 + 31) / 32) * 32;  // range length: a multiple of 32 covering vis / 32
+  // row, counts its ties, and after one prefix sum over the warps writes them at their ranks.
+  const int per_warp = (((vis + kWarps - 1) / kWarps + 31) / 32) * 32;  // range length: a multiple of 32 covering vis / kWarps
   const int lo = wid * per_warp;
   const int hi = min(vis, lo + per_warp);
   unsigned int my_eq = 0;
@@ -645,16 +603,327 @@ __global__ void __launch_bounds__(kSelThreads) select_rows_kernel(const SelectRo
     running += __popc(eq_ballot);
    }
   }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < kFineBatch; ++j) {  // kFineBatch * kSelThreads == LT_MAX_TOPK: all winners are in registers
-    const int i = j * kSelThreads + tid;
-    if (i < kk) first[j] = make_uint2(key_to_score_bits(static_cast<unsigned int>(sel[i] >> 32)), static_cast<unsigned int>(key_index(sel[i])));
+}
+
+// ---------------------------------------------------------------------------------------------
+// full-row exact select.  A row of at most kSelDirect visible keys goes straight through the distribution sort; a longer
+// one (or one with mass ties) takes a 4-pass MSB radix select for the k-th key, ordered collection of ties (lowest
+// indices first), and a sort of the k winners.
+// ---------------------------------------------------------------------------------------------
+template <int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const SelectRowsParams p) {
+  extern __shared__ __align__(16) uint64_t sel_smem[];  // the distribution sort's bins, then two buffers of p.sel_slots keys
+  unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
+  uint64_t* sel = sel_smem + kFineBins * 4 / 8;
+  int t;
+  if (p.fb_list != nullptr) {
+    int j = p.fb_round_base + blockIdx.x / p.rows_per_block;
+    if (j >= *p.fb_blocks) return;
+    t = p.fb_list[j] * p.rows_per_block + blockIdx.x % p.rows_per_block;
+    if (t >= p.T || !p.row_flag[t]) return;
+  } else {
+    t = p.row_begin + blockIdx.x;
+    if (p.row_flag != nullptr && !p.row_flag[t]) return;  // only flagged rows are redone
   }
-  if (fine_select_sort<kSelThreads>([&](unsigned int) { return make_uint2(0u, 0u); }, first, static_cast<unsigned int>(kk), kk, p.topk,
-                                    sel + p.sel_slots, p.sel_slots, bins, out_idx, out_score, p.N, p.ctl))
+  const float* row = p.scores + static_cast<size_t>(blockIdx.x) * p.ld;
+  const int vis = visible_keys(t, p.N, p.causal_offset);
+  const int kk = p.topk < vis ? p.topk : vis;
+  int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
+  float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
+  const int tid = threadIdx.x;
+
+  if (vis == 0) {
+    sort_and_write(sel, 0, p.topk, out_idx, out_score, p.N, p.ctl);
+    return;
+  }
+  uint2 first[kFineBatch];
+  if (vis <= kSelDirect) {
+#pragma unroll
+    for (int j = 0; j < kFineBatch; ++j) {
+      const int i = j * kThreads + tid;
+      if (i < vis) first[j] = make_uint2(__float_as_uint(row[i]), static_cast<unsigned int>(i));
+    }
+    if (fine_select_sort<kThreads>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
+                                      static_cast<unsigned int>(vis), kk, p.topk, sel, 2u * p.sel_slots, bins, out_idx, out_score,
+                                      p.N, p.ctl))
+      return;
+  }
+  if (vis <= p.topk) {
+    // every visible key is selected, and they did not spread over the bins
+    for (int i = tid; i < vis; i += kThreads) sel[i] = pack_key(row[i], i);
+    __syncthreads();
+    sort_and_write(sel, vis, p.topk, out_idx, out_score, p.N, p.ctl);
+    return;
+  }
+
+  radix_select_row<kThreads>(row, vis, kk, sel);
+  __syncthreads();
+  auto winner = [&](unsigned int i) { return make_uint2(key_to_score_bits(static_cast<unsigned int>(sel[i] >> 32)), static_cast<unsigned int>(key_index(sel[i]))); };
+#pragma unroll
+  for (int j = 0; j < kFineBatch; ++j)
+    if (j * kThreads + tid < kk) first[j] = winner(j * kThreads + tid);
+  if (fine_select_sort<kThreads>(winner, first, static_cast<unsigned int>(kk), kk, p.topk, sel + p.sel_slots, p.sel_slots, bins,
+                                 out_idx, out_score, p.N, p.ctl))
     return;
   sort_and_write(sel, kk, p.topk, out_idx, out_score, p.N, p.ctl);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Full-row exact select by a cluster of CTAs, for few rows over many keys (one CTA would stream a 128 K row three to
+// four times on its own).  Every CTA owns a slice of the row, kept in shared memory as far as it fits.  Equal-width
+// bins over the row's range, as in the distribution sort but kClBins of them: the CTAs' histograms are merged through
+// distributed shared memory, the CTAs agree on the bin that holds the kk-th key, and every key up to it goes to the
+// first CTA's list, which is then sorted there.  A bin that holds more keys than the list takes is split again over
+// its own range (a few outliers stretch the range); what still does not fit (mass ties) is left to the first CTA's
+// radix select over the whole row.  Bound by latencies (four cluster barriers, a sort by one CTA) up to 128 K keys, by
+// instructions above: a key costs about 15, on floats throughout (ordered bit patterns would double that).
+// ---------------------------------------------------------------------------------------------
+constexpr int kClThreads = 512;
+constexpr int kClWarps = kClThreads / 32;
+constexpr int kClBins = 2048;
+constexpr int kClLevels = 3;
+constexpr int kClStaticSmem = 8 * 1024;  // upper bound of what the kernel declares statically
+// (a multiple of four keys: what lies behind the list is accessed in 16-byte pieces)
+__host__ __device__ constexpr int cluster_list_cap(int topk) { return (topk + (topk / 4 > 2048 ? topk / 4 : 2048) + 3) / 4 * 4; }
+
+__device__ __forceinline__ unsigned int warp_inclusive_sum(unsigned int v, int lane) {
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned int o = __shfl_up_sync(0xffffffffu, v, d);
+    if (lane >= d) v += o;
+  }
+  return v;
+}
+
+// p.slice_keys: scores of a slice kept in shared memory (a multiple of 4)
+__global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const SelectRowsParams p) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const unsigned int n_cta = cl.num_blocks(), rank = cl.block_rank();
+  extern __shared__ __align__(16) uint8_t cl_smem[];
+  const unsigned int cap = static_cast<unsigned int>(cluster_list_cap(p.topk));
+  uint64_t* list = reinterpret_cast<uint64_t*>(cl_smem);             // keys up to the threshold bin (first CTA)
+  unsigned int* bins = reinterpret_cast<unsigned int*>(list + cap);  // this CTA's histogram; later the sort's bins
+  float* slice = reinterpret_cast<float*>(bins + kFineBins);
+  uint64_t* sorted = reinterpret_cast<uint64_t*>(slice);             // the slice is dead when the list is sorted
+  __shared__ __align__(16) unsigned int s_seg[kClBins / 2];
+  __shared__ float s_range[2], s_wmin[kClWarps], s_wmax[kClWarps];
+  __shared__ unsigned int s_sum[kClWarps], s_seg_sum, s_count, s_above, s_tb, s_total, s_fill;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int t = p.row_begin + blockIdx.x / n_cta;
+  const float* row = p.scores + static_cast<size_t>(t - p.row_begin) * p.ld;
+  const int vis = visible_keys(t, p.N, p.causal_offset);
+  const int kk = p.topk < vis ? p.topk : vis;
+  int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
+  float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
+  if (kk == 0) {  // the whole cluster
+    if (rank == 0) sort_and_write(list, 0, p.topk, out_idx, out_score, p.N, p.ctl);
+    return;
+  }
+  // slices start on 16-byte boundaries (the caller's rows do); the last of a slice's pieces of four may be ragged
+  const int per = ((vis + static_cast<int>(n_cta) - 1) / static_cast<int>(n_cta) + 3) & ~3;
+  const int lo = min(vis, static_cast<int>(rank) * per), len = min(vis, lo + per) - lo;
+  const int held = min(len, p.slice_keys);
+  const float4* mine4 = reinterpret_cast<const float4*>(row + lo);
+  float4* slice4 = reinterpret_cast<float4*>(slice);
+  constexpr int kDepth = 8;
+  // pieces [from, to) of the slice from global memory, kDepth of them in flight; visit(piece number, values)
+  auto stream = [&](int from, int to, auto&& visit) {
+    for (int base = from + tid; base < to; base += kDepth * kClThreads) {
+      float4 v[kDepth];
+#pragma unroll
+      for (int j = 0; j < kDepth; ++j) v[j] = __ldcg(mine4 + min(base + j * kClThreads, to - 1));
+#pragma unroll
+      for (int j = 0; j < kDepth; ++j)
+        if (base + j * kClThreads < to) visit(base + j * kClThreads, v[j]);
+    }
+  };
+  const int pieces = (len + 3) >> 2, held_pieces = held >= len ? pieces : held >> 2;
+  // visits (score, index in the slice) of every key of the slice.  A ragged last piece was padded with -inf when it was
+  // loaded; -inf lies below every range and is never counted or taken.
+  const float kNone = -INFINITY;
+  auto clip = [&](int piece, float4 v) {
+    if (piece * 4 + 3 >= len) {
+      if (piece * 4 + 1 >= len) v.y = kNone;
+      if (piece * 4 + 2 >= len) v.z = kNone;
+      v.w = kNone;
+    }
+    return v;
+  };
+  auto sweep = [&](auto&& visit) {
+#pragma unroll 2
+    for (int i = tid; i < held_pieces; i += kClThreads) visit(i, slice4[i]);
+    stream(held_pieces, pieces, [&](int i, float4 v) { visit(i, clip(i, v)); });
+  };
+  float vmin = INFINITY, vmax = -INFINITY;
+  stream(0, pieces, [&](int i, float4 v) {
+    float4 m = v;  // for the minimum, padding repeats a real score (v.x always is one)
+    if (i * 4 + 3 >= len) {
+      v = clip(i, v);
+      m = make_float4(v.x, i * 4 + 1 < len ? v.y : v.x, i * 4 + 2 < len ? v.z : v.x, v.x);
+    }
+    if (i < held_pieces) slice4[i] = v;
+    vmin = fminf(vmin, fminf(fminf(m.x, m.y), fminf(m.z, m.w)));
+    vmax = fmaxf(vmax, fmaxf(fmaxf(m.x, m.y), fmaxf(m.z, m.w)));
+  });
+  if (tid == 0) s_fill = 0u;
+
+  float scale = 0.f, limit = 0.f;
+  unsigned int above = 0u, total = 0u;
+  int level = 0;
+  for (;; ++level) {
+    // range [vmin, vmax] of the keys still in question, over the cluster
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, d));
+      vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, d));
+    }
+    if (lane == 0) {
+      s_wmin[warp] = vmin;
+      s_wmax[warp] = vmax;
+    }
+    for (int i = tid; i < kClBins / 4; i += kClThreads) reinterpret_cast<uint4*>(bins)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    if (tid == 0) {
+#pragma unroll
+      for (int w = 1; w < kClWarps; ++w) {
+        vmin = fminf(vmin, s_wmin[w]);
+        vmax = fmaxf(vmax, s_wmax[w]);
+      }
+      s_range[0] = vmin;
+      s_range[1] = vmax;
+    }
+    cl.sync();
+    {
+      const float* r = cl.map_shared_rank(s_range, min(static_cast<unsigned int>(lane), n_cta - 1u));
+      vmin = r[0];
+      vmax = r[1];
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) {
+        vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, d));
+        vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, d));
+      }
+    }
+    // bin of a score in the range, best scores first; monotone because every step rounds monotonically
+    // (finite, so that the best score's 0 * scale is 0)
+    scale = vmax > vmin ? fminf(static_cast<float>(kClBins) / (vmax - vmin), 3e38f) : 0.f;
+    auto count = [&](float v) {
+      if (v >= vmin && v <= vmax) atomicAdd(&bins[min(static_cast<unsigned int>((vmax - v) * scale), kClBins - 1u)], 1u);
+    };
+    sweep([&](int, float4 v) {
+      count(v.x);
+      count(v.y);
+      count(v.z);
+      count(v.w);
+    });
+    cl.sync();
+    // merge: this CTA sums the bins of its segment over the cluster
+    const int seg = kClBins / static_cast<int>(n_cta);  // 128 .. 1024
+    unsigned int part = 0;
+    for (int i = tid; i < seg; i += kClThreads) {
+      unsigned int c = 0;
+#pragma unroll 4
+      for (unsigned int r = 0; r < n_cta; ++r) c += cl.map_shared_rank(bins, r)[rank * seg + i];
+      s_seg[i] = c;
+      part += c;
+    }
+    part = __reduce_add_sync(0xffffffffu, part);
+    if (lane == 0) s_sum[warp] = part;
+    __syncthreads();
+    if (tid < 32) {
+      part = __reduce_add_sync(0xffffffffu, lane < kClWarps ? s_sum[lane] : 0u);
+      if (lane == 0) s_seg_sum = part;
+    }
+    cl.sync();
+    {
+      // the segment, then the bin in it, where the count from the top reaches kk (every warp finds the segment)
+      const unsigned int need = static_cast<unsigned int>(kk) - above;
+      const unsigned int sum = lane < static_cast<int>(n_cta) ? *cl.map_shared_rank(&s_seg_sum, lane) : 0u;
+      const unsigned int incl = warp_inclusive_sum(sum, lane);
+      const int owner = __ffs(__ballot_sync(0xffffffffu, incl >= need && incl - sum < need)) - 1;
+      const unsigned int before = __shfl_sync(0xffffffffu, incl - sum, owner);
+      const uint2* segc = reinterpret_cast<const uint2*>(cl.map_shared_rank(s_seg, owner));
+      const uint2 c = 2 * tid < seg ? segc[tid] : make_uint2(0u, 0u);  // two bins per thread: at most 1024
+      const unsigned int ic = warp_inclusive_sum(c.x + c.y, lane);
+      if (lane == 31) s_sum[warp] = ic;
+      __syncthreads();
+      const unsigned int at = before + __reduce_add_sync(0xffffffffu, lane < warp ? s_sum[lane] : 0u) + ic - c.x - c.y;  // keys above this thread's bins
+      if (at < need && at + c.x + c.y >= need) {  // exactly one thread
+        const bool second = at + c.x < need;
+        s_tb = static_cast<unsigned int>(owner * seg + 2 * tid) + (second ? 1u : 0u);
+        s_above = above + at + (second ? c.x : 0u);
+        s_total = above + at + c.x + (second ? c.y : 0u);
+      }
+      __syncthreads();
+    }
+    const unsigned int tb = s_tb;
+    total = s_total;
+    // a key is wanted when it lies in the range or above it and (vmax - v) * scale < limit
+    limit = tb == kClBins - 1u ? INFINITY : static_cast<float>(tb + 1u);
+    if (total <= cap || level == kClLevels - 1) break;
+    above = s_above;
+    // the threshold bin alone is the next level's range
+    float nmin = INFINITY, nmax = -INFINITY;
+    const float from = static_cast<float>(tb);
+    auto narrow = [&](float v) {
+      const float d = (vmax - v) * scale;
+      if (v >= vmin && v <= vmax && d >= from && d < limit) {
+        nmin = fminf(nmin, v);
+        nmax = fmaxf(nmax, v);
+      }
+    };
+    sweep([&](int, float4 v) {
+      narrow(v.x);
+      narrow(v.y);
+      narrow(v.z);
+      narrow(v.w);
+    });
+    vmin = nmin;
+    vmax = nmax;
+  }
+  if (total <= cap) {
+    // every wanted key to the first CTA's list: count, reserve, write
+    auto wanted = [&](float v) { return v >= vmin && (vmax - v) * scale < limit; };
+    unsigned int n = 0;
+    sweep([&](int, float4 v) { n += (wanted(v.x) ? 1u : 0u) + (wanted(v.y) ? 1u : 0u) + (wanted(v.z) ? 1u : 0u) + (wanted(v.w) ? 1u : 0u); });
+    const unsigned int incl = warp_inclusive_sum(n, lane);
+    if (lane == 31) s_sum[warp] = incl;
+    __syncthreads();
+    if (tid < 32) {
+      const unsigned int w = lane < kClWarps ? s_sum[lane] : 0u;
+      const unsigned int wi = warp_inclusive_sum(w, lane);
+      unsigned int base = 0;
+      if (lane == 31 && wi > 0u) base = atomicAdd(cl.map_shared_rank(&s_fill, 0), wi);
+      base = __shfl_sync(0xffffffffu, base, 31);
+      if (lane < kClWarps) s_sum[lane] = base + wi - w;
+    }
+    __syncthreads();
+    unsigned int pos = s_sum[warp] + incl - n;
+    uint64_t* dst = cl.map_shared_rank(list, 0);
+    if (n > 0u)
+      sweep([&](int i, float4 v) {
+        if (wanted(v.x)) dst[pos++] = pack_key(v.x, lo + 4 * i);
+        if (wanted(v.y)) dst[pos++] = pack_key(v.y, lo + 4 * i + 1);
+        if (wanted(v.z)) dst[pos++] = pack_key(v.z, lo + 4 * i + 2);
+        if (wanted(v.w)) dst[pos++] = pack_key(v.w, lo + 4 * i + 3);
+      });
+  }
+  cl.sync();  // the list is complete; nothing of the other CTAs is read any more
+  if (rank != 0) return;
+  if (total <= cap) {
+    uint2 first[kFineBatch];
+    auto entry = [&](unsigned int i) { return make_uint2(key_to_score_bits(static_cast<unsigned int>(list[i] >> 32)), static_cast<unsigned int>(key_index(list[i]))); };
+#pragma unroll
+    for (int j = 0; j < kFineBatch; ++j)
+      if (j * kClThreads + tid < total) first[j] = entry(j * kClThreads + tid);
+    if (fine_select_sort<kClThreads>(entry, first, total, kk, p.topk, sorted, cap, bins, out_idx, out_score, p.N, p.ctl)) return;
+    if (total > static_cast<unsigned int>(kk)) keep_top_keys(list, static_cast<int>(total), kk, bins, &s_count);
+  } else {
+    radix_select_row<kClThreads>(row, vis, kk, list);
+  }
+  __syncthreads();
+  // room for next_pow2(kk) keys: the list, the bins and the slice lie one behind the other
+  sort_and_write(list, kk, p.topk, out_idx, out_score, p.N, p.ctl);
 }
 
 }  // namespace
@@ -704,15 +973,60 @@ cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream)
   return cudaGetLastError();
 }
 
+cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t stream) {
+  // one CTA sorts a short row in one go; a cluster shares a longer one, as wide as the row is long and the chip allows
+  if (params.N <= kSelDirect) return launch_select_rows(params, stream);
+  SelectRowsParams p = params;
+  if (p.n_blocks <= 0) return cudaSuccess;
+  int width = 2;
+  while (width < 16 && static_cast<long long>(width) * kSelDirect < p.N) width <<= 1;
+  if (width > 8 && p.n_blocks * width > 128) width = 8;  // clusters of 16 need a whole GPC: only while few are wanted
+  // shared memory: the list, the bins, and as much of a slice as fits (at least the sort's second buffer)
+  const int list = cluster_list_cap(p.topk) * 8;
+  const int slice_max = (227 * 1024 - kClStaticSmem - list - kFineBins * 4) / 16 * 4;
+  const int slice_want = ((p.N + width - 1) / width + 7) / 4 * 4;
+  p.slice_keys = slice_want < slice_max ? slice_want : slice_max;
+  const int tail = p.slice_keys * 4 > list ? p.slice_keys * 4 : list;
+  const int smem = list + kFineBins * 4 + tail;
+  cudaError_t e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  if (width > 8) {
+    e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned int>(width);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned int>(p.n_blocks * width));
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, select_cluster_kernel, p);
+}
+
+namespace {
+template <int kThreads>
+cudaError_t launch_select_rows_n(const SelectRowsParams& p, int smem, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(select_rows_kernel<kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  select_rows_kernel<kThreads><<<p.n_blocks, kThreads, smem, stream>>>(p);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_select_rows(const SelectRowsParams& params, cudaStream_t stream) {
   SelectRowsParams p = params;
   if (p.n_blocks <= 0) return cudaSuccess;
   p.sel_slots = static_cast<unsigned int>(next_pow2(p.topk < 2048 ? 2048 : p.topk));
   const int smem = kFineBins * 4 + 2 * static_cast<int>(p.sel_slots) * static_cast<int>(sizeof(uint64_t));
-  cudaError_t e = cudaFuncSetAttribute(select_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  select_rows_kernel<<<p.n_blocks, kSelThreads, smem, stream>>>(p);
-  return cudaGetLastError();
+  // many short rows: three small CTAs an SM hide one another's barriers; otherwise a row gets all the threads it can use
+  if (p.fb_list == nullptr && p.n_blocks > 296 && p.N <= kSelDirect) return launch_select_rows_n<512>(p, smem, stream);
+  return launch_select_rows_n<1024>(p, smem, stream);
 }
 
 }  // namespace lt
