@@ -21,7 +21,12 @@ constexpr int kSelBatch = 8;  // independent row loads in flight per thread of t
 constexpr int kSelCap = 2 * LT_MAX_TOPK;  // 64-bit keys the final select can sort in shared memory
 
 // ---------------------------------------------------------------------------------------------
-// generic SIMT scoring: one CTA = one query row x 128 keys; thread = one key.
+// generic SIMT scoring (any H, D, dtype).  Bound by fp32 FMA issue once there is enough of it: a thread keeps 4 keys x 8
+// heads of dots in registers (three 16-byte shared loads per 32 FMAs), a warp covers 128 keys of one query row, the eight
+// warps of a CTA share the key tile (kRows query rows x 8 / kRows runs of 128 keys).  With a thread per key that fetched
+// both operands of every FMA, 64 x 4096 x 8 heads x 64 took 49 us and
+// 128 x 16384 x 32 x 128 2659 us; now 14 and 457 us (half of the fp32 FMA peak).  Dots run over d and the head sum over h in
+// ascending order, one FMA each: every launch shape gives the same bits.
 // ---------------------------------------------------------------------------------------------
 template <int kDtype>
 __device__ __forceinline__ float load_elem(const void* base, size_t i) {
@@ -31,37 +36,101 @@ __device__ __forceinline__ float load_elem(const void* base, size_t i) {
   return __half2float(__half(hr));
 }
 
-template <int kDtype>
-__global__ void __launch_bounds__(128) simt_scores_kernel(const void* __restrict__ q, const float* __restrict__ w,
-                                                          const void* __restrict__ k, const float* __restrict__ k_scale, int N,
-                                                          int H, int D, int causal_offset, int row_begin, float* __restrict__ out,
-                                                          long long ld) {
-  extern __shared__ float sm[];
-  float* qs = sm;                 // [H][D]
-  float* ks = sm + H * D;         // [128][D + 1]
-  const int t = row_begin + blockIdx.y;
-  const int s0 = blockIdx.x * 128;
-  for (int i = threadIdx.x; i < H * D; i += 128) qs[i] = load_elem<kDtype>(q, static_cast<size_t>(t) * H * D + i);
-  for (int i = threadIdx.x; i < 128 * D; i += 128) {
-    int r = i / D, d = i - r * D;
-    int s = s0 + r;
-    ks[r * (D + 1) + d] = (s < N) ? load_elem<kDtype>(k, static_cast<size_t>(s) * D + d) : 0.f;
+constexpr int kSimtThreads = 256;
+constexpr int kSimtD = 16;           // coordinates staged at a time
+constexpr int kSimtHeads = 8;        // heads in registers
+constexpr int kSimtKeyPad = 4;       // (keeps 16-byte alignment, spreads the transposing stores over the banks)
+
+template <int kDtype, int kRows>
+__global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void* __restrict__ q, const float* __restrict__ w,
+                                                                   const void* __restrict__ k, const float* __restrict__ k_scale, int N,
+                                                                   int H, int D, int causal_offset, int row_begin, int row_end,
+                                                                   float* __restrict__ out, long long ld) {
+  constexpr int kKeys = 128 * (8 / kRows);  // keys of the CTA's tile
+  __shared__ __align__(16) float ks[kSimtD][kKeys + kSimtKeyPad];
+  __shared__ __align__(16) float qs[kRows][kSimtD][kSimtHeads];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int t0 = row_begin + blockIdx.y * kRows, s0 = blockIdx.x * kKeys;
+  const int tr = warp % kRows, t = t0 + tr;
+  const int key = (warp / kRows) * 128 + lane * 4;  // first of the thread's four keys in the tile
+  // the next piece of both operands travels in registers while the current one is worked on
+  constexpr int kK = kKeys * kSimtD / kSimtThreads, kQ = kRows * kSimtHeads * kSimtD / kSimtThreads;
+  static_assert(kK * kSimtThreads == kKeys * kSimtD && kQ * kSimtThreads == kRows * kSimtHeads * kSimtD, "whole loads per thread");
+  float kr[kK], qr[kQ];
+  // thread -> (coordinate d, key sj + 16 j) and (coordinate d, head hj, row rj + 2 j)
+  static_assert(kSimtThreads == 256 && kSimtD == 16 && kSimtHeads == 8, "the index arithmetic below");
+  const int dj = tid & 15, sj = tid >> 4, hj = (tid >> 4) & 7, rj = tid >> 7;
+  const size_t k_at = static_cast<size_t>(s0 + sj) * D + dj, q_at = (static_cast<size_t>(t0 + rj) * H + hj) * D + dj;
+  const int live = min(kK, (N - s0 - sj + 15) / 16);  // keys of this thread that exist (may be negative)
+  auto fetch = [&](int h0, int d0) {
+    const bool in = d0 + dj < D;
+#pragma unroll
+    for (int j = 0; j < kK; ++j) kr[j] = in && j < live ? load_elem<kDtype>(k, k_at + d0 + static_cast<size_t>(j) * 16 * D) : 0.f;
+#pragma unroll
+    for (int j = 0; j < kQ; ++j)
+      qr[j] = in && h0 + hj < H && t0 + rj + 2 * j < row_end
+                  ? load_elem<kDtype>(q, q_at + static_cast<size_t>(h0) * D + d0 + static_cast<size_t>(j) * 2 * H * D) : 0.f;
+  };
+  fetch(0, 0);
+  float total[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int h0 = 0; h0 < H; h0 += kSimtHeads) {
+    float acc[kSimtHeads][4];
+#pragma unroll
+    for (int h = 0; h < kSimtHeads; ++h)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) acc[h][j] = 0.f;
+    for (int d0 = 0; d0 < D; d0 += kSimtD) {
+      __syncthreads();
+#pragma unroll
+      for (int j = 0; j < kK; ++j) ks[dj][sj + 16 * j] = kr[j];
+#pragma unroll
+      for (int j = 0; j < kQ; ++j) qs[rj + 2 * j][dj][hj] = qr[j];
+      __syncthreads();
+      if (d0 + kSimtD < D) {
+        fetch(h0, d0 + kSimtD);
+      } else if (h0 + kSimtHeads < H) {
+        fetch(h0 + kSimtHeads, 0);
+      }
+#pragma unroll
+      for (int d = 0; d < kSimtD; ++d) {
+        const float4 kv = *reinterpret_cast<const float4*>(&ks[d][key]);
+        const float4 qa = *reinterpret_cast<const float4*>(&qs[tr][d][0]), qb = *reinterpret_cast<const float4*>(&qs[tr][d][4]);
+        const float qv[kSimtHeads] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w};
+#pragma unroll
+        for (int h = 0; h < kSimtHeads; ++h) {
+          acc[h][0] = __fmaf_rn(qv[h], kv.x, acc[h][0]);
+          acc[h][1] = __fmaf_rn(qv[h], kv.y, acc[h][1]);
+          acc[h][2] = __fmaf_rn(qv[h], kv.z, acc[h][2]);
+          acc[h][3] = __fmaf_rn(qv[h], kv.w, acc[h][3]);
+        }
+      }
+    }
+    if (t < row_end) {
+#pragma unroll
+      for (int h = 0; h < kSimtHeads; ++h) {
+        const float wh = h0 + h < H ? __ldg(w + static_cast<size_t>(t) * H + h0 + h) : 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) total[j] = __fmaf_rn(wh, fmaxf(acc[h][j], 0.f), total[j]);
+      }
+    }
   }
-  __syncthreads();
-  const int s = s0 + threadIdx.x;
-  if (s >= N) return;
-  const float* kr = ks + threadIdx.x * (D + 1);
-  float total = 0.f;
-  for (int h = 0; h < H; ++h) {
-    const float* qh = qs + h * D;
-    float dot = 0.f;
-    for (int d = 0; d < D; ++d) dot = __fmaf_rn(qh[d], kr[d], dot);
-    total = __fmaf_rn(w[static_cast<size_t>(t) * H + h], fmaxf(dot, 0.f), total);
-  }
-  if (k_scale != nullptr) total *= k_scale[s];
-  total += 0.f;  // -0 -> +0
+  if (t >= row_end) return;
   const int vis = visible_keys(t, N, causal_offset);
-  out[static_cast<size_t>(blockIdx.y) * ld + s] = (s < vis) ? total : -INFINITY;
+  float* dst = out + static_cast<size_t>(t - row_begin) * ld + s0 + key;
+  float v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int s = s0 + key + j;
+    if (k_scale != nullptr && s < N) total[j] *= k_scale[s];
+    v[j] = s < vis ? total[j] + 0.f : -INFINITY;  // -0 -> +0
+  }
+  if (s0 + key + 3 < N && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (s0 + key + j < N) dst[j] = v[j];
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -928,28 +997,40 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
 
 }  // namespace
 
+namespace {
+template <int kDtype, int kRows>
+cudaError_t launch_simt_rows(const void* q, const float* w, const void* k, const float* k_scale, int N, int H, int D, int causal_offset,
+                             int row_begin, int row_end, float* out, long long ld, cudaStream_t stream) {
+  constexpr int kKeys = 128 * (8 / kRows);
+  const int tiles = (N + kKeys - 1) / kKeys;
+  // (at most 65,535 row blocks to a launch)
+  for (int r0 = row_begin; r0 < row_end; r0 += kRows * 65535) {
+    const int r1 = row_end - r0 < kRows * 65535 ? row_end : r0 + kRows * 65535;
+    simt_scores_kernel<kDtype, kRows><<<dim3(tiles, (r1 - r0 + kRows - 1) / kRows), kSimtThreads, 0, stream>>>(
+        q, w, k, k_scale, N, H, D, causal_offset, r0, r1, out + static_cast<size_t>(r0 - row_begin) * ld, ld);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+template <int kDtype>
+cudaError_t launch_simt_typed(const void* q, const float* w, const void* k, const float* k_scale, int N, int H, int D, int causal_offset,
+                              int row_begin, int row_end, float* out, long long ld, cudaStream_t stream) {
+  const int rows = row_end - row_begin;
+  // a key tile is read once per kRows query rows; a few rows over many keys give the warps more keys instead
+  if (rows > 4 || N <= 256 * 148) return launch_simt_rows<kDtype, 8>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
+  return launch_simt_rows<kDtype, 4>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
+}
+}  // namespace
+
 cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N,
                                int H, int D, int causal_offset, int row_begin, int row_end, float* out, long long ld,
                                cudaStream_t stream) {
   (void)T;
-  const int rows = row_end - row_begin;
-  if (rows <= 0) return cudaSuccess;
-  const size_t smem = (static_cast<size_t>(H) * D + 128 * (D + 1)) * sizeof(float);
-  dim3 grid((N + 127) / 128, rows);
-  cudaError_t e;
-#define LT_SIMT_CASE(DT)                                                                                              \
-  e = cudaFuncSetAttribute(simt_scores_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)); \
-  if (e != cudaSuccess) return e;                                                                                       \
-  simt_scores_kernel<DT><<<grid, 128, smem, stream>>>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, out, ld);
-  if (dtype == LT_DTYPE_F32) {
-    LT_SIMT_CASE(LT_DTYPE_F32)
-  } else if (dtype == LT_DTYPE_BF16) {
-    LT_SIMT_CASE(LT_DTYPE_BF16)
-  } else {
-    LT_SIMT_CASE(LT_DTYPE_E4M3)
-  }
-#undef LT_SIMT_CASE
-  return cudaGetLastError();
+  if (row_end <= row_begin) return cudaSuccess;
+  if (dtype == LT_DTYPE_F32) return launch_simt_typed<LT_DTYPE_F32>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
+  if (dtype == LT_DTYPE_BF16) return launch_simt_typed<LT_DTYPE_BF16>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
+  return launch_simt_typed<LT_DTYPE_E4M3>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
 }
 
 cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int rank, float* smin, float* width, float* thr,
