@@ -379,7 +379,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     return LT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   Control* ctl = reinterpret_cast<Control*>(ws + L.ctl);
-  LT_CUDA(cudaMemsetAsync(ws, 0, L.zero_end, stream));
+  LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
 
   if (!fused) {
     return run_unfused(dtype, false, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score,
@@ -717,7 +717,8 @@ int lt_topk_frequent(const int32_t* idx, int T, int topk, int N, int n_out, int3
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   unsigned int* counts = reinterpret_cast<unsigned int*>(ws);
   void* scratch = ws + align_up(static_cast<size_t>(N) * 4);
-  LT_CUDA(cudaMemsetAsync(counts, 0, static_cast<size_t>(N) * 4, stream));
+  // the counts and, behind them, the ranking's state, key list and ranks
+  LT_LAUNCH(launch_zero(ws, align_up(static_cast<size_t>(N) * 4) + align_up(rank_scratch_bytes(n_out)), stream));
   LT_LAUNCH(launch_count_positions(idx, static_cast<long long>(T) * topk, N, counts, stream));
   // rank the N (count, position) pairs with a grid-wide radix select and order the n_out winners; no position can
   // occur more often than there are entries
@@ -906,7 +907,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     return LT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   Control* ctl = reinterpret_cast<Control*>(ws + L.ctl);
-  LT_CUDA(cudaMemsetAsync(ws, 0, L.zero_end, stream));
+  LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
   const int grid = tun.grid > 0 ? tun.grid : sm_count();
   if (L.direct) {  // small problem: dense scores and a select over them (see use_direct)
     mark_phase(0, stream);
@@ -1078,7 +1079,7 @@ int lt_unfused_topk(int dtype, const void* q, const float* w, const void* k, con
   if (rows > T) rows = T;
   if (mma && rows >= kRowsPerBlock) rows -= rows % kRowsPerBlock;
   Control* ctl = reinterpret_cast<Control*>(score_buf);
-  LT_CUDA(cudaMemsetAsync(ctl, 0, kAlign, stream));
+  LT_LAUNCH(launch_zero(ctl, kAlign, stream));
   float* scores = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(score_buf) + kAlign);
   return run_unfused(dtype, mma, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score, scores,
                      static_cast<int>(rows), ctl, tun, stream);
@@ -1103,7 +1104,7 @@ int lt_indexer_topk_static(int dtype, const void* q, const float* w, const void*
   // the array keeps whatever the previous call left: the status block must start at zero; the
   // score rows are fully rewritten before they are read
   Control* ctl = static_cast<Control*>(base);
-  LT_CUDA(cudaMemsetAsync(ctl, 0, kAlign, stream));
+  LT_LAUNCH(launch_zero(ctl, kAlign, stream));
   float* scores = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + kAlign);
   return run_unfused(dtype, mma, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score, scores,
                      static_cast<int>(rows), ctl, tun, stream);

@@ -41,6 +41,17 @@ __device__ __forceinline__ bool lt_in_bounds(bool cond, Control* ctl) {
 #endif
 
 // ---------------------------------------------------------------------------------------------
+// Chained launches.  Every kernel of a call is launched so that it may start before the kernel ahead of it in the stream has
+// ended (launch_chained in lt_host.h): its launch latency and set-up then run beside the other's tail.  chain_begin()
+// lets the next kernel start as soon as every CTA of this one has; chain_wait() returns once everything ahead in the
+// stream has completed and its writes are visible.  EVERY thread of every kernel launched that way that touches global
+// memory calls chain_wait() before it does, on every path: a grid that ended without waiting would let the kernel
+// behind it run ahead of the kernel before it.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void chain_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// ---------------------------------------------------------------------------------------------
 // total order on (score, index): larger key = better.  Scores are canonicalised (-0 -> +0)
 // where they are produced, so bit order equals value order.
 // ---------------------------------------------------------------------------------------------

@@ -77,6 +77,8 @@ __global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_
   unsigned int list_len = 0;  // entries of earlier windows (uniform across the cluster)
 
   for (int i = tid; i < p.buf_words; i += kUnionThreads) masks[i] = 0u;
+  chain_begin();
+  chain_wait();
   for (long long wbase = 0; wbase < p.N; wbase += static_cast<long long>(p.window_words) * 32) {
     const long long left = p.N - wbase;
     const int span = static_cast<int>(left < static_cast<long long>(p.window_words) * 32 ? left : static_cast<long long>(p.window_words) * 32);
@@ -293,19 +295,7 @@ cudaError_t launch_dsa_union(const int32_t* idx, int T, int topk, int N, int gro
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned int>(width);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned int>(n_groups * width));
-  cfg.blockDim = dim3(kUnionThreads);
-  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, p);
+  return launch_chained(kernel, n_groups * width, kUnionThreads, smem, stream, width, p);
 }
 
 }  // namespace lt

@@ -5,9 +5,32 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "lt_common.cuh"
 
 namespace lt {
+
+// Launch of a kernel that calls chain_wait (see lt_common.cuh), optionally in clusters of `cluster` CTAs.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster,
+                                  Args&&... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = static_cast<unsigned int>(cluster);
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
 
 constexpr int kModeFilter = 0;
 constexpr int kModeDump = 1;
@@ -109,6 +132,9 @@ cudaError_t launch_scan_knn(int mode, const void* q, int T, const void* x, long 
                             const KnnScanParams& p, int grid, cudaStream_t stream);
 
 // ---- lt_select.cu ---------------------------------------------------------------------------
+// Clears `bytes` bytes at p (16-byte aligned, a multiple of 16): a kernel and not a memset, so that it chains.
+cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t stream);
+
 // Generic SIMT scoring (any H, D, dtype): dense scores of rows [row_begin, row_end), -inf where masked.
 cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N,
                                int H, int D, int causal_offset, int row_begin, int row_end, float* out, long long ld,

@@ -14,6 +14,8 @@ namespace {
 // counts[p] += 1 for every entry p of idx with 0 <= p < N (fire-and-forget atomics; 16-byte loads)
 __global__ void __launch_bounds__(256) count_positions_kernel(const int32_t* __restrict__ idx, long long n, int N,
                                                               unsigned int* __restrict__ counts) {
+  chain_begin();
+  chain_wait();
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
   long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const long long n4 = ((reinterpret_cast<uintptr_t>(idx) & 15u) == 0) ? n / 4 : 0;
@@ -59,6 +61,8 @@ __global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __re
   __shared__ unsigned int hist[256];
   __shared__ bool last;
   const unsigned long long mask = first_pass ? 0ull : (~0ull << (shift + 8));
+  chain_begin();
+  chain_wait();
   const unsigned long long prefix = st->prefix;
   hist[threadIdx.x] = 0;
   __syncthreads();
@@ -127,6 +131,8 @@ __global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __re
 // every key at or above the n_out-th largest goes to the list (any order; exactly n_out of them)
 __global__ void __launch_bounds__(256) rank_collect_kernel(const unsigned int* __restrict__ counts, int N, RankState* st,
                                                             unsigned long long* __restrict__ keys, int n_out, int pos_bits) {
+  chain_begin();
+  chain_wait();
   const unsigned long long kth = st->prefix;
   const int lane = threadIdx.x & 31;
   const int per_thread = (N + gridDim.x * blockDim.x - 1) / (gridDim.x * blockDim.x);
@@ -168,6 +174,8 @@ constexpr int kOrderSlice = 1024;
 __global__ void __launch_bounds__(256) rank_count_larger_kernel(const unsigned long long* __restrict__ keys, int n_out,
                                                                  unsigned int* __restrict__ rank) {
   __shared__ unsigned long long slice[kOrderSlice];
+  chain_begin();
+  chain_wait();
   const int s0 = blockIdx.y * kOrderSlice;
   const int len = min(kOrderSlice, n_out - s0);
   for (int i = threadIdx.x; i < len; i += blockDim.x) slice[i] = keys[s0 + i];
@@ -184,6 +192,8 @@ __global__ void __launch_bounds__(256) rank_count_larger_kernel(const unsigned l
 __global__ void __launch_bounds__(256) rank_write_kernel(const unsigned long long* __restrict__ keys, int n_out,
                                                           const unsigned int* __restrict__ rank, int pos_bits,
                                                           int32_t* __restrict__ out_pos, int32_t* __restrict__ out_count) {
+  chain_begin();
+  chain_wait();
   const int me = blockIdx.x * blockDim.x + threadIdx.x;
   if (me >= n_out) return;
   const unsigned long long key = keys[me];
@@ -202,6 +212,8 @@ __global__ void __launch_bounds__(256) gather_keys_kernel(const uint8_t* __restr
                                                           const int* __restrict__ page_table, long long pool_rows,
                                                           Control* ctl, uint8_t* __restrict__ out_k,
                                                           float* __restrict__ out_scale) {
+  chain_begin();
+  chain_wait();
   const int pieces = row_bytes >> 4;
   const long long g = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const long long j = g / pieces;
@@ -225,8 +237,7 @@ cudaError_t launch_count_positions(const int32_t* idx, long long n, int N, unsig
   long long blocks = (n / 4 + 255) / 256;
   if (blocks < 1) blocks = 1;
   if (blocks > 148 * 16) blocks = 148 * 16;
-  count_positions_kernel<<<static_cast<int>(blocks), 256, 0, stream>>>(idx, n, N, counts);
-  return cudaGetLastError();
+  return launch_chained(count_positions_kernel, static_cast<unsigned int>(blocks), 256, 0, stream, 1, idx, n, N, counts);
 }
 
 size_t rank_scratch_bytes(int n_out) { return 1280 + static_cast<size_t>(n_out) * 12; }
@@ -239,7 +250,7 @@ int bits_for(unsigned long long max_value) {
 }
 }  // namespace
 
-// Ranks the N counts and writes the n_out most frequent positions; scratch: rank_scratch_bytes(n_out) bytes,
+// Ranks the N counts and writes the n_out most frequent positions; scratch: rank_scratch_bytes(n_out) bytes, zeroed,
 // 256-byte aligned.  max_count: an upper bound of any count (it fixes how many digits the select has to visit).
 cudaError_t launch_rank_counts(const unsigned int* counts, int N, int n_out, unsigned long long max_count, void* scratch,
                                int32_t* out_pos, int32_t* out_count, cudaStream_t stream) {
@@ -247,33 +258,31 @@ cudaError_t launch_rank_counts(const unsigned int* counts, int N, int n_out, uns
   RankState* st = static_cast<RankState*>(scratch);
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(scratch) + 1280);
   unsigned int* rank = reinterpret_cast<unsigned int*>(keys + n_out);
-  cudaError_t e = cudaMemsetAsync(st, 0, sizeof(RankState), stream);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(rank, 0, static_cast<size_t>(n_out) * 4, stream);
-  if (e != cudaSuccess) return e;
   if (max_count > 0xffffffffull) max_count = 0xffffffffull;
   const int pos_bits = bits_for(static_cast<unsigned long long>(N - 1));
   const int passes = (bits_for(max_count) + pos_bits + 7) / 8;
   int blocks = (N + 256 * kRankBatch - 1) / (256 * kRankBatch);
   if (blocks < 1) blocks = 1;
   if (blocks > 148 * 4) blocks = 148 * 4;
-  for (int pass = 0; pass < passes; ++pass)
-    rank_pass_kernel<<<blocks, 256, 0, stream>>>(counts, N, st, 8 * (passes - 1 - pass), pass == 0 ? 1 : 0, pos_bits, n_out);
-  rank_collect_kernel<<<blocks, 256, 0, stream>>>(counts, N, st, keys, n_out, pos_bits);
+  cudaError_t e = cudaSuccess;
+  for (int pass = 0; pass < passes && e == cudaSuccess; ++pass)
+    e = launch_chained(rank_pass_kernel, blocks, 256, 0, stream, 1, counts, N, st, 8 * (passes - 1 - pass), pass == 0 ? 1 : 0, pos_bits, n_out);
+  if (e == cudaSuccess) e = launch_chained(rank_collect_kernel, blocks, 256, 0, stream, 1, counts, N, st, keys, n_out, pos_bits);
   const int key_blocks = (n_out + 255) / 256;
-  rank_count_larger_kernel<<<dim3(key_blocks, (n_out + kOrderSlice - 1) / kOrderSlice), 256, 0, stream>>>(keys, n_out, rank);
-  rank_write_kernel<<<key_blocks, 256, 0, stream>>>(keys, n_out, rank, pos_bits, out_pos, out_count);
-  return cudaGetLastError();
+  if (e == cudaSuccess)
+    e = launch_chained(rank_count_larger_kernel, dim3(key_blocks, (n_out + kOrderSlice - 1) / kOrderSlice), 256, 0, stream, 1, keys, n_out, rank);
+  if (e == cudaSuccess)
+    e = launch_chained(rank_write_kernel, key_blocks, 256, 0, stream, 1, keys, n_out, rank, pos_bits, out_pos, out_count);
+  return e;
 }
 
 cudaError_t launch_gather_keys(const void* k, const float* k_scale, const int32_t* sample_idx, long long stride, int n_sample,
                                int N, int row_bytes, const int* page_table, long long pool_rows, Control* ctl, void* out_k,
                                float* out_scale, cudaStream_t stream) {
   const long long threads = static_cast<long long>(n_sample) * (row_bytes >> 4);
-  gather_keys_kernel<<<static_cast<int>((threads + 255) / 256), 256, 0, stream>>>(
-      static_cast<const uint8_t*>(k), k_scale, sample_idx, stride, n_sample, N, row_bytes, page_table, pool_rows, ctl,
-      static_cast<uint8_t*>(out_k), out_scale);
-  return cudaGetLastError();
+  return launch_chained(gather_keys_kernel, static_cast<unsigned int>((threads + 255) / 256), 256, 0, stream, 1,
+                        static_cast<const uint8_t*>(k), k_scale, sample_idx, stride, n_sample, N, row_bytes, page_table, pool_rows, ctl,
+                        static_cast<uint8_t*>(out_k), out_scale);
 }
 
 }  // namespace lt

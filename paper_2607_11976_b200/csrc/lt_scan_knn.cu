@@ -166,9 +166,11 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
 
+  chain_begin();
   // a fallback round has nothing to do unless some block of 8 rows in [row_begin, row_end) was flagged
   // (uniform across the grid)
   if (p.fb_flag != nullptr) {
+    chain_wait();
     unsigned int any = 0u;
     for (int b = p.row_begin / kRowsPerBlock; b * kRowsPerBlock < p.row_end; ++b) any |= p.fb_flag[b];
     if (any == 0u) return;
@@ -202,6 +204,7 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem_base = st->tmem_base;
   volatile int* abort_flag = &st->abort_flag;
+  chain_wait();  // barriers, TMEM and tensor maps are ready by now
 
   const int qb_lo = p.row_begin / kQB;
   const int n_qb = (p.row_end - 1) / kQB - qb_lo + 1;
@@ -519,8 +522,7 @@ cudaError_t knn_launch(const CUtensorMap& tq, const CUtensorMap& tx, const KnnSc
   const int bytes = knn_smem_bytes(p.D / kSliceElems);
   cudaError_t e = cudaFuncSetAttribute(knn_scan_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, knn_smem_bytes(kKnnMaxSlices));
   if (e != cudaSuccess) return e;
-  knn_scan_kernel<kMode><<<grid, kKnnThreads, bytes, stream>>>(tq, tx, p);
-  return cudaGetLastError();
+  return launch_chained(knn_scan_kernel<kMode>, grid, kKnnThreads, bytes, stream, 1, tq, tx, p);
 }
 
 }  // namespace

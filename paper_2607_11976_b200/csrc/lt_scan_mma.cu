@@ -259,8 +259,12 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
 
+  chain_begin();
   // a fallback round with no flagged block left has nothing to do (uniform across the CTA)
-  if (p.fb_list != nullptr && *p.fb_blocks <= p.fb_round_base) return;
+  if (p.fb_list != nullptr) {
+    chain_wait();
+    if (*p.fb_blocks <= p.fb_round_base) return;
+  }
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < C::kStages; ++i) {
@@ -290,6 +294,7 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   tc_fence_after();
   const uint32_t tmem_base = st->tmem_base;
   volatile int* abort_flag = &st->abort_flag;
+  chain_wait();  // barriers, TMEM and tensor maps are ready by now
 
   // number of query blocks / items of this launch
   int n_blocks;
@@ -667,8 +672,7 @@ cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const ScanP
   constexpr int bytes = smem_bytes<kFp8, kU, kUQ>();
   cudaError_t e = cudaFuncSetAttribute(scan_kernel<kFp8, kMode, kPaged, kU, kUQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  scan_kernel<kFp8, kMode, kPaged, kU, kUQ><<<grid, kThreads, bytes, stream>>>(tq, tk, p);
-  return cudaGetLastError();
+  return launch_chained(scan_kernel<kFp8, kMode, kPaged, kU, kUQ>, grid, kThreads, bytes, stream, 1, tq, tk, p);
 }
 // the paged variant is a separate instantiation so that the dense kernels carry none of its address arithmetic; the
 // one-unit variants serve chunks of at most kUnitQ rows (see Cfg)

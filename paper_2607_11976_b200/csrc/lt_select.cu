@@ -36,6 +36,13 @@ __device__ __forceinline__ float load_elem(const void* base, size_t i) {
   return __half2float(__half(hr));
 }
 
+__global__ void __launch_bounds__(256) zero_kernel(uint4* p, long long n) {
+  chain_begin();
+  chain_wait();
+  for (long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x; i < n; i += static_cast<long long>(gridDim.x) * 256)
+    p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 constexpr int kSimtThreads = 256;
 constexpr int kSimtD = 16;           // coordinates staged at a time
 constexpr int kSimtHeads = 8;        // heads in registers
@@ -71,6 +78,8 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void
       qr[j] = in && h0 + hj < H && t0 + rj + 2 * j < row_end
                   ? load_elem<kDtype>(q, q_at + static_cast<size_t>(h0) * D + d0 + static_cast<size_t>(j) * 2 * H * D) : 0.f;
   };
+  chain_begin();
+  chain_wait();
   fetch(0, 0);
   float total[4] = {0.f, 0.f, 0.f, 0.f};
   for (int h0 = 0; h0 < H; h0 += kSimtHeads) {
@@ -150,6 +159,8 @@ __global__ void __launch_bounds__(kStatsMaxThreads) sample_stats_kernel(const fl
   const int t = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* row = sample + static_cast<size_t>(t) * n_sample;
+  chain_begin();
+  chain_wait();
   // minimum and maximum in ordered bit patterns (integer warp reductions)
   unsigned int mn = 0xffffffffu, mx = 0u;
   for (int base = tid; base < n_sample; base += n_threads * kStatsBatch) {
@@ -334,6 +345,8 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
   const int t = blockIdx.x;
   const int lane = threadIdx.x & 31;
   const uint2* cand = p.cand + static_cast<size_t>(t) * p.cap;
+  chain_begin();
+  chain_wait();
   // The candidates are fetched without waiting for their number: most rows have between 1 and 2 topk of them.
   uint2 first[kFineBatch];
   const int ahead = min(p.cap, 2 * p.topk);
@@ -685,6 +698,8 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
   unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
   uint64_t* sel = sel_smem + kFineBins * 4 / 8;
   int t;
+  chain_begin();
+  chain_wait();
   if (p.fb_list != nullptr) {
     int j = p.fb_round_base + blockIdx.x / p.rows_per_block;
     if (j >= *p.fb_blocks) return;
@@ -785,6 +800,8 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
   const int kk = p.topk < vis ? p.topk : vis;
   int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
   float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
+  chain_begin();
+  chain_wait();
   if (kk == 0) {  // the whole cluster
     if (rank == 0) sort_and_write(list, 0, p.topk, out_idx, out_score, p.N, p.ctl);
     return;
@@ -1006,9 +1023,9 @@ cudaError_t launch_simt_rows(const void* q, const float* w, const void* k, const
   // (at most 65,535 row blocks to a launch)
   for (int r0 = row_begin; r0 < row_end; r0 += kRows * 65535) {
     const int r1 = row_end - r0 < kRows * 65535 ? row_end : r0 + kRows * 65535;
-    simt_scores_kernel<kDtype, kRows><<<dim3(tiles, (r1 - r0 + kRows - 1) / kRows), kSimtThreads, 0, stream>>>(
-        q, w, k, k_scale, N, H, D, causal_offset, r0, r1, out + static_cast<size_t>(r0 - row_begin) * ld, ld);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_chained(simt_scores_kernel<kDtype, kRows>, dim3(tiles, (r1 - r0 + kRows - 1) / kRows), kSimtThreads, 0,
+                                         stream, 1, q, w, k, k_scale, N, H, D, causal_offset, r0, r1,
+                                         out + static_cast<size_t>(r0 - row_begin) * ld, ld);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1022,6 +1039,13 @@ cudaError_t launch_simt_typed(const void* q, const float* w, const void* k, cons
   return launch_simt_rows<kDtype, 4>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
 }
 }  // namespace
+
+cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t stream) {
+  const long long n = static_cast<long long>(bytes / 16);
+  if (n <= 0) return cudaSuccess;
+  const long long blocks = (n + 1023) / 1024 < 592 ? (n + 1023) / 1024 : 592;
+  return launch_chained(zero_kernel, static_cast<unsigned int>(blocks), 256, 0, stream, 1, static_cast<uint4*>(p), n);
+}
 
 cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N,
                                int H, int D, int causal_offset, int row_begin, int row_end, float* out, long long ld,
@@ -1037,8 +1061,7 @@ cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int ra
                                 cudaStream_t stream) {
   // few rows leave the chip idle: a large CTA then shortens the sweeps; with many rows small CTAs overlap better
   const int threads = T <= 296 ? 1024 : 256;
-  sample_stats_kernel<<<T, threads, 0, stream>>>(sample, n_sample, rank, smin, width, thr);
-  return cudaGetLastError();
+  return launch_chained(sample_stats_kernel, T, threads, 0, stream, 1, sample, n_sample, rank, smin, width, thr);
 }
 
 cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream) {
@@ -1050,8 +1073,7 @@ cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream)
   const int smem = sel_cap * static_cast<int>(sizeof(uint64_t));
   cudaError_t e = cudaFuncSetAttribute(final_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  final_select_kernel<<<p.T, kFinalThreads, smem, stream>>>(p, sel_cap);
-  return cudaGetLastError();
+  return launch_chained(final_select_kernel, p.T, kFinalThreads, smem, stream, 1, p, sel_cap);
 }
 
 cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t stream) {
@@ -1075,19 +1097,7 @@ cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t str
     e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
   }
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned int>(width);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned int>(p.n_blocks * width));
-  cfg.blockDim = dim3(kClThreads);
-  cfg.dynamicSmemBytes = static_cast<size_t>(smem);
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, select_cluster_kernel, p);
+  return launch_chained(select_cluster_kernel, p.n_blocks * width, kClThreads, smem, stream, width, p);
 }
 
 namespace {
@@ -1095,8 +1105,7 @@ template <int kThreads>
 cudaError_t launch_select_rows_n(const SelectRowsParams& p, int smem, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(select_rows_kernel<kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  select_rows_kernel<kThreads><<<p.n_blocks, kThreads, smem, stream>>>(p);
-  return cudaGetLastError();
+  return launch_chained(select_rows_kernel<kThreads>, p.n_blocks, kThreads, smem, stream, 1, p);
 }
 }  // namespace
 
