@@ -141,12 +141,14 @@ def _ptr(t: Optional[torch.Tensor]):
         return None
     if not t.is_cuda or not t.is_contiguous():
         raise ValueError("expected a contiguous CUDA tensor")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()  # (the functions' argtypes make pointers of plain integers)
 
 
-def _stream(stream) -> ctypes.c_void_p:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    # the current stream's handle without building a Stream object, which costs as much as a kernel launch
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _check(code: int, what: str) -> None:
@@ -201,7 +203,7 @@ def lt_indexer_topk_strided(dtype, q, w, k_view, k_scale, topk: int, causal_offs
     N, D2 = k_view.shape
     if D2 != D or k_view.stride(1) != 1 or not k_view.is_cuda:
         raise ValueError("expected an [N, D] CUDA view with unit inner stride")
-    _check(load().lt_indexer_topk_strided(dtype_code(dtype), _ptr(q), _ptr(w), ctypes.c_void_p(k_view.data_ptr()),
+    _check(load().lt_indexer_topk_strided(dtype_code(dtype), _ptr(q), _ptr(w), k_view.data_ptr(),
                                           int(k_view.stride(0)), _ptr(k_scale), T, N, H, D, topk, causal_offset,
                                           _ptr(out_idx), _ptr(out_score), _ptr(workspace),
                                           workspace.numel() * workspace.element_size(),

@@ -288,13 +288,10 @@ cudaError_t launch_dsa_union(const int32_t* idx, int T, int topk, int N, int gro
   const long long all_rows = static_cast<long long>(p.mask_words) * p.rows_per_cta;
   p.buf_words = all_rows < kMaskBufWords ? static_cast<int>(all_rows + 3) / 4 * 4 : kMaskBufWords;
   const int smem = (p.window_words + prefix_words(word_prefix, p.window_words) + p.buf_words) * 4;
+  static std::atomic<unsigned long long> done[2];
   auto kernel = word_prefix ? dsa_union_kernel<true> : dsa_union_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel), done[word_prefix ? 1 : 0], true);
   if (e != cudaSuccess) return e;
-  if (width > 8) {
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
   return launch_chained(kernel, n_groups * width, kUnionThreads, smem, stream, width, p);
 }
 

@@ -5,11 +5,29 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 #include "lt_common.cuh"
 
 namespace lt {
+
+// Lets a kernel use all the dynamic shared memory an SM has (and clusters of 16).  A property of the loaded function on a device,
+// set once for each: `done` holds one bit per device and belongs to that kernel alone.
+inline cudaError_t allow_smem(const void* kernel, std::atomic<unsigned long long>& done, bool wide_clusters = false) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  cudaFuncAttributes a;
+  e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - static_cast<int>(a.sharedSizeBytes));
+  if (e == cudaSuccess && wide_clusters) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
 
 // Launch of a kernel that calls chain_wait (see lt_common.cuh), optionally in clusters of `cluster` CTAs.
 template <typename... Params, typename... Args>

@@ -520,7 +520,8 @@ bool knn_map(CUtensorMap* map, const void* base, uint64_t d, uint64_t rows, uint
 template <int kMode>
 cudaError_t knn_launch(const CUtensorMap& tq, const CUtensorMap& tx, const KnnScanParams& p, int grid, cudaStream_t stream) {
   const int bytes = knn_smem_bytes(p.D / kSliceElems);
-  cudaError_t e = cudaFuncSetAttribute(knn_scan_kernel<kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize, knn_smem_bytes(kKnnMaxSlices));
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(knn_scan_kernel<kMode>), done);
   if (e != cudaSuccess) return e;
   return launch_chained(knn_scan_kernel<kMode>, grid, kKnnThreads, bytes, stream, 1, tq, tx, p);
 }

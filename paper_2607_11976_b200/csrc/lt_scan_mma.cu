@@ -670,7 +670,8 @@ bool make_map(CUtensorMap* map, bool fp8, const void* base, uint64_t rows, uint6
 template <bool kFp8, int kMode, bool kPaged, int kU, int kUQ>
 cudaError_t launch_one(const CUtensorMap& tq, const CUtensorMap& tk, const ScanParams& p, int grid, cudaStream_t stream) {
   constexpr int bytes = smem_bytes<kFp8, kU, kUQ>();
-  cudaError_t e = cudaFuncSetAttribute(scan_kernel<kFp8, kMode, kPaged, kU, kUQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(scan_kernel<kFp8, kMode, kPaged, kU, kUQ>), done);
   if (e != cudaSuccess) return e;
   return launch_chained(scan_kernel<kFp8, kMode, kPaged, kU, kUQ>, grid, kThreads, bytes, stream, 1, tq, tk, p);
 }

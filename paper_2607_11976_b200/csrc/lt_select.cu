@@ -1071,7 +1071,8 @@ cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream)
   if (sel_cap < 8192) sel_cap = 8192;
   if (sel_cap > kSelCap) sel_cap = kSelCap;
   const int smem = sel_cap * static_cast<int>(sizeof(uint64_t));
-  cudaError_t e = cudaFuncSetAttribute(final_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(final_select_kernel), done);
   if (e != cudaSuccess) return e;
   return launch_chained(final_select_kernel, p.T, kFinalThreads, smem, stream, 1, p, sel_cap);
 }
@@ -1091,19 +1092,17 @@ cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t str
   p.slice_keys = slice_want < slice_max ? slice_want : slice_max;
   const int tail = p.slice_keys * 4 > list ? p.slice_keys * 4 : list;
   const int smem = list + kFineBins * 4 + tail;
-  cudaError_t e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_cluster_kernel), done, true);
   if (e != cudaSuccess) return e;
-  if (width > 8) {
-    e = cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
   return launch_chained(select_cluster_kernel, p.n_blocks * width, kClThreads, smem, stream, width, p);
 }
 
 namespace {
 template <int kThreads>
 cudaError_t launch_select_rows_n(const SelectRowsParams& p, int smem, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(select_rows_kernel<kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static std::atomic<unsigned long long> done{0};
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_rows_kernel<kThreads>), done);
   if (e != cudaSuccess) return e;
   return launch_chained(select_rows_kernel<kThreads>, p.n_blocks, kThreads, smem, stream, 1, p);
 }
