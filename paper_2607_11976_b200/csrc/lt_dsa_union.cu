@@ -77,7 +77,6 @@ __global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_
   unsigned int list_len = 0;  // entries of earlier windows (uniform across the cluster)
 
   for (int i = tid; i < p.buf_words; i += kUnionThreads) masks[i] = 0u;
-  chain_begin();
   chain_wait();
   for (long long wbase = 0; wbase < p.N; wbase += static_cast<long long>(p.window_words) * 32) {
     const long long left = p.N - wbase;

@@ -14,7 +14,6 @@ namespace {
 // counts[p] += 1 for every entry p of idx with 0 <= p < N (fire-and-forget atomics; 16-byte loads)
 __global__ void __launch_bounds__(256) count_positions_kernel(const int32_t* __restrict__ idx, long long n, int N,
                                                               unsigned int* __restrict__ counts) {
-  chain_begin();
   chain_wait();
   const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
   long long i = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -61,7 +60,6 @@ __global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __re
   __shared__ unsigned int hist[256];
   __shared__ bool last;
   const unsigned long long mask = first_pass ? 0ull : (~0ull << (shift + 8));
-  chain_begin();
   chain_wait();
   const unsigned long long prefix = st->prefix;
   hist[threadIdx.x] = 0;
@@ -131,7 +129,6 @@ __global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __re
 // every key at or above the n_out-th largest goes to the list (any order; exactly n_out of them)
 __global__ void __launch_bounds__(256) rank_collect_kernel(const unsigned int* __restrict__ counts, int N, RankState* st,
                                                             unsigned long long* __restrict__ keys, int n_out, int pos_bits) {
-  chain_begin();
   chain_wait();
   const unsigned long long kth = st->prefix;
   const int lane = threadIdx.x & 31;
@@ -174,7 +171,6 @@ constexpr int kOrderSlice = 1024;
 __global__ void __launch_bounds__(256) rank_count_larger_kernel(const unsigned long long* __restrict__ keys, int n_out,
                                                                  unsigned int* __restrict__ rank) {
   __shared__ unsigned long long slice[kOrderSlice];
-  chain_begin();
   chain_wait();
   const int s0 = blockIdx.y * kOrderSlice;
   const int len = min(kOrderSlice, n_out - s0);
@@ -192,7 +188,6 @@ __global__ void __launch_bounds__(256) rank_count_larger_kernel(const unsigned l
 __global__ void __launch_bounds__(256) rank_write_kernel(const unsigned long long* __restrict__ keys, int n_out,
                                                           const unsigned int* __restrict__ rank, int pos_bits,
                                                           int32_t* __restrict__ out_pos, int32_t* __restrict__ out_count) {
-  chain_begin();
   chain_wait();
   const int me = blockIdx.x * blockDim.x + threadIdx.x;
   if (me >= n_out) return;
@@ -212,7 +207,6 @@ __global__ void __launch_bounds__(256) gather_keys_kernel(const uint8_t* __restr
                                                           const int* __restrict__ page_table, long long pool_rows,
                                                           Control* ctl, uint8_t* __restrict__ out_k,
                                                           float* __restrict__ out_scale) {
-  chain_begin();
   chain_wait();
   const int pieces = row_bytes >> 4;
   const long long g = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;

@@ -166,7 +166,6 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
 
-  chain_begin();
   // a fallback round has nothing to do unless some block of 8 rows in [row_begin, row_end) was flagged
   // (uniform across the grid)
   if (p.fb_flag != nullptr) {

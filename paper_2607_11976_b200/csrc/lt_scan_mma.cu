@@ -261,7 +261,6 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
 
-  chain_begin();
   // a fallback round with no flagged block left has nothing to do (uniform across the CTA)
   if (p.fb_list != nullptr) {
     chain_wait();

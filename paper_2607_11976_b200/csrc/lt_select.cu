@@ -37,7 +37,6 @@ __device__ __forceinline__ float load_elem(const void* base, size_t i) {
 }
 
 __global__ void __launch_bounds__(256) zero_kernel(uint4* p, long long n) {
-  chain_begin();
   chain_wait();
   for (long long i = static_cast<long long>(blockIdx.x) * 256 + threadIdx.x; i < n; i += static_cast<long long>(gridDim.x) * 256)
     p[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -78,7 +77,6 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void
       qr[j] = in && h0 + hj < H && t0 + rj + 2 * j < row_end
                   ? load_elem<kDtype>(q, q_at + static_cast<size_t>(h0) * D + d0 + static_cast<size_t>(j) * 2 * H * D) : 0.f;
   };
-  chain_begin();
   chain_wait();
   fetch(0, 0);
   float total[4] = {0.f, 0.f, 0.f, 0.f};
@@ -159,7 +157,6 @@ __global__ void __launch_bounds__(kStatsMaxThreads) sample_stats_kernel(const fl
   const int t = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* row = sample + static_cast<size_t>(t) * n_sample;
-  chain_begin();
   chain_wait();
   // minimum and maximum in ordered bit patterns (integer warp reductions)
   unsigned int mn = 0xffffffffu, mx = 0u;
@@ -345,7 +342,6 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
   const int t = blockIdx.x;
   const int lane = threadIdx.x & 31;
   const uint2* cand = p.cand + static_cast<size_t>(t) * p.cap;
-  chain_begin();
   chain_wait();
   // The candidates are fetched without waiting for their number: most rows have between 1 and 2 topk of them.
   uint2 first[kFineBatch];
@@ -698,7 +694,6 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
   unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
   uint64_t* sel = sel_smem + kFineBins * 4 / 8;
   int t;
-  chain_begin();
   chain_wait();
   if (p.fb_list != nullptr) {
     int j = p.fb_round_base + blockIdx.x / p.rows_per_block;
@@ -800,7 +795,6 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
   const int kk = p.topk < vis ? p.topk : vis;
   int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
   float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
-  chain_begin();
   chain_wait();
   if (kk == 0) {  // the whole cluster
     if (rank == 0) sort_and_write(list, 0, p.topk, out_idx, out_score, p.N, p.ctl);
