@@ -307,6 +307,7 @@ cudaError_t launch_scan(bool abs_form, int dtype, int mode, const void* q, int T
 __device__ Control g_scores_ctl;
 
 // ---- the generic path: dense scores of a few rows at a time, then a full-row select ----------
+// ctl need not be cleared by the caller when mma is false
 int run_unfused(int dtype, bool mma, const void* q, const float* w, const void* k, const float* k_scale, int T, int N, int H,
                 int D, int topk, int causal_offset, int32_t* out_idx, float* out_score, float* scores, int rows_per_pass,
                 Control* ctl, const Tun& tun, cudaStream_t stream) {
@@ -332,7 +333,7 @@ int run_unfused(int dtype, bool mma, const void* q, const float* w, const void* 
       p.ctl = ctl;
       LT_LAUNCH(launch_scan_mma(dtype, kModeDump, q, T, k, N, D, p, grid, stream));
     } else {
-      LT_LAUNCH(launch_simt_scores(dtype, q, w, k, k_scale, T, N, H, D, causal_offset, r0, r1, scores, N, stream));
+      LT_LAUNCH(launch_simt_scores(dtype, q, w, k, k_scale, T, N, H, D, causal_offset, r0, r1, scores, N, r0 == 0 ? ctl : nullptr, stream));
     }
     if (topk > 0) {
       SelectRowsParams sp{};
@@ -347,7 +348,8 @@ int run_unfused(int dtype, bool mma, const void* q, const float* w, const void* 
       sp.out_idx = out_idx;
       sp.out_score = out_score;
       sp.ctl = ctl;
-      LT_LAUNCH(launch_select_rows(sp, stream));
+      // rows on 16-byte boundaries can be shared by clusters of CTAs
+      LT_LAUNCH(N % 4 == 0 ? launch_select_dense(sp, stream) : launch_select_rows(sp, stream));
     }
   }
   return LT_OK;
@@ -379,7 +381,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     return LT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   Control* ctl = reinterpret_cast<Control*>(ws + L.ctl);
-  LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
+  if (fused) LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
 
   if (!fused) {
     return run_unfused(dtype, false, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score,
@@ -840,7 +842,7 @@ int lt_indexer_scores(int dtype, const void* q, const float* w, const void* k, c
     LT_LAUNCH(launch_scan(abs_form, dtype, kModeDump, q, T, k, N, D, p, grid, stream));
     if (lin != nullptr) LT_CUDA(cudaFreeAsync(lin, stream));
   } else {
-    LT_LAUNCH(launch_simt_scores(dtype, q, w, k, kk, T, N, H, D, causal_offset, row_begin, row_end, out_scores, N, stream));
+    LT_LAUNCH(launch_simt_scores(dtype, q, w, k, kk, T, N, H, D, causal_offset, row_begin, row_end, out_scores, N, nullptr, stream));
   }
   return LT_OK;
 }
@@ -1079,7 +1081,7 @@ int lt_unfused_topk(int dtype, const void* q, const float* w, const void* k, con
   if (rows > T) rows = T;
   if (mma && rows >= kRowsPerBlock) rows -= rows % kRowsPerBlock;
   Control* ctl = reinterpret_cast<Control*>(score_buf);
-  LT_LAUNCH(launch_zero(ctl, kAlign, stream));
+  if (mma) LT_LAUNCH(launch_zero(ctl, kAlign, stream));
   float* scores = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(score_buf) + kAlign);
   return run_unfused(dtype, mma, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score, scores,
                      static_cast<int>(rows), ctl, tun, stream);
@@ -1104,7 +1106,7 @@ int lt_indexer_topk_static(int dtype, const void* q, const float* w, const void*
   // the array keeps whatever the previous call left: the status block must start at zero; the
   // score rows are fully rewritten before they are read
   Control* ctl = static_cast<Control*>(base);
-  LT_LAUNCH(launch_zero(ctl, kAlign, stream));
+  if (mma) LT_LAUNCH(launch_zero(ctl, kAlign, stream));
   float* scores = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + kAlign);
   return run_unfused(dtype, mma, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score, scores,
                      static_cast<int>(rows), ctl, tun, stream);

@@ -153,10 +153,11 @@ cudaError_t launch_scan_knn(int mode, const void* q, int T, const void* x, long 
 // Clears `bytes` bytes at p (16-byte aligned, a multiple of 16): a kernel and not a memset, so that it chains.
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t stream);
 
+// clear_ctl: a control block to clear on the way, or null.
 // Generic SIMT scoring (any H, D, dtype): dense scores of rows [row_begin, row_end), -inf where masked.
 cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N,
                                int H, int D, int causal_offset, int row_begin, int row_end, float* out, long long ld,
-                               cudaStream_t stream);
+                               Control* clear_ctl, cudaStream_t stream);
 
 // Sample statistics (paper Sec. 3.2 "Sampling"): per row min / max of the sampled scores, bin
 // width, and the threshold edge of the bin holding the rank-th largest sampled score.

@@ -51,7 +51,7 @@ template <int kDtype, int kRows>
 __global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void* __restrict__ q, const float* __restrict__ w,
                                                                    const void* __restrict__ k, const float* __restrict__ k_scale, int N,
                                                                    int H, int D, int causal_offset, int row_begin, int row_end,
-                                                                   float* __restrict__ out, long long ld) {
+                                                                   float* __restrict__ out, long long ld, Control* clear_ctl) {
   constexpr int kKeys = 128 * (8 / kRows);  // keys of the CTA's tile
   __shared__ __align__(16) float ks[kSimtD][kKeys + kSimtKeyPad];
   __shared__ __align__(16) float qs[kRows][kSimtD][kSimtHeads];
@@ -78,6 +78,8 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void
                   ? load_elem<kDtype>(q, q_at + static_cast<size_t>(h0) * D + d0 + static_cast<size_t>(j) * 2 * H * D) : 0.f;
   };
   chain_wait();
+  // the status block of the call, which only later kernels write to
+  if (clear_ctl != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && tid < static_cast<int>(sizeof(Control) / 4)) reinterpret_cast<int*>(clear_ctl)[tid] = 0;
   fetch(0, 0);
   float total[4] = {0.f, 0.f, 0.f, 0.f};
   for (int h0 = 0; h0 < H; h0 += kSimtHeads) {
@@ -1011,7 +1013,7 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
 namespace {
 template <int kDtype, int kRows>
 cudaError_t launch_simt_rows(const void* q, const float* w, const void* k, const float* k_scale, int N, int H, int D, int causal_offset,
-                             int row_begin, int row_end, float* out, long long ld, cudaStream_t stream) {
+                             int row_begin, int row_end, float* out, long long ld, Control* clear_ctl, cudaStream_t stream) {
   constexpr int kKeys = 128 * (8 / kRows);
   const int tiles = (N + kKeys - 1) / kKeys;
   // (at most 65,535 row blocks to a launch)
@@ -1019,18 +1021,18 @@ cudaError_t launch_simt_rows(const void* q, const float* w, const void* k, const
     const int r1 = row_end - r0 < kRows * 65535 ? row_end : r0 + kRows * 65535;
     const cudaError_t e = launch_chained(simt_scores_kernel<kDtype, kRows>, dim3(tiles, (r1 - r0 + kRows - 1) / kRows), kSimtThreads, 0,
                                          stream, 1, q, w, k, k_scale, N, H, D, causal_offset, r0, r1,
-                                         out + static_cast<size_t>(r0 - row_begin) * ld, ld);
+                                         out + static_cast<size_t>(r0 - row_begin) * ld, ld, r0 == row_begin ? clear_ctl : nullptr);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 template <int kDtype>
 cudaError_t launch_simt_typed(const void* q, const float* w, const void* k, const float* k_scale, int N, int H, int D, int causal_offset,
-                              int row_begin, int row_end, float* out, long long ld, cudaStream_t stream) {
+                              int row_begin, int row_end, float* out, long long ld, Control* clear_ctl, cudaStream_t stream) {
   const int rows = row_end - row_begin;
   // a key tile is read once per kRows query rows; a few rows over many keys give the warps more keys instead
-  if (rows > 4 || N <= 256 * 148) return launch_simt_rows<kDtype, 8>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
-  return launch_simt_rows<kDtype, 4>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
+  if (rows > 4 || N <= 256 * 148) return launch_simt_rows<kDtype, 8>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, clear_ctl, stream);
+  return launch_simt_rows<kDtype, 4>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, clear_ctl, stream);
 }
 }  // namespace
 
@@ -1043,12 +1045,12 @@ cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t stream) {
 
 cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N,
                                int H, int D, int causal_offset, int row_begin, int row_end, float* out, long long ld,
-                               cudaStream_t stream) {
+                               Control* clear_ctl, cudaStream_t stream) {
   (void)T;
   if (row_end <= row_begin) return cudaSuccess;
-  if (dtype == LT_DTYPE_F32) return launch_simt_typed<LT_DTYPE_F32>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
-  if (dtype == LT_DTYPE_BF16) return launch_simt_typed<LT_DTYPE_BF16>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
-  return launch_simt_typed<LT_DTYPE_E4M3>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, stream);
+  if (dtype == LT_DTYPE_F32) return launch_simt_typed<LT_DTYPE_F32>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, clear_ctl, stream);
+  if (dtype == LT_DTYPE_BF16) return launch_simt_typed<LT_DTYPE_BF16>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, clear_ctl, stream);
+  return launch_simt_typed<LT_DTYPE_E4M3>(q, w, k, k_scale, N, H, D, causal_offset, row_begin, row_end, out, ld, clear_ctl, stream);
 }
 
 cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int rank, float* smin, float* width, float* thr,
