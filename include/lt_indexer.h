@@ -75,7 +75,8 @@ extern "C" {
 #define LT_BINS 256 /* m, the number of equal-width score bins (paper Sec. 3.2, "Sampling") */
 
 /* which implementation lt_indexer_topk_ex uses */
-#define LT_PATH_AUTO 0    /* fused tensor-core path when the shape allows it, else generic */
+#define LT_PATH_AUTO 0    /* tensor-core path when the shape allows it (small problems: dense scores and a full-row
+                             select, nothing sampled or filtered; else fused), else generic; same bits either way */
 #define LT_PATH_FUSED 1   /* fused tcgen05 path; LT_ERR_UNSUPPORTED if the shape does not fit */
 #define LT_PATH_GENERIC 2 /* generic SIMT scoring + full-row select (any H, D, dtype)      */
 #define LT_PATH_FUSED_ABS 3 /* fp8 only: an alternative fused tensor-core scan that evaluates Eq. 1 as
@@ -335,7 +336,8 @@ int lt_indexer_topk_static_max_keys(void);
 /*
  * Copies the 8-int status block of a workspace to host memory after synchronising
  * `stream`: [0] LT_STATUS_* bits, [1] rows that took the fallback, [2] largest
- * survivor count of any row, [3] total survivors (low 31 bits, saturating),
+ * survivor count of any row, [3] total survivors (low 31 bits, saturating; both 0
+ * where LT_PATH_AUTO took the dense form of small problems),
  * [4] rows whose candidate buffer overflowed, [5..7] reserved.
  * workspace == NULL reads the library-owned workspace of lt_indexer_topk.
  */
