@@ -97,16 +97,20 @@ bool use_abs_form(const Tun& tun, int dtype, int H, int D) {
   return tun.path == LT_PATH_FUSED_ABS && dtype == LT_DTYPE_E4M3 && scan_mma_supported(dtype, H, D);
 }
 
-// Small problems: score everything into a dense buffer and select from it (two launches) instead of sample, statistics,
-// gated scan, final select and fallback.  Both give the same bits.  The dense form saves four launches and the
-// gate's work per key, and pays 4 bytes of traffic per pair and a select over whole rows.  Measured on one B200, dense
-// against sampled, us per call, topk 2048.  Rows of up to kDenseKeys keys are selected by one CTA each: 1 row x 8 K keys
-// 20 / 41, 256 x 16 K 72 / 107, 4096 x 4 K (bf16, first chunk) 211 / 351, 4096 x 16 K 766 / 937; many rows with a small topk
-// are the exception, their candidate lists are short (topk 64, 4096 x 16 K 864 / 802, 4096 x 8 K 418 / 456).  Longer rows
-// are shared by clusters of CTAs, which pays up to about kDensePairs pairs and kDenseMaxKeys keys: 1 x 128 K 29 / 42,
-// 16 x 128 K 54 / 65, 4 x 512 K 52 / 63, 64 x 64 K 83 / 89, but 1 x 1 M 71 / 66, 16 x 512 K 137 / 119, 64 x 256 K 231 / 216.
-// The k-NN variant follows the same lines (64 x 16 K x 128: 24 / 65, 16 x 200 K x 768: 94 / 102, 4 x 1 M x 128: 111 / 91).
+// Small problems: score everything into a dense buffer and select from it (three launches) instead of sample, statistics,
+// gated scan, final select and fallback.  Both give the same bits.  The dense form saves four launches and the gate's work
+// per key, and pays 4 bytes of traffic per pair and a select over whole rows.  Measured on one B200, dense against sampled,
+// us per call, topk 2048 unless given.  Rows of up to kDenseKeys keys are selected by one CTA each: 256 x 16 K 63 / 85,
+// 4096 x 4 K (bf16, first chunk) 194 / 333, 4096 x 16 K 744 / 881, topk 64 4096 x 8 K 342 / 377, 1024 x 16 K 197 / 214; many
+// rows of 16 K with a small topk are the exception, their candidate lists are short.  Longer rows are shared by clusters of
+// CTAs.  With rows of up to kDenseMidKeys that pays up to kDensePairs pairs: 64 x 32 K 40 / 50, 40 x 100 K 72 / 74, 64 x 64
+// K 71 / 75 (bf16, topk 64 65 / 70), 32 x 128 K topk 64 59 / 70, 16 x 128 K 49 / 49.  Still longer rows end the call with a
+// longer select, and the line is at half as many pairs: 1 x 128 K 24 / 33 (topk 8192 36 / 39), 4 x 256 K 33 / 37, 7 x 300 K
+// bf16 49 / 54, 10 x 200 K 51 / 59, 4 x 512 K 47 / 48; beyond it 11 x 200 K 59 / 59, 16 x 200 K 64 / 59, 16 x 256 K 74 / 68,
+// 8 x 512 K 79 / 66.  The k-NN variant takes the same lines (64 x 32 K x 128 22 / 36, 64 x 64 K x 768 44 / 56, 8 x 200 K x 768
+// 80 / 88, 4 x 256 K x 128 39 / 38; beyond them 16 x 256 K x 128 55 / 38).
 constexpr int kDenseKeys = 16384;
+constexpr int kDenseMidKeys = 128 << 10;
 constexpr int kDenseMaxKeys = 512 << 10;
 constexpr long long kDensePairs = 4ll << 20;
 bool use_direct(const Tun& tun, int T, int N, int topk, bool paged) {
@@ -116,7 +120,9 @@ bool use_direct(const Tun& tun, int T, int N, int topk, bool paged) {
   // equal those over dense keys and which callers compare
   if (paged && T > kRowsPerBlock) return false;
   if (N <= kDenseKeys / 2 || (N <= kDenseKeys && topk >= 512)) return true;
-  return (N <= kDenseKeys && T <= 1024) || (N <= kDenseMaxKeys && static_cast<long long>(T) * N <= kDensePairs);
+  const long long pairs = static_cast<long long>(T) * N;
+  return (N <= kDenseKeys && T <= 1024) || (N <= kDenseMidKeys && pairs <= kDensePairs) ||
+         (N <= kDenseMaxKeys && pairs <= kDensePairs / 2);
 }
 
 // ---- workspace layout ------------------------------------------------------------------------

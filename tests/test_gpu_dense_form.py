@@ -27,7 +27,8 @@ def _check(inp, oracle_rows=()):
 
 @pytest.mark.parametrize("recipe,dtype", [("iid", "bf16"), ("ar1", "e4m3")])
 @pytest.mark.parametrize("T,N,topk", [(1, 16384, 2048), (1, 16385, 2047), (3, 16389, 1), (2, 32769, 500), (4, 65537, 8191),
-                                      (1, 131073, 2048), (5, 131077, 3000), (17, 200001, 64), (300, 4097, 2048), (9, 127, 127)])
+                                      (1, 131073, 2048), (5, 131077, 3000), (10, 200001, 64), (31, 131071, 64),
+                                      (300, 4097, 2048), (9, 127, 127)])
 def test_sizes(recipe, dtype, T, N, topk):
     inp = make_inputs(recipe, dtype, T=T, N=N, H=64, D=128, topk=topk, seed=N)
     _check(inp, oracle_rows=(0, T - 1))
