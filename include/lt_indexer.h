@@ -116,7 +116,8 @@ typedef struct lt_tunables {
 } lt_tunables;
 
 /* lt_tunables.debug_flags (no counterpart in the paper; used by the library's own tests) */
-#define LT_DEBUG_SKIP_ONE_KTILE 1 /* the fused scan's first CTA never loads its first key tile: with a short
+#define LT_DEBUG_SKIP_ONE_KTILE 1 /* the first CTA of the fused scan (of the scoring scan where LT_PATH_AUTO takes
+                                     the dense form) never loads its first key tile: with a short
                                      wait_limit_us this exercises the bounded-wait timeout path without
                                      any fault (the call returns, status has LT_STATUS_TIMEOUT)        */
 

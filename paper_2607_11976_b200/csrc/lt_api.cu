@@ -115,7 +115,7 @@ constexpr int kDenseMaxKeys = 512 << 10;
 constexpr long long kDensePairs = 4ll << 20;
 bool use_direct(const Tun& tun, int T, int N, int topk, bool paged) {
   // an explicit path or a tunable of the sampled form asks for that form
-  if (tun.path != LT_PATH_AUTO || tun.sample_mult_given || tun.cap_mult_given || tun.sample_rank != 0 || tun.debug_flags != 0) return false;
+  if (tun.path != LT_PATH_AUTO || tun.sample_mult_given || tun.cap_mult_given || tun.sample_rank != 0) return false;
   // over a paged cache only up to one query block: larger chunks report the survivor counts of the sampled form, which
   // equal those over dense keys and which callers compare
   if (paged && T > kRowsPerBlock) return false;
@@ -431,6 +431,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     p.page_table = page_table;
     p.n_pages = n_pages;
     p.pool_pages = pool_rows / kPageKeys;
+    p.debug_flags = tun.debug_flags;
     p.ctl = ctl;
     LT_LAUNCH(launch_scan_mma(dtype, kModeDump, q, T, k, key_rows, key_pitch, p, grid, stream));
     mark_phase(3, stream);

@@ -92,7 +92,7 @@ struct ScanParams {
   int n_pages;
   long long pool_pages;    // pages of the pool behind page_table (bounds checks of the debug build)
   unsigned int wait_limit_us;  // bound of every device-side wait (0 is replaced by the default at launch)
-  int debug_flags;         // LT_DEBUG_* test hooks (filter mode only)
+  int debug_flags;         // LT_DEBUG_* test hooks
   // alternative fp8 scan only: the linear part of Eq. 1 prepared by launch_lin_terms
   const void* lin_q;       // [T][kLinTerms][128] e4m3 codes
   const float* lin_scale;  // [T][kLinScaleStride], the first kLinTerms entries of a row are used

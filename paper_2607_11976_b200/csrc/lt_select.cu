@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 #include <cuda_runtime.h>
+#include <float.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -552,7 +553,7 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
 }
 
 // ---------------------------------------------------------------------------------------------
-// The kk (< vis) best of row[0 .. vis), by one CTA: 4-pass MSB radix select for the kk-th score, then everything above it and
+// The kk (<= vis) best of row[0 .. vis), by one CTA, whatever bits the row holds: 4-pass MSB radix select for the kk-th score, then everything above it and
 // the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.
 // ---------------------------------------------------------------------------------------------
 template <int kThreads>
@@ -755,8 +756,8 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
 // bins over the row's range, as in the distribution sort but kClBins of them: the CTAs' histograms are merged through
 // distributed shared memory, the CTAs agree on the bin that holds the kk-th key, and every key up to it goes to the
 // first CTA's list, which is then sorted there.  A bin that holds more keys than the list takes is split again over
-// its own range (a few outliers stretch the range); what still does not fit (mass ties) is left to the first CTA's
-// radix select over the whole row.  Bound by latencies (four cluster barriers, a sort by one CTA) up to 128 K keys, by
+// its own range (a few outliers stretch the range); what still does not fit (mass ties), and a row with infinite or NaN scores
+// or with whatever a scan that gave up left behind, goes to the first CTA's radix select over the whole row, which is total.  Bound by latencies (four cluster barriers, a sort by one CTA) up to 128 K keys, by
 // instructions above: a key costs about 15, on floats throughout (ordered bit patterns would double that).
 // ---------------------------------------------------------------------------------------------
 constexpr int kClThreads = 512;
@@ -886,6 +887,12 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
         vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, d));
       }
     }
+    // Infinite scores (sums that overflowed) and ranges too wide for a float have no bins: the first CTA ranks the row's bit
+    // patterns instead.  Every CTA has the same range, so all of them leave together.
+    if (!(fabsf(vmax - vmin) <= FLT_MAX)) {
+      total = cap + 1u;
+      break;
+    }
     // bin of a score in the range, best scores first; monotone because every step rounds monotonically
     // (finite, so that the best score's 0 * scale is 0)
     scale = vmax > vmin ? fminf(static_cast<float>(kClBins) / (vmax - vmin), 3e38f) : 0.f;
@@ -922,7 +929,14 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
       const unsigned int need = static_cast<unsigned int>(kk) - above;
       const unsigned int sum = lane < static_cast<int>(n_cta) ? *cl.map_shared_rank(&s_seg_sum, lane) : 0u;
       const unsigned int incl = warp_inclusive_sum(sum, lane);
-      const int owner = __ffs(__ballot_sync(0xffffffffu, incl >= need && incl - sum < need)) - 1;
+      const unsigned int crossing = __ballot_sync(0xffffffffu, incl >= need && incl - sum < need);
+      // NaN scores are counted nowhere: as above.  (crossing is zero only where keys are missing from the counts; it is tested
+      // because the address below is made from it.)
+      if ((level == 0 && __shfl_sync(0xffffffffu, incl, 31) != static_cast<unsigned int>(vis)) || crossing == 0u) {
+        total = cap + 1u;
+        break;
+      }
+      const int owner = __ffs(crossing) - 1;
       const unsigned int before = __shfl_sync(0xffffffffu, incl - sum, owner);
       const uint2* segc = reinterpret_cast<const uint2*>(cl.map_shared_rank(s_seg, owner));
       const uint2 c = 2 * tid < seg ? segc[tid] : make_uint2(0u, 0u);  // two bins per thread: at most 1024

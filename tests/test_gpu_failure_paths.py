@@ -43,6 +43,19 @@ def test_skipped_key_tile_times_out_and_the_next_call_is_clean(name):
     assert_matches_oracle(inp, idx, score, list(range(inp.T)))
 
 
+@pytest.mark.parametrize("name,T,N", [("fp8_ar1", 3, 40000), ("dsa_bf16", 1, 20011), ("fp8_ar1", 16, 9000)])
+def test_dense_form_times_out_and_the_next_call_is_clean(name, T, N):
+    """The same in the scoring scan of the dense form, whose select then ranks rows that were never written: status
+    LT_STATUS_TIMEOUT, no index outside the keys, and a clean call right after it."""
+    inp = make_config(name, T=T, N=N, topk=300)
+    idx, _, status = run_topk(inp, lt.Tunables(wait_limit_us=1000, debug_flags=lt.LT_DEBUG_SKIP_ONE_KTILE))
+    assert status[0] & lt.LT_STATUS_TIMEOUT, "the skipped tile should have made a wait run out"
+    assert idx.min() >= -1 and idx.max() < N
+    idx, score, status = run_topk(inp)
+    assert status[0] == 0 and status[3] == 0
+    assert_matches_oracle(inp, idx, score, [0, T - 1])
+
+
 def test_wait_limit_is_not_a_result_tunable():
     inp = make_config("fp8_ar1", T=24, N=5000, topk=128)
     a = run_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED))
