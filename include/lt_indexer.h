@@ -160,7 +160,10 @@ int lt_indexer_topk_strided(int dtype, const void* q, const float* w, const void
                             int32_t* out_idx, float* out_score,
                             void* workspace, size_t workspace_bytes, const lt_tunables* tunables, void* stream);
 
-/* Bytes of workspace lt_indexer_topk_ex needs for this problem (0 on invalid arguments). */
+/*
+ * Bytes of workspace lt_indexer_topk_ex needs for this problem (0 on invalid arguments).  The size for default
+ * tunables serves the problem by every path of LT_PATH_AUTO, LT_PATH_FUSED and LT_PATH_GENERIC.
+ */
 size_t lt_indexer_topk_workspace_bytes(int dtype, int T, int N, int H, int D, int topk,
                                        const lt_tunables* tunables);
 

@@ -260,6 +260,19 @@ Layout make_layout(bool fused, int T, int N, int topk, int causal_offset, const 
   return L;
 }
 
+// Bytes a caller sets aside for a problem: the larger of what LT_PATH_AUTO's two forms take, so that a workspace sized once
+// serves the problem by whatever path and with whatever default-sized tunables it is called, and a smaller problem as well.
+// A call itself asks only for what the form it runs takes.
+size_t workspace_for(bool fused, int T, int N, int topk, const Tun& tun, int n_given, int key_row_bytes, bool gather_default, bool abs_form) {
+  // the sample can never be larger with a different causal_offset than with the whole context visible
+  const size_t own = make_layout(fused, T, N, topk, N - 1, tun, n_given, key_row_bytes, gather_default, abs_form).total;
+  if (!fused || tun.path != LT_PATH_AUTO) return own;
+  Tun sampled = tun;
+  sampled.path = LT_PATH_FUSED;
+  const size_t other = make_layout(true, T, N, topk, N - 1, sampled, n_given, key_row_bytes, gather_default, abs_form).total;
+  return own > other ? own : other;
+}
+
 int sm_count() {
   static int cached[64] = {0};
   int dev = 0;
@@ -665,8 +678,7 @@ size_t lt_indexer_topk_workspace_bytes(int dtype, int T, int N, int H, int D, in
       topk <= 0 || topk > N || topk > LT_MAX_TOPK)
     return 0;
   const Tun tun = resolve_tunables(tunables);
-  // the sample can never be larger with a different causal_offset than with the whole context visible
-  return make_layout(use_fused(tun, dtype, H, D), T, N, topk, N - 1, tun, 0, 0, false, use_abs_form(tun, dtype, H, D)).total;
+  return workspace_for(use_fused(tun, dtype, H, D), T, N, topk, tun, 0, 0, false, use_abs_form(tun, dtype, H, D));
 }
 
 int lt_indexer_topk_sampled(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N, int H,
@@ -684,8 +696,8 @@ size_t lt_indexer_topk_sampled_workspace_bytes(int dtype, int T, int N, int H, i
       topk <= 0 || topk > N || topk > LT_MAX_TOPK || n_sample <= 0 || n_sample > LT_MAX_SAMPLE)
     return 0;
   const Tun tun = resolve_tunables(tunables);
-  return make_layout(use_fused(tun, dtype, H, D), T, N, topk, N - 1, tun, n_sample,
-                     static_cast<int>(static_cast<size_t>(D) * elem_bytes(dtype)), false, use_abs_form(tun, dtype, H, D)).total;
+  return workspace_for(use_fused(tun, dtype, H, D), T, N, topk, tun, n_sample,
+                       static_cast<int>(static_cast<size_t>(D) * elem_bytes(dtype)), false, use_abs_form(tun, dtype, H, D));
 }
 
 int lt_indexer_topk_paged(int dtype, const void* q, const float* w, const void* k_pool, const float* k_scale_pool,
@@ -705,8 +717,8 @@ size_t lt_indexer_topk_paged_workspace_bytes(int dtype, int T, int N, int H, int
     return 0;
   const Tun tun = resolve_tunables(tunables);
   if (!use_fused(tun, dtype, H, D)) return 0;
-  return make_layout(true, T, N, topk, N - 1, tun, 0, static_cast<int>(static_cast<size_t>(D) * elem_bytes(dtype)), true,
-                     use_abs_form(tun, dtype, H, D)).total;
+  return workspace_for(true, T, N, topk, tun, 0, static_cast<int>(static_cast<size_t>(D) * elem_bytes(dtype)), true,
+                       use_abs_form(tun, dtype, H, D));
 }
 
 size_t lt_topk_frequent_workspace_bytes(int N) {
@@ -877,7 +889,7 @@ int knn_seg_tiles(const Tun& tun, int n_keys, int grid) {
 
 size_t lt_knn_topk_workspace_bytes(int dtype, int T, int N, int D, int topk, const lt_tunables* tunables) {
   if (dtype != LT_DTYPE_BF16 || T <= 0 || N <= 0 || !scan_knn_supported(D) || topk <= 0 || topk > N || topk > LT_MAX_TOPK) return 0;
-  return make_layout(true, T, N, topk, N - 1, resolve_tunables(tunables)).total;
+  return workspace_for(true, T, N, topk, resolve_tunables(tunables), 0, 0, false, false);
 }
 
 int lt_knn_scores(int dtype, const void* q, const void* x, int T, int N, int D, int row_begin, int row_end, float* out_scores,

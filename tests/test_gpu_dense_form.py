@@ -72,3 +72,17 @@ def test_paged_keys_take_the_dense_form_too():
                              inp.causal_offset, idx, score, ws)
     assert lt.lt_read_status(ws)[0] == 0
     assert np.array_equal(idx.cpu().numpy(), want_idx) and np.array_equal(score.cpu().numpy().view(np.uint32), want_score.view(np.uint32))
+
+
+def test_a_workspace_of_the_default_size_serves_every_path():
+    inp = make_inputs("ar1", "e4m3", T=64, N=16384, H=64, D=128, topk=256, seed=3)
+    want_idx, want_score, _ = run_topk(inp)
+    q, w, k, ks = lt.to_device(inp)
+    ws = lt.alloc_workspace("e4m3", 64, 16384, 64, 128, 256)
+    for topk, path in ((256, lt.LT_PATH_FUSED), (256, lt.LT_PATH_AUTO), (100, lt.LT_PATH_FUSED)):
+        idx = torch.empty((64, topk), dtype=torch.int32, device="cuda")
+        score = torch.empty((64, topk), device="cuda")
+        lt.lt_indexer_topk_ex("e4m3", q, w, k, ks, topk, inp.causal_offset, idx, score, ws, lt.Tunables(path=path))
+        assert lt.lt_read_status(ws)[0] == 0
+        assert np.array_equal(idx.cpu().numpy(), want_idx[:, :topk])
+        assert np.array_equal(score.cpu().numpy().view(np.uint32), want_score[:, :topk].view(np.uint32))
