@@ -169,6 +169,7 @@ __global__ void __launch_bounds__(kStatsMaxThreads) sample_stats_kernel(const fl
     for (int j = 0; j < kStatsBatch; ++j) v[j] = row[min(base + j * n_threads, n_sample - 1)];
 #pragma unroll
     for (int j = 0; j < kStatsBatch; ++j) {
+      if (v[j] != v[j]) continue;  // a NaN (sums that overflowed) would leave the row without bins; the gate lets none pass
       const unsigned int k = score_to_key(__float_as_uint(v[j]));
       mn = min(mn, k);
       mx = max(mx, k);

@@ -78,3 +78,18 @@ def test_dense_form(kind, N, topk):
     dumped = dump_scores(inp, 0, inp.T)
     assert not np.isnan(dumped).any()
     assert_own_scores_rule(inp, idx, score, dumped, range(inp.T))
+
+
+@pytest.mark.parametrize("dtype,N", [("bf16", 70000), ("bf16", 30000)])
+def test_nan_in_the_sample_costs_the_row_nothing(dtype, N):
+    """Key 0 is in every sample.  Its score is NaN, which the gate never passes: the row is selected from the other keys, by the
+    sampled form's own means and not by its fallback."""
+    inp = make_inputs("iid", dtype, T=20, N=N, H=64, D=128, topk=100, seed=5)
+    inp.w[:, ::2], inp.w[:, 1::2] = np.abs(inp.w[:, ::2]), -np.abs(inp.w[:, 1::2])
+    inp.q[:, 0], inp.q[:, 1] = inp.q[:, 0] & 0x7FFF, inp.q[:, 0] & 0x7FFF  # a head of each sign that sees key 0 overflow
+    inp.k[0] = np.float32(3e38).view(np.uint32) >> 16
+    idx, score, status = run_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED))
+    assert status[0] == 0 and status[1] == 0  # no row took the fallback
+    dumped = dump_scores(inp, 0, inp.T)
+    assert np.isnan(dumped[:, 0]).all() and not np.isnan(dumped[:, 1:]).any()
+    assert_own_scores_rule(inp, idx, score, dumped, range(inp.T))  # (the host's ranking puts NaN last)
