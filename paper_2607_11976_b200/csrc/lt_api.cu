@@ -458,6 +458,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     sp.causal_offset = causal_offset;
     sp.out_idx = out_idx;
     sp.out_score = out_score;
+    sp.nan_last = 1;
     sp.ctl = ctl;
     LT_LAUNCH(launch_select_dense(sp, stream));
     mark_phase(4, stream);
@@ -957,6 +958,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     sp.causal_offset = N;
     sp.out_idx = out_idx;
     sp.out_score = out_score;
+    sp.nan_last = 1;
     sp.ctl = ctl;
     LT_LAUNCH(launch_select_dense(sp, stream));
     mark_phase(4, stream);

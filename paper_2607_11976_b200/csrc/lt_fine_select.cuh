@@ -27,6 +27,7 @@ namespace lt {
 //   load(i)   score bits and index of the i-th key, i < n; called for i >= kFineBatch * kThreads only, several times
 //   c         the first kFineBatch * kThreads keys, key j * kThreads + tid in c[j] (anything past n)
 //   keys      key_cap 64-bit slots, bins: kFineBins counters (both shared memory)
+//   leave_nan rows with a NaN among their scores are left to the caller too
 // ---------------------------------------------------------------------------------------------
 constexpr int kFineBins = 4096;
 constexpr int kFineBatch = 8;
@@ -34,7 +35,7 @@ constexpr int kFineBatch = 8;
 template <int kThreads, class Load>
 __device__ __forceinline__ bool fine_select_sort(const Load& load, uint2 (&c)[kFineBatch], unsigned int n, int kk, int topk,
                                                  uint64_t* keys, unsigned int key_cap, unsigned int* bins, int32_t* out_idx,
-                                                 float* out_score, int n_keys, Control* ctl) {
+                                                 float* out_score, int n_keys, Control* ctl, bool leave_nan = false) {
   constexpr int kWarps = kThreads / 32;
   constexpr int kBinsPerThread = kFineBins / kThreads;
   static_assert(kWarps <= 32 && kBinsPerThread % 4 == 0, "one warp combines the warps' results; bins are swept in 16-byte pieces");
@@ -80,6 +81,10 @@ __device__ __forceinline__ bool fine_select_sort(const Load& load, uint2 (&c)[kF
     if (attempt == 0) {
       kmin = __reduce_min_sync(0xffffffffu, lane < kWarps ? s_min[lane] : 0xffffffffu);
       kmax = __reduce_max_sync(0xffffffffu, lane < kWarps ? s_max[lane] : 0u);
+      if (leave_nan && (kmax > score_to_key(0x7f800000u) || kmin < score_to_key(0xff800000u))) {  // beyond an infinity
+        __syncthreads();
+        return false;
+      }
     }
     const float fmax = __uint_as_float(key_to_score_bits(kmax)), fmin = __uint_as_float(key_to_score_bits(kmin));
     const float fscale = static_cast<float>(kFineBins) / (fmax - fmin);

@@ -200,6 +200,9 @@ struct SelectRowsParams {
   int rows_per_block;
   const unsigned char* row_flag;
   Control* ctl;
+  // NaN scores rank as their bit patterns do, above +inf.  nan_last != 0: they are selected only where a row has too few others,
+  // which is what becomes of them in the sampled form (its gate lets none pass; a row that is then short of keys is redone)
+  int nan_last;
   unsigned int sel_slots;  // set by the launch: a power of two >= topk
   int slice_keys;          // set by the launch of the cluster form
 };

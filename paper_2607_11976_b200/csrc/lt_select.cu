@@ -558,12 +558,32 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
 // the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.
 // ---------------------------------------------------------------------------------------------
 template <int kThreads>
-__device__ __forceinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel) {
+__device__ __forceinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel, bool nan_last) {
   constexpr int kWarps = kThreads / 32;
   __shared__ unsigned int hist[256];
   __shared__ unsigned int s_prefix, s_remaining, s_gt;
   __shared__ unsigned int warp_cnt[kWarps];
+  __shared__ int s_nan;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  // NaN scores below everything, -inf included, where the row has enough others.  They are told by their bits: a test of the float
+  // (isnan) next to the selection of its bits came out of nvcc 12.9 as if drop_nan were always set.
+  constexpr unsigned int kLowest = 0x007fffffu, kRange = 0xff800000u - kLowest;  // ordered bit patterns of -inf .. +inf
+  bool drop_nan = false;
+  if (nan_last) {
+    if (tid == 0) s_nan = 0;
+    __syncthreads();
+    int n = 0;
+    for (int i = tid; i < vis; i += kThreads) n += score_to_key(__float_as_uint(row[i])) - kLowest > kRange ? 1 : 0;
+    n = __reduce_add_sync(0xffffffffu, n);
+    if (lane == 0 && n > 0) atomicAdd(&s_nan, n);
+    __syncthreads();
+    drop_nan = vis - s_nan >= kk;
+  }
+  const unsigned int key_lo = drop_nan ? kLowest : 0u, key_range = drop_nan ? kRange : 0xffffffffu;
+  auto key_of = [&](float v) {
+    const unsigned int k = score_to_key(__float_as_uint(v));
+    return k - key_lo > key_range ? 0u : k;
+  };
   if (tid == 0) {
     s_prefix = 0;
     s_remaining = static_cast<unsigned int>(kk);
@@ -590,7 +610,7 @@ __device__ __forceinline__ void radix_select_row(const float* row, int vis, int 
         const int i = base + j * kThreads + tid;
         unsigned int digit = 0x100u;  // "not a candidate" (out of range or another prefix)
         if (i < vis) {
-          const unsigned int key = score_to_key(__float_as_uint(v[j]));
+          const unsigned int key = key_of(v[j]);
           if ((key & mask) == prefix) digit = (key >> shift) & 255u;
         }
         if (digit < 0x100u) {
@@ -644,7 +664,7 @@ __device__ __forceinline__ void radix_select_row(const float* row, int vis, int 
 #pragma unroll
     for (int j = 0; j < kSelBatch; ++j) {
       const int i = base + j * 32 + lane;
-      const bool eq = i < hi && score_to_key(__float_as_uint(v[j])) == kth;
+      const bool eq = i < hi && key_of(v[j]) == kth;
       my_eq += __popc(__ballot_sync(0xffffffffu, eq));
     }
   }
@@ -665,7 +685,7 @@ __device__ __forceinline__ void radix_select_row(const float* row, int vis, int 
     unsigned int key = 0;
     bool gt = false, eq = false;
     if (i < hi) {
-      key = score_to_key(__float_as_uint(v[j]));
+      key = key_of(v[j]);
       gt = key > kth;
       eq = key == kth;
     }
@@ -728,7 +748,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
     }
     if (fine_select_sort<kThreads>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
                                       static_cast<unsigned int>(vis), kk, p.topk, sel, 2u * p.sel_slots, bins, out_idx, out_score,
-                                      p.N, p.ctl))
+                                      p.N, p.ctl, p.nan_last != 0 && vis > p.topk))
       return;
   }
   if (vis <= p.topk) {
@@ -739,7 +759,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
     return;
   }
 
-  radix_select_row<kThreads>(row, vis, kk, sel);
+  radix_select_row<kThreads>(row, vis, kk, sel, p.nan_last != 0);
   __syncthreads();
   auto winner = [&](unsigned int i) { return make_uint2(key_to_score_bits(static_cast<unsigned int>(sel[i] >> 32)), static_cast<unsigned int>(key_index(sel[i]))); };
 #pragma unroll
@@ -1016,7 +1036,7 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
     if (fine_select_sort<kClThreads>(entry, first, total, kk, p.topk, sorted, cap, bins, out_idx, out_score, p.N, p.ctl)) return;
     if (total > static_cast<unsigned int>(kk)) keep_top_keys(list, static_cast<int>(total), kk, bins, &s_count);
   } else {
-    radix_select_row<kClThreads>(row, vis, kk, list);
+    radix_select_row<kClThreads>(row, vis, kk, list, p.nan_last != 0);
   }
   __syncthreads();
   // room for next_pow2(kk) keys: the list, the bins and the slice lie one behind the other

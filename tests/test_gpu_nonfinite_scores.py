@@ -93,3 +93,28 @@ def test_nan_in_the_sample_costs_the_row_nothing(dtype, N):
     dumped = dump_scores(inp, 0, inp.T)
     assert np.isnan(dumped[:, 0]).all() and not np.isnan(dumped[:, 1:]).any()
     assert_own_scores_rule(inp, idx, score, dumped, range(inp.T))  # (the host's ranking puts NaN last)
+
+
+@pytest.mark.parametrize("N,topk", [(9000, 500), (20011, 2000), (65540, 64), (140000, 2048), (5000, 5000), (30000, 8192)])
+@pytest.mark.parametrize("nan", ["some", "most"])
+def test_nan_scores_rank_alike_in_both_forms(nan, N, topk):
+    """The gate of the sampled form lets no NaN pass, and a row that is then short of keys is redone by the order of the bit patterns:
+    the dense form of the same problem has to put NaN scores last where there are enough others, first where there are not."""
+    inp = make_inputs("iid", "bf16", T=3, N=N, H=64, D=128, topk=topk, seed=5)
+    inp.w[:, ::2], inp.w[:, 1::2] = np.abs(inp.w[:, ::2]), -np.abs(inp.w[:, 1::2])
+    inp.q[:, 0], inp.q[:, 1] = inp.q[:, 0] & 0x7FFF, inp.q[:, 0] & 0x7FFF  # a head of each sign that sees the large keys overflow
+    large = np.random.default_rng(N).permutation(N)[:20 if nan == "some" else N - topk // 2]
+    inp.k[large] = np.float32(3e38).view(np.uint32) >> 16
+    dumped = dump_scores(inp, 0, inp.T)
+    idx, score, status = run_topk(inp)
+    assert status[3] == 0  # the dense form ran
+    f_idx, f_score, _ = run_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED))
+    assert np.array_equal(idx, f_idx) and np.array_equal(score.view(np.uint32), f_score.view(np.uint32))
+    for t in range(inp.T):
+        row = dumped[t][:inp.visible(t)]
+        enough = np.count_nonzero(~np.isnan(row)) >= min(topk, row.size)
+        if nan == "some" and topk < N - 100:
+            assert enough and np.isnan(row).any()
+        want_idx, want_bits = rank_bits(np.where(np.isnan(row), -np.inf, row) if enough else row, topk)
+        n = want_idx.size
+        assert np.array_equal(idx[t][:n], want_idx) and np.array_equal(score[t][:n].view(np.uint32), want_bits)
