@@ -107,13 +107,23 @@ bool use_abs_form(const Tun& tun, int dtype, int H, int D) {
 // K 71 / 75 (bf16, topk 64 65 / 70), 32 x 128 K topk 64 59 / 70, 16 x 128 K 49 / 49.  Still longer rows end the call with a
 // longer select, and the line is at half as many pairs: 1 x 128 K 24 / 33 (topk 8192 36 / 39), 4 x 256 K 33 / 37, 7 x 300 K
 // bf16 49 / 54, 10 x 200 K 51 / 59, 4 x 512 K 47 / 48; beyond it 11 x 200 K 59 / 59, 16 x 200 K 64 / 59, 16 x 256 K 74 / 68,
-// 8 x 512 K 79 / 66.  The k-NN variant takes the same lines (64 x 32 K x 128 22 / 36, 64 x 64 K x 768 44 / 56, 8 x 200 K x 768
-// 80 / 88, 4 x 256 K x 128 39 / 38; beyond them 16 x 256 K x 128 55 / 38).
+// 8 x 512 K 79 / 66.
+// The k-NN variant takes the same lines for long vectors (D = 768: 64 x 64 K topk 100 0.79 of the sampled form's time, 32 x 128 K
+// 0.92, 8 x 256 K 0.95, 4 x 512 K 0.99; D = 256: 0.82, 1.01, 1.02, 1.01).  Short ones are scanned so fast that the second pass
+// over the scores shows earlier: with D below kDenseShortDim rows of more than kDenseShortKeys keys are dense only up to
+// kDenseShortPairs pairs, and rows of more than kDenseMidKeys never (D = 128, topk 10 / 1024: 64 x 50 K 0.90 / 0.53, 64 x 64 K
+// 0.95 / 0.54, 8 x 100 K 0.93 / 0.89, 8 x 128 K 0.99 / 0.96; beyond the line 16 x 100 K 1.02 / 0.88, 32 x 128 K 1.14 / 0.80, 1 x
+// 200 K 1.03 / 1.01, 8 x 256 K 1.21 / 1.16, 4 x 512 K 1.20 / 1.18; D = 64: 0.90 / 0.53, 0.94 / 0.54, 0.96 / 0.90, 1.04 / 0.99;
+// 1.07 / 0.90, 1.17 / 0.82, 1.12 / 1.09, 1.35 / 1.27, 1.44 / 1.34).
 constexpr int kDenseKeys = 16384;
 constexpr int kDenseMidKeys = 128 << 10;
 constexpr int kDenseMaxKeys = 512 << 10;
 constexpr long long kDensePairs = 4ll << 20;
-bool use_direct(const Tun& tun, int T, int N, int topk, bool paged) {
+constexpr int kDenseShortDim = 256;
+constexpr int kDenseShortKeys = 64 << 10;
+constexpr long long kDenseShortPairs = 1ll << 20;
+// knn_dim: the vectors' dimension of the k-NN variant, 0 for the indexer
+bool use_direct(const Tun& tun, int T, int N, int topk, bool paged, int knn_dim) {
   // an explicit path or a tunable of the sampled form asks for that form
   if (tun.path != LT_PATH_AUTO || tun.sample_mult_given || tun.cap_mult_given || tun.sample_rank != 0) return false;
   // over a paged cache only up to one query block: larger chunks report the survivor counts of the sampled form, which
@@ -121,6 +131,7 @@ bool use_direct(const Tun& tun, int T, int N, int topk, bool paged) {
   if (paged && T > kRowsPerBlock) return false;
   if (N <= kDenseKeys / 2 || (N <= kDenseKeys && topk >= 512)) return true;
   const long long pairs = static_cast<long long>(T) * N;
+  if (knn_dim != 0 && knn_dim < kDenseShortDim && N > kDenseShortKeys) return N <= kDenseMidKeys && pairs <= kDenseShortPairs;
   return (N <= kDenseKeys && T <= 1024) || (N <= kDenseMidKeys && pairs <= kDensePairs) ||
          (N <= kDenseMaxKeys && pairs <= kDensePairs / 2);
 }
@@ -142,7 +153,7 @@ struct Layout {
 // gathered into a dense buffer of the workspace (key_row_bytes each) and scored from there.
 // gather_default: the default strided sample is gathered too (paged key cache: a strided view cannot reach it).
 Layout make_layout(bool fused, int T, int N, int topk, int causal_offset, const Tun& tun, int n_given = 0,
-                   int key_row_bytes = 0, bool gather_default = false, bool abs_form = false) {
+                   int key_row_bytes = 0, bool gather_default = false, bool abs_form = false, int knn_dim = 0) {
   Layout L{};
   L.fused = fused;
   L.abs_form = fused && abs_form;
@@ -159,7 +170,7 @@ Layout make_layout(bool fused, int T, int N, int topk, int causal_offset, const 
     L.total = off;
     return L;
   }
-  if (n_given == 0 && !L.abs_form && use_direct(tun, T, N, topk, gather_default)) {
+  if (n_given == 0 && !L.abs_form && use_direct(tun, T, N, topk, gather_default, knn_dim)) {
     L.direct = true;
     L.direct_ld = (N + 31) / 32 * 32;
     L.zero_end = off;
@@ -924,7 +935,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
   if (rc != LT_OK) return rc;
   if (out_idx == nullptr || topk <= 0 || topk > N || topk > LT_MAX_TOPK) return LT_ERR_INVALID_ARG;
   const Tun tun = resolve_tunables(tunables);
-  const Layout L = make_layout(true, T, N, topk, N - 1, tun);  // every query sees the whole corpus
+  const Layout L = make_layout(true, T, N, topk, N - 1, tun, 0, 0, false, false, D);  // every query sees the whole corpus
   if (workspace == nullptr || (reinterpret_cast<uintptr_t>(workspace) & (kAlign - 1)) != 0 || workspace_bytes < L.total)
     return LT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);

@@ -78,6 +78,20 @@ def test_topk_matches_oracle_and_own_scores(T, N, D, topk):
         assert np.array_equal(score[t].view(np.uint32), want_val.view(np.uint32))
 
 
+@pytest.mark.parametrize("T,N,D,dense", [(64, 65536, 64, True), (16, 65537, 64, False), (15, 65537, 192, True), (8, 131072, 128, True),
+                                         (9, 131072, 128, False), (1, 131073, 192, False), (1, 131073, 256, True), (32, 131072, 256, True)])
+def test_dense_form_by_the_length_of_the_vectors(T, N, D, dense):
+    """Points on both sides of the line between the two forms, which lies elsewhere for short vectors: the one expected runs (the dense
+    form filters nothing), and both give the same bits."""
+    inp = make_knn(T=T, N=N, D=D, topk=50)
+    idx, score, st = gpu_topk(inp)
+    assert st[0] == 0 and (st[3] == 0) == dense
+    f_idx, f_score, st = gpu_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED))
+    assert st[0] == 0 and st[3] > 0
+    assert np.array_equal(idx, f_idx) and np.array_equal(score.view(np.uint32), f_score.view(np.uint32))
+    check(inp, idx, score, [0, T - 1])
+
+
 def test_fallback_and_tunables_keep_every_bit():
     inp = make_knn(T=20, N=30000, D=256, topk=256)
     base_idx, base_score, st0 = gpu_topk(inp)
