@@ -555,10 +555,12 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
 
 // ---------------------------------------------------------------------------------------------
 // The kk (<= vis) best of row[0 .. vis), by one CTA, whatever bits the row holds: 4-pass MSB radix select for the kk-th score, then everything above it and
-// the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.
+// the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.  Out of line: it is the rare way of
+// kernels that live for a few microseconds, whose usual way is shorter without it (1 x 32 K dense, topk 2048, 20.9 -> 20.4 us
+// together with the tied slices below).
 // ---------------------------------------------------------------------------------------------
 template <int kThreads>
-__device__ __forceinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel, bool nan_last) {
+__device__ __noinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel, bool nan_last) {
   constexpr int kWarps = kThreads / 32;
   __shared__ unsigned int hist[256];
   __shared__ unsigned int s_prefix, s_remaining, s_gt;
@@ -777,7 +779,9 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
 // bins over the row's range, as in the distribution sort but kClBins of them: the CTAs' histograms are merged through
 // distributed shared memory, the CTAs agree on the bin that holds the kk-th key, and every key up to it goes to the
 // first CTA's list, which is then sorted there.  A bin that holds more keys than the list takes is split again over
-// its own range (a few outliers stretch the range); what still does not fit (mass ties), and a row with infinite or NaN scores
+// its own range (a few outliers stretch the range), and a bin of one single value by the keys' indices, in whose order ties
+// are taken (1 x 300 K keys of 50 different scores, topk 64: 453 us when the row was left to a radix select by one CTA, now 42);
+// what still does not fit, and a row with infinite or NaN scores
 // or with whatever a scan that gave up left behind, goes to the first CTA's radix select over the whole row, which is total.  Bound by latencies (four cluster barriers, a sort by one CTA) up to 128 K keys, by
 // instructions above: a key costs about 15, on floats throughout (ordered bit patterns would double that).
 // ---------------------------------------------------------------------------------------------
@@ -798,8 +802,42 @@ __device__ __forceinline__ unsigned int warp_inclusive_sum(unsigned int v, int l
   return v;
 }
 
-// p.slice_keys: scores of a slice kept in shared memory (a multiple of 4)
-__global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const SelectRowsParams p) {
+// The rare case of a threshold bin of one value, out of line.  A CTA's slice in pieces of four: the first n_held from shared memory.
+__device__ __forceinline__ int tied_shift(int vis) { return 32 - __clz(static_cast<unsigned int>(vis - 1) / kClBins); }
+struct TiedSlice {
+  const float4* held;
+  const float4* rest;
+  int n_held, n, lo, len, shift;
+  float value;
+  template <class Visit>
+  __device__ __forceinline__ void sweep(Visit&& visit) const {  // visit(score, index in the row)
+    for (int i = threadIdx.x; i < n; i += kClThreads) {
+      const float4 v = i < n_held ? held[i] : __ldcg(rest + i);
+      visit(v.x, lo + 4 * i);
+      if (4 * i + 1 < len) visit(v.y, lo + 4 * i + 1);
+      if (4 * i + 2 < len) visit(v.z, lo + 4 * i + 2);
+      if (4 * i + 3 < len) visit(v.w, lo + 4 * i + 3);
+    }
+  }
+};
+// bins[b] = ties among the keys of run b (2^shift consecutive keys of the row)
+__device__ __noinline__ void count_tied(const TiedSlice t, unsigned int* bins) {
+  t.sweep([&](float v, int i) {
+    if (v == t.value) atomicAdd(&bins[i >> t.shift], 1u);
+  });
+}
+// every key above the ties, and the ties of the runs up to last_run, to the list; *fill counts it
+__device__ __noinline__ void collect_tied(const TiedSlice t, int last_run, uint64_t* list, unsigned int* fill) {
+  t.sweep([&](float v, int i) {
+    if (v > t.value || (v == t.value && (i >> t.shift) <= last_run)) list[atomicAdd(fill, 1u)] = pack_key(v, i);
+  });
+}
+
+// p.slice_keys: scores of a slice kept in shared memory (a multiple of 4).  kPerSm: CTAs to an SM the registers are cut for: one while
+// clusters find free SMs easily (up to 64 CTAs: no spills, 16 x 32 K 25.2 -> 24.4 us), two beyond (128 CTAs in clusters of 8: 16 x
+// 100 K 40.3 -> 35.3 us).
+template <int kPerSm>
+__global__ void __launch_bounds__(kClThreads, kPerSm) select_cluster_kernel(const SelectRowsParams p) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const unsigned int n_cta = cl.num_blocks(), rank = cl.block_rank();
@@ -874,6 +912,7 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
 
   float scale = 0.f, limit = 0.f;
   unsigned int above = 0u, total = 0u;
+  bool tied = false;
   int level = 0;
   for (;; ++level) {
     // range [vmin, vmax] of the keys still in question, over the cluster
@@ -916,16 +955,21 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
     }
     // bin of a score in the range, best scores first; monotone because every step rounds monotonically
     // (finite, so that the best score's 0 * scale is 0)
-    scale = vmax > vmin ? fminf(static_cast<float>(kClBins) / (vmax - vmin), 3e38f) : 0.f;
+    tied = vmax == vmin;
+    scale = tied ? 0.f : fminf(static_cast<float>(kClBins) / (vmax - vmin), 3e38f);
     auto count = [&](float v) {
       if (v >= vmin && v <= vmax) atomicAdd(&bins[min(static_cast<unsigned int>((vmax - v) * scale), kClBins - 1u)], 1u);
     };
-    sweep([&](int, float4 v) {
-      count(v.x);
-      count(v.y);
-      count(v.z);
-      count(v.w);
-    });
+    if (tied) {
+      count_tied(TiedSlice{slice4, mine4, held_pieces, pieces, lo, len, tied_shift(vis), vmax}, bins);
+    } else {
+      sweep([&](int, float4 v) {
+        count(v.x);
+        count(v.y);
+        count(v.z);
+        count(v.w);
+      });
+    }
     cl.sync();
     // merge: this CTA sums the bins of its segment over the cluster
     const int seg = kClBins / static_cast<int>(n_cta);  // 128 .. 1024
@@ -977,7 +1021,7 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
     total = s_total;
     // a key is wanted when it lies in the range or above it and (vmax - v) * scale < limit
     limit = tb == kClBins - 1u ? INFINITY : static_cast<float>(tb + 1u);
-    if (total <= cap || level == kClLevels - 1) break;
+    if (total <= cap || tied || level == kClLevels - 1) break;
     above = s_above;
     // the threshold bin alone is the next level's range
     float nmin = INFINITY, nmax = -INFINITY;
@@ -998,7 +1042,10 @@ __global__ void __launch_bounds__(kClThreads) select_cluster_kernel(const Select
     vmin = nmin;
     vmax = nmax;
   }
-  if (total <= cap) {
+  if (total <= cap && tied) {
+    collect_tied(TiedSlice{slice4, mine4, held_pieces, pieces, lo, len, tied_shift(vis), vmax}, static_cast<int>(s_tb),
+                 cl.map_shared_rank(list, 0), cl.map_shared_rank(&s_fill, 0));
+  } else if (total <= cap) {
     // every wanted key to the first CTA's list: count, reserve, write
     auto wanted = [&](float v) { return v >= vmin && (vmax - v) * scale < limit; };
     unsigned int n = 0;
@@ -1123,10 +1170,12 @@ cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t str
   p.slice_keys = slice_want < slice_max ? slice_want : slice_max;
   const int tail = p.slice_keys * 4 > list ? p.slice_keys * 4 : list;
   const int smem = list + kFineBins * 4 + tail;
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_cluster_kernel), done, true);
+  static std::atomic<unsigned long long> done[2];
+  const bool alone = p.n_blocks * width <= 64;
+  auto kernel = alone ? select_cluster_kernel<1> : select_cluster_kernel<2>;
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel), done[alone ? 0 : 1], true);
   if (e != cudaSuccess) return e;
-  return launch_chained(select_cluster_kernel, p.n_blocks * width, kClThreads, smem, stream, width, p);
+  return launch_chained(kernel, p.n_blocks * width, kClThreads, smem, stream, width, p);
 }
 
 namespace {

@@ -54,6 +54,17 @@ def test_one_score_everywhere():
     _check(inp)
 
 
+@pytest.mark.parametrize("N,topk", [(16388, 64), (20011, 2048), (131072, 8192), (300001, 64), (500000, 2048)])
+@pytest.mark.parametrize("values", [2, 50])
+def test_few_different_scores(values, N, topk):
+    """A threshold bin of one value: its keys are told apart by their indices, in the clusters' slices and at their borders."""
+    inp = make_inputs("iid", "bf16", T=3, N=N, H=64, D=128, topk=topk, seed=N)
+    inp.k[:] = inp.k[np.random.default_rng(values).integers(0, values, size=N)]
+    _check(inp)
+    inp.k[N // 3:] = inp.k[0]  # two thirds of the row are one run of ties
+    _check(inp)
+
+
 def test_paged_keys_take_the_dense_form_too():
     N, T = 30011, 3
     inp = make_inputs("ar1", "e4m3", T=T, N=N, H=64, D=128, topk=600, seed=8)
