@@ -26,7 +26,8 @@ constexpr int kSelCap = 2 * LT_MAX_TOPK;  // 64-bit keys the final select can so
 // heads of dots in registers (three 16-byte shared loads per 32 FMAs), a warp covers 128 keys of one query row, the eight
 // warps of a CTA share the key tile (kRows query rows x 8 / kRows runs of 128 keys).  With a thread per key that fetched
 // both operands of every FMA, 64 x 4096 x 8 heads x 64 took 49 us and
-// 128 x 16384 x 32 x 128 2659 us; now 14 and 457 us (half of the fp32 FMA peak).  Dots run over d and the head sum over h in
+// 128 x 16384 x 32 x 128 2659 us; now 14 and 457 us (half of the fp32 FMA peak).  Warps without a row only help to stage: with their
+// FMAs 1 x 20001 x 32 x 128, nine CTAs more than SMs, took 65 us, now 36 for the scores.  Dots run over d and the head sum over h in
 // ascending order, one FMA each: every launch shape gives the same bits.
 // ---------------------------------------------------------------------------------------------
 template <int kDtype>
@@ -101,6 +102,7 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void
       } else if (h0 + kSimtHeads < H) {
         fetch(h0 + kSimtHeads, 0);
       }
+      if (t >= row_end) continue;  // a warp without a row leaves the FMA units to the others
 #pragma unroll
       for (int d = 0; d < kSimtD; ++d) {
         const float4 kv = *reinterpret_cast<const float4*>(&ks[d][key]);
