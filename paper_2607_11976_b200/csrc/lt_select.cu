@@ -790,7 +790,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
 constexpr int kClThreads = 512;
 constexpr int kClWarps = kClThreads / 32;
 constexpr int kClBins = 2048;
-constexpr int kClLevels = 3;
+constexpr int kClLevels = 6;  // ties next to a dense stretch of scores (ReLU's exact zeros) take one more for every factor of 2048
 constexpr int kClStaticSmem = 8 * 1024;  // upper bound of what the kernel declares statically
 // (a multiple of four keys: what lies behind the list is accessed in 16-byte pieces)
 __host__ __device__ constexpr int cluster_list_cap(int topk) { return (topk + (topk / 4 > 2048 ? topk / 4 : 2048) + 3) / 4 * 4; }
