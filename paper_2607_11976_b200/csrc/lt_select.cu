@@ -630,19 +630,33 @@ __device__ __noinline__ void radix_select_row(const float* row, int vis, int kk,
     }
     if (run_len > 0) atomicAdd(&hist[run_digit], run_len);
     __syncthreads();
-    if (tid == 0) {
-      unsigned int remaining = s_remaining, cum = 0;
-      int digit = 0;
-      for (int d = 255; d >= 0; --d) {
-        unsigned int c = hist[d];
-        if (cum + c >= remaining) {
-          digit = d;
-          break;
-        }
-        cum += c;
+    if (tid < 32) {
+      // suffix sums over the 256 digits, 8 per lane: the digit where the count from the top reaches what is still needed
+      unsigned int c[8], mine = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        c[j] = hist[lane * 8 + j];
+        mine += c[j];
       }
-      s_remaining = remaining - cum;  // still needed among keys that share the longer prefix
-      s_prefix = prefix | (static_cast<unsigned int>(digit) << shift);
+      unsigned int incl = mine;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const unsigned int o = __shfl_down_sync(0xffffffffu, incl, d);
+        if (lane + d < 32) incl += o;
+      }
+      const unsigned int remaining = s_remaining;
+      unsigned int cum = incl - mine;
+      __syncwarp();
+      if (cum < remaining && incl >= remaining) {  // exactly one lane
+        int digit = -1;
+#pragma unroll
+        for (int j = 7; j >= 0; --j) {
+          if (digit < 0 && cum + c[j] >= remaining) digit = lane * 8 + j;
+          if (digit < 0) cum += c[j];
+        }
+        s_remaining = remaining - cum;  // still needed among keys that share the longer prefix
+        s_prefix = prefix | (static_cast<unsigned int>(digit) << shift);
+      }
     }
     mask |= 0xffu << shift;
     __syncthreads();
