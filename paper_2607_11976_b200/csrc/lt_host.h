@@ -29,6 +29,40 @@ inline cudaError_t allow_smem(const void* kernel, std::atomic<unsigned long long
   return e;
 }
 
+// Clusters of `cluster` CTAs of a kernel that the current device (or the part of it that this process may use) holds at once; 0 where
+// it can place none.
+template <typename... Params>
+inline int clusters_at_once(void (*kernel)(Params...), int threads, size_t smem, int cluster) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = static_cast<unsigned int>(cluster);
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned int>(cluster));
+  cfg.blockDim = dim3(static_cast<unsigned int>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess) return n;
+  cudaGetLastError();
+  return 0;
+}
+// The widest cluster of up to 16 CTAs with `smem` bytes each that the current device can place, found once for each device: cache[dev]
+// belongs to that kernel.
+template <typename... Params>
+inline int widest_cluster(void (*kernel)(Params...), int threads, size_t smem, std::atomic<signed char>* cache) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  int width = cache[dev & 63].load(std::memory_order_relaxed);
+  if (width == 0) {
+    for (width = 16; width > 1 && clusters_at_once(kernel, threads, smem, width) < 1;) width >>= 1;
+    cache[dev & 63].store(static_cast<signed char>(width), std::memory_order_relaxed);
+  }
+  return width;
+}
+
 // Launch of a kernel that calls chain_wait (see lt_common.cuh), optionally in clusters of `cluster` CTAs.
 template <typename... Params, typename... Args>
 inline cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, int cluster,

@@ -9,6 +9,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "lt_cluster_width.h"
 #include "lt_common.cuh"
 #include "lt_fine_select.cuh"
 #include "lt_host.h"
@@ -17,7 +18,6 @@ namespace lt {
 
 namespace {
 
-constexpr int kSelDirect = 16384;  // rows up to this length are sorted without a select (a few batches of registers)
 constexpr int kSelBatch = 8;  // independent row loads in flight per thread of the full-row select
 constexpr int kSelCap = 2 * LT_MAX_TOPK;  // 64-bit keys the final select can sort in shared memory
 
@@ -1176,9 +1176,13 @@ cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t str
   if (params.N <= kSelDirect) return launch_select_rows(params, stream);
   SelectRowsParams p = params;
   if (p.n_blocks <= 0) return cudaSuccess;
-  int width = 2;
-  while (width < 16 && static_cast<long long>(width) * kSelDirect < p.N) width <<= 1;
-  if (width > 8 && p.n_blocks * width > 128) width = 8;  // clusters of 16 need a whole GPC: only while few are wanted
+  static std::atomic<unsigned long long> done[2];
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_cluster_kernel<1>), done[0], true);
+  if (e == cudaSuccess) e = allow_smem(reinterpret_cast<const void*>(select_cluster_kernel<2>), done[1], true);
+  if (e != cudaSuccess) return e;
+  static std::atomic<signed char> widest[64];
+  const int width = select_cluster_width(p.N, p.n_blocks, widest_cluster(select_cluster_kernel<1>, kClThreads, 227 * 1024 - kClStaticSmem, widest));
+  if (width < 2) return launch_select_rows(params, stream);
   // shared memory: the list, the bins, and as much of a slice as fits (at least the sort's second buffer)
   const int list = cluster_list_cap(p.topk) * 8;
   const int slice_max = (227 * 1024 - kClStaticSmem - list - kFineBins * 4) / 16 * 4;
@@ -1186,11 +1190,7 @@ cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t str
   p.slice_keys = slice_want < slice_max ? slice_want : slice_max;
   const int tail = p.slice_keys * 4 > list ? p.slice_keys * 4 : list;
   const int smem = list + kFineBins * 4 + tail;
-  static std::atomic<unsigned long long> done[2];
-  const bool alone = p.n_blocks * width <= 64;
-  auto kernel = alone ? select_cluster_kernel<1> : select_cluster_kernel<2>;
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel), done[alone ? 0 : 1], true);
-  if (e != cudaSuccess) return e;
+  auto kernel = static_cast<long long>(p.n_blocks) * width <= 64 ? select_cluster_kernel<1> : select_cluster_kernel<2>;
   return launch_chained(kernel, p.n_blocks * width, kClThreads, smem, stream, width, p);
 }
 
