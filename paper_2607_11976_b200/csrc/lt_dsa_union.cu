@@ -9,13 +9,14 @@
 // distributed shared memory (a CTA combines one slice and hands it to all), and from then on every CTA can turn a
 // position into its slot on its own: it writes its slice of the list and builds its rows' masks in shared memory.
 // With one CTA per group, outputs cleared by memsets and masks built by global atomics, 4096 rows x 2048 over 128 K
-// positions in groups of 64 took 201 us; now 69 us, with 25 us the time of
+// positions in groups of 64 took 201 us; now 63 us, with 25 us the time of
 // moving the bytes.  What is left is the chain of phases of a CTA (mark 5 us, combine 5, prefix 2, list 4, masks 20 - 28) and
 // clusters that fill some GPCs' SMs with four CTAs and others' with three.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lt_cluster_width.h"
 #include "lt_common.cuh"
 #include "lt_host.h"
 
@@ -23,11 +24,16 @@ namespace lt {
 
 namespace {
 
-constexpr int kUnionThreads = 512;
-constexpr int kUnionWarps = kUnionThreads / 32;
-constexpr int kWindowWords = 32768;     // bitmap words per pass: 1,048,576 positions, 128 KB
-constexpr int kWordPrefixMax = 8192;    // windows of up to this many words keep a prefix per word, larger ones per 4 words
-constexpr int kMaskBufWords = 4096;     // mask buffer: 131,072 slots
+// Bitmap words per pass, words to a stored prefix and words of the mask buffer.  The longer the context, the more of the shared
+// memory the bitmap takes: up to 262,144 positions a prefix per word, up to 1,048,576 (128 KB of bitmap) one per 4 words, beyond
+// that windows of 1,572,864 positions (192 KB) with one per 8 - or of 1,048,576, where a mask does not fit the smaller buffer
+// beside the large window (each piece of a mask looks all entries up again).
+constexpr int kWordPrefixMax = 8192;
+constexpr int kFourPrefixMax = 32768;
+constexpr int kWindowWords = 49152;
+constexpr int kMaskBufWords = 4096;      // 131,072 slots
+constexpr int kMaskBufWordsWide = 2048;  // ... beside a bitmap of 192 KB
+constexpr int kUnionWideEntries = 2048;  // see the launch
 
 struct UnionParams {
   const int32_t* idx;   // [T][topk]
@@ -43,7 +49,7 @@ struct UnionParams {
 };
 
 // (a multiple of four: the masks behind the prefix are accessed in 16-byte pieces)
-__host__ __device__ constexpr int prefix_words(bool per_word, int window_words) { return per_word ? window_words : (window_words / 4 + 3) / 4 * 4; }
+__host__ __device__ constexpr int prefix_words(int unit, int window_words) { return unit == 1 ? window_words : (window_words / unit + 3) / 4 * 4; }
 
 __device__ __forceinline__ unsigned int popc4(uint4 v) { return __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w); }
 
@@ -56,16 +62,17 @@ __device__ __forceinline__ unsigned int warp_inclusive_sum(unsigned int v, int l
   return v;
 }
 
-// kWordPrefix: the window is small enough for a prefix per word
-template <bool kWordPrefix>
-__global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_kernel(const UnionParams p) {
+// kUnit: words to a stored prefix (1, 4 or 8).  512 threads while several CTAs share an SM, 1024 where one has it to itself.
+template <int kUnit, int kUnionThreads>
+__global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUnit == 1 ? 4 : 2) dsa_union_kernel(const UnionParams p) {
+  constexpr int kUnionWarps = kUnionThreads / 32;
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   const int n_cta = static_cast<int>(cl.num_blocks()), rank = static_cast<int>(cl.block_rank());
   extern __shared__ __align__(16) uint32_t smem_u[];
   uint32_t* bitmap = smem_u;
-  uint32_t* prefix = bitmap + p.window_words;  // list slots before every word, or every 4 words (within the window)
-  uint32_t* masks = prefix + prefix_words(kWordPrefix, p.window_words);
+  uint32_t* prefix = bitmap + p.window_words;  // list slots before every kUnit words (within the window)
+  uint32_t* masks = prefix + prefix_words(kUnit, p.window_words);
   __shared__ unsigned int warp_tot[kUnionWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int grp = static_cast<int>(blockIdx.x) / n_cta;
@@ -130,14 +137,15 @@ __global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_
       }
       cl.sync();
     }
-    // 3. list slots before every 4 words: each warp owns a run of consecutive 128-word groups, 4 words per lane
+    // 3. list slots before every unit: each warp owns a run of consecutive groups of 32 pieces of 4 (or 8) words, a piece per lane
     const uint4* bitmap4 = reinterpret_cast<const uint4*>(bitmap);
-    const int units = words / 4;
+    const int units = words / (kUnit == 8 ? 8 : 4);
+    auto popc_piece = [&](int u) { return kUnit == 8 ? popc4(bitmap4[2 * u]) + popc4(bitmap4[2 * u + 1]) : popc4(bitmap4[u]); };
     const int groups = (units + 31) / 32;
     const int per_warp = (groups + kUnionWarps - 1) / kUnionWarps;
     const int u0 = min(groups, warp * per_warp) * 32, u1 = min(units, u0 + per_warp * 32);
     unsigned int mine = 0;
-    for (int u = u0 + lane; u < u1; u += 32) mine += popc4(bitmap4[u]);
+    for (int u = u0 + lane; u < u1; u += 32) mine += popc_piece(u);
     mine = __reduce_add_sync(0xffffffffu, mine);
     if (lane == 0) warp_tot[warp] = mine;
     __syncthreads();
@@ -145,11 +153,11 @@ __global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_
     const unsigned int total = __reduce_add_sync(0xffffffffu, wt);
     unsigned int run = __reduce_add_sync(0xffffffffu, lane < warp ? wt : 0u);
     for (int u = u0; u < u1; u += 32) {
-      const unsigned int c = u + lane < u1 ? popc4(bitmap4[u + lane]) : 0u;
+      const unsigned int c = u + lane < u1 ? popc_piece(u + lane) : 0u;
       const unsigned int incl = warp_inclusive_sum(c, lane);
       if (u + lane < u1) {
         const unsigned int before = run + incl - c;
-        if (kWordPrefix) {
+        if (kUnit == 1) {
           const uint4 v = bitmap4[u + lane];
           const unsigned int p1 = before + __popc(v.x), p2 = p1 + __popc(v.y), p3 = p2 + __popc(v.z);
           reinterpret_cast<uint4*>(prefix)[u + lane] = make_uint4(before, p1, p2, p3);
@@ -164,18 +172,28 @@ __global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_
     // warp and step, which coalesces the stores, sparse ones (a context much longer than the list) a word per lane
     for (int w = s0 + warp * 32; w < s1; w += kUnionThreads) {
       const uint32_t own = w + lane < s1 ? bitmap[w + lane] : 0u;
-      const unsigned int c = __popc(own);
-      const unsigned int incl = warp_inclusive_sum(c, lane);
-      int32_t* dst = out + list_len + prefix[kWordPrefix ? w : w >> 2];
-      if (__shfl_sync(0xffffffffu, incl, 31) >= 96u) {
+      const unsigned int in_all = __reduce_add_sync(0xffffffffu, static_cast<unsigned int>(__popc(own)));
+      if (in_all == 0u) continue;
+      int32_t* dst = out + list_len;
+      if (in_all >= 96u) {
+        dst += prefix[w / kUnit];  // (w is a multiple of eight)
 #pragma unroll 8
         for (int j = 0; j < 32; ++j) {
           const uint32_t word = __shfl_sync(0xffffffffu, own, j);
           if ((word >> lane) & 1u) dst[__popc(word & ((1u << lane) - 1u))] = base + (w + j) * 32 + lane;
           dst += __popc(word);
         }
-      } else {
-        dst += incl - c;
+      } else if (kUnit == 8) {  // (a scan over the warp is shorter than the set bits of up to seven words of the unit)
+        const unsigned int c = __popc(own);
+        dst += prefix[w / kUnit] + warp_inclusive_sum(c, lane) - c;
+        for (uint32_t word = own; word != 0u; word &= word - 1u) *dst++ = base + (w + lane) * 32 + __ffs(word) - 1;
+      } else if (own != 0u) {
+        dst += prefix[(w + lane) / kUnit];
+        if (kUnit == 4) {
+          const uint4 v = bitmap4[(w + lane) >> 2];
+          const int k = lane & 3;
+          dst += (k > 0 ? __popc(v.x) : 0) + (k > 1 ? __popc(v.y) : 0) + (k > 2 ? __popc(v.z) : 0);
+        }
         for (uint32_t word = own; word != 0u; word &= word - 1u) *dst++ = base + (w + lane) * 32 + __ffs(word) - 1;
       }
     }
@@ -206,13 +224,14 @@ __global__ void __launch_bounds__(kUnionThreads, kWordPrefix ? 4 : 1) dsa_union_
               if (pos[j] < base || q >= static_cast<unsigned int>(span)) continue;
               const unsigned int below = (1u << (q & 31)) - 1u;
               unsigned int slot = list_len;
-              if (kWordPrefix) {
+              if (kUnit == 1) {
                 slot += prefix[q >> 5] + __popc(bitmap[q >> 5] & below);
               } else {
                 const uint4 v = bitmap4[q >> 7];
                 const unsigned int k = (q >> 5) & 3u;
                 const uint32_t word = k == 0u ? v.x : k == 1u ? v.y : k == 2u ? v.z : v.w;
-                slot += prefix[q >> 7] + __popc(word & below) + (k > 0u ? __popc(v.x) : 0) + (k > 1u ? __popc(v.y) : 0) + (k > 2u ? __popc(v.z) : 0);
+                if (kUnit == 8 && ((q >> 7) & 1u) != 0u) slot += popc4(bitmap4[(q >> 7) - 1u]);
+                slot += prefix[(q >> 5) / kUnit] + __popc(word & below) + (k > 0u ? __popc(v.x) : 0) + (k > 1u ? __popc(v.y) : 0) + (k > 2u ? __popc(v.z) : 0);
               }
               const int mw = static_cast<int>(slot >> 5) - w0;
               const int r = rows == 1 ? 0 : min(i + j * kUnionThreads, n - 1) / p.topk;
@@ -273,25 +292,61 @@ cudaError_t launch_dsa_union(const int32_t* idx, int T, int topk, int N, int gro
   p.mask = mask;
   const int n_groups = (T + group - 1) / group;
   const int words = (static_cast<int>((static_cast<long long>(N) + 31) / 32) + 7) / 8 * 8;
-  p.window_words = words < kWindowWords ? words : kWindowWords;
-  const bool word_prefix = p.window_words <= kWordPrefixMax;
-  // As many CTAs per group as it has rows and as run at the same time: a CTA that waits for a second wave pays the clearing,
-  // combining and sweeping of its copy of the bitmap all over (4096 x 2048 over 1 M positions in 64 groups: width 2 / 4 / 8
-  // 106 / 117 / 188 us; over 128 K positions 103 / 72 / 69 us).  Sixteen CTAs need a whole GPC: only for few groups.
-  const int resident = 148 * (word_prefix ? 4 : 1);
-  int width = 1;
-  while (width < 8 && width < group && n_groups * width * 2 <= resident) width <<= 1;
-  if (width == 8 && group >= 16 && n_groups * 16 <= 128) width = 16;
-  p.rows_per_cta = (group + width - 1) / width;
-  // the buffer holds all of a CTA's rows, or as much as kMaskBufWords
-  const long long all_rows = static_cast<long long>(p.mask_words) * p.rows_per_cta;
-  p.buf_words = all_rows < kMaskBufWords ? static_cast<int>(all_rows + 3) / 4 * 4 : kMaskBufWords;
-  const int smem = (p.window_words + prefix_words(word_prefix, p.window_words) + p.buf_words) * 4;
-  static std::atomic<unsigned long long> done[2];
-  auto kernel = word_prefix ? dsa_union_kernel<true> : dsa_union_kernel<false>;
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernel), done[word_prefix ? 1 : 0], true);
+  const int unit = words <= kWordPrefixMax ? 1 : words <= kFourPrefixMax || p.mask_words > kMaskBufWordsWide ? 4 : 8;
+  const int window_max = unit == 8 ? kWindowWords : kFourPrefixMax;
+  p.window_words = words < window_max ? words : window_max;
+  const int buf_max = unit == 8 ? kMaskBufWordsWide : kMaskBufWords;
+  const int rows = group < T ? group : T;
+  // shared memory with a mask buffer for n rows, or for as much of them as buf_max
+  auto shared_bytes = [&](int n) {
+    const long long n_words = static_cast<long long>(p.mask_words) * n;
+    p.buf_words = n_words < buf_max ? static_cast<int>(n_words + 3) / 4 * 4 : buf_max;
+    return (p.window_words + prefix_words(unit, p.window_words) + p.buf_words) * 4;
+  };
+
+  // by unit and threads
+  static std::atomic<unsigned long long> done[5];
+  using Kernel = void (*)(UnionParams);
+  const Kernel kernels[5] = {dsa_union_kernel<1, 512>, dsa_union_kernel<1, 1024>, dsa_union_kernel<4, 512>, dsa_union_kernel<4, 1024>,
+                             dsa_union_kernel<8, 1024>};
+  const int first = unit == 1 ? 0 : unit == 4 ? 2 : 4;
+  cudaError_t e = cudaSuccess;
+  for (int k = first; k < (unit == 8 ? 5 : first + 2) && e == cudaSuccess; ++k) e = allow_smem(reinterpret_cast<const void*>(kernels[k]), done[k], true);
   if (e != cudaSuccess) return e;
-  return launch_chained(kernel, n_groups * width, kUnionThreads, smem, stream, width, p);
+  // how many clusters of a width run at once: asked for once for each device, unit, CTAs of that size to an SM, and width (with the
+  // largest mask buffer, of one CTA for all rows)
+  const int smem_max = shared_bytes(rows);
+  const int per_sm = (228 * 1024) / (smem_max + 2048) < 4 ? (228 * 1024) / (smem_max + 2048) : 4;
+  static std::atomic<short> at_once_cache[64][3][4][5];
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  auto at_once = [&](int width) {
+    // (sharing an SM pays CTAs of at most 32 KB of bitmap: 1024 x 2048 over 524,288 positions in 32 groups, width 4 / 8, 31 / 34 us)
+    if (unit != 1 && static_cast<long long>(n_groups) * width > sms) return 0;
+    int log2 = 0;
+    while ((1 << log2) < width) ++log2;
+    std::atomic<short>& known = at_once_cache[dev & 63][first / 2][per_sm > 0 ? per_sm - 1 : 0][log2];
+    int n = known.load(std::memory_order_relaxed);
+    if (n == 0) {
+      n = 1 + clusters_at_once(kernels[first], unit == 8 ? 1024 : 512, smem_max, width);
+      known.store(static_cast<short>(n), std::memory_order_relaxed);
+    }
+    return n - 1;
+  };
+  const int width = union_cluster_width(n_groups, rows, static_cast<long long>(rows) * topk, sms, at_once);
+  p.rows_per_cta = (rows + width - 1) / width;
+  const int smem = shared_bytes(p.rows_per_cta);
+  // A CTA with an SM to itself and little to mark is bound by its sweeps over the bitmap: 1024 threads halve them (8 rows x 2048 over
+  // 200,000 positions, width 8, 13.6 -> 12.2 us; but 64 x 2048 over 131,072, width 16, 8192 entries a CTA, 17.2 -> 21.1).
+  // Wide CTAs do not share an SM, which leaves few places for clusters of 8 (500 x 512 in 16 groups, width 8, 17.4 -> 22.7).  Beside
+  // a window of 192 KB there is one CTA to an SM in any case.
+  const bool wide = unit == 8 ||
+                    (static_cast<long long>(n_groups) * width <= (width == 1 ? sms : unit == 1 ? sms / 2 : 0) &&
+                     static_cast<long long>(p.rows_per_cta) * topk <= kUnionWideEntries);
+  const Kernel kernel = kernels[unit == 8 || !wide ? first : first + 1];
+  return launch_chained(kernel, n_groups * width, wide ? 1024 : 512, smem, stream, width, p);
 }
 
 }  // namespace lt

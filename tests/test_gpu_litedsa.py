@@ -74,10 +74,12 @@ def test_union_of_real_topk_rows_and_bad_arguments():
 
 
 @pytest.mark.parametrize("T,topk,N,group", [(3, 5, 262144, 3), (40, 64, 262145, 40), (130, 33, 1 << 20, 1), (20, 700, (1 << 20) + 1, 10),
-                                            (300, 40, 60000, 32), (12, 4096, 9000, 12), (64, 4100, 70000, 64), (9, 16, 2_100_000, 9)])
+                                            (300, 40, 60000, 32), (12, 4096, 9000, 12), (64, 4100, 70000, 64), (9, 16, 2_100_000, 9),
+                                            (20, 700, 1_572_864, 10), (3, 40, 1_572_865, 3), (40, 64, 1_572_865, 20), (64, 4100, 1_700_000, 64)])
 def test_window_buffer_and_cluster_edges(T, topk, N, group):
-    """Around the sizes where the kernel changes its layout: a prefix per word or per four words (262,144 positions), one or
-    several windows (2^20), masks of several rows at once or of one row in pieces (131,072 slots), 1 to 16 CTAs a group."""
+    """Around the sizes where the kernel changes its layout: a prefix per word, per four words (262,144 positions) or
+    per eight (2^20), one or several windows (1,572,864), masks of several rows at once or of one row in pieces (131,072 or 65,536
+    slots), 1 to 16 CTAs a group."""
     rng = np.random.default_rng(N + T)
     idx = rng.integers(0, N, size=(T, topk))
     idx[:, :2] = [0, N - 1] if topk > 1 else 0
