@@ -33,8 +33,11 @@ def test_ordinary_cases_leave_the_bounds_bit_clear(name, T, N, topk, debug_libra
     lt.use_library(None)
     want = run_topk(inp)
     lt.use_library(debug_library)
-    for tun in (None, lt.Tunables(cap_mult=1, sample_rank=1)):  # the second one forces rows through the exact fallback
+    fused = [] if inp.dtype == "f32" else [lt.Tunables(path=lt.LT_PATH_FUSED)]  # the sampled form, which small problems leave out
+    for tun in [None, lt.Tunables(cap_mult=1, sample_rank=1)] + fused:  # the second one forces rows through the exact fallback
         got = run_topk(inp, tun)
+        if tun in fused:
+            assert got[2][3] > 0
         assert got[2][0] & lt.LT_STATUS_BOUNDS == 0, "a bounds check failed on a valid problem"
         assert got[2][0] & lt.LT_STATUS_TIMEOUT == 0
         assert np.array_equal(got[0], want[0]) and np.array_equal(got[1].view(np.uint32), want[1].view(np.uint32))
@@ -58,12 +61,13 @@ def test_paged_cache_is_clean_and_a_bad_page_table_is_caught(debug_library):
     assert got[2][0] & lt.LT_STATUS_TIMEOUT == 0
 
 
-def test_knn_is_clean(debug_library):
+@pytest.mark.parametrize("tun", [None, lt.Tunables(path=lt.LT_PATH_FUSED)], ids=["dense", "sampled"])
+def test_knn_is_clean(tun, debug_library):
     from test_gpu_knn import gpu_topk  # the driver of the k-NN parity tests
     inp = make_knn(T=64, N=20000, D=256, topk=128)
     lt.use_library(None)
     want = gpu_topk(inp)
     lt.use_library(debug_library)
-    got = gpu_topk(inp)
-    assert got[2][0] & lt.LT_STATUS_BOUNDS == 0
+    got = gpu_topk(inp, tun)
+    assert got[2][0] & lt.LT_STATUS_BOUNDS == 0 and (got[2][3] > 0) == (tun is not None)
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1].view(np.uint32), want[1].view(np.uint32))

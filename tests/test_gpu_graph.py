@@ -17,16 +17,21 @@ def _bits(t):
     return t.cpu().numpy().view(np.uint32)
 
 
+# both forms of the tensor-core path: dense scores and a select (default at these sizes), and the whole sampled chain
+FORMS = [None, lt.Tunables(path=lt.LT_PATH_FUSED)]
+
+
+@pytest.mark.parametrize("tun", FORMS, ids=["dense", "sampled"])
 @pytest.mark.parametrize("name", ["dsa_bf16", "fp8_ar1"])
-def test_indexer_topk_replays_from_a_cuda_graph(name):
+def test_indexer_topk_replays_from_a_cuda_graph(name, tun):
     a = make_config(name, T=72, N=20000, topk=384)
     q, w, k, ks = lt.to_device(a)
     idx = torch.empty((a.T, a.topk), dtype=torch.int32, device="cuda")
     score = torch.empty((a.T, a.topk), dtype=torch.float32, device="cuda")
-    ws = lt.alloc_workspace(a.dtype, a.T, a.N, a.H, a.D, a.topk)
+    ws = lt.alloc_workspace(a.dtype, a.T, a.N, a.H, a.D, a.topk, tun)
 
     def call():
-        lt.lt_indexer_topk_ex(a.dtype, q, w, k, ks, a.topk, a.causal_offset, idx, score, ws)
+        lt.lt_indexer_topk_ex(a.dtype, q, w, k, ks, a.topk, a.causal_offset, idx, score, ws, tun)
 
     call()  # eager once: loads the kernels and sets their attributes outside the capture
     torch.cuda.synchronize()
@@ -41,7 +46,8 @@ def test_indexer_topk_replays_from_a_cuda_graph(name):
     graph.replay()
     torch.cuda.synchronize()
     assert lt.lt_launch_count() == launches  # a replay goes through no library call
-    assert lt.lt_read_status(ws)[0] == 0
+    status = lt.lt_read_status(ws)
+    assert status[0] == 0 and (status[3] > 0) == (tun is not None)  # survivors of the gate: the sampled form ran, or did not
     assert torch.equal(idx, want_idx) and np.array_equal(_bits(score), _bits(want_score))
 
     # new inputs behind the same pointers: reversed key order (and scales), rows shifted by one
@@ -59,16 +65,17 @@ def test_indexer_topk_replays_from_a_cuda_graph(name):
     assert torch.equal(got_idx, idx) and np.array_equal(_bits(got_score), _bits(score))
 
 
-def test_knn_topk_replays_from_a_cuda_graph():
+@pytest.mark.parametrize("tun", FORMS, ids=["dense", "sampled"])
+def test_knn_topk_replays_from_a_cuda_graph(tun):
     kn = make_knn(T=24, N=30000, D=256, topk=200)
     q = torch.from_numpy(kn.q.view("int16")).to("cuda").view(torch.bfloat16)
     x = torch.from_numpy(kn.x.view("int16")).to("cuda").view(torch.bfloat16)
     idx = torch.empty((kn.T, kn.topk), dtype=torch.int32, device="cuda")
     score = torch.empty((kn.T, kn.topk), dtype=torch.float32, device="cuda")
-    ws = torch.empty(lt.lt_knn_topk_workspace_bytes(kn.T, kn.N, kn.D, kn.topk), dtype=torch.uint8, device="cuda")
+    ws = torch.empty(lt.lt_knn_topk_workspace_bytes(kn.T, kn.N, kn.D, kn.topk, tun), dtype=torch.uint8, device="cuda")
 
     def call():
-        lt.lt_knn_topk(q, x, kn.topk, idx, score, ws)
+        lt.lt_knn_topk(q, x, kn.topk, idx, score, ws, tun)
 
     call()
     torch.cuda.synchronize()
@@ -81,5 +88,6 @@ def test_knn_topk_replays_from_a_cuda_graph():
     got_idx, got_score = idx.clone(), score.clone()
     call()
     torch.cuda.synchronize()
-    assert lt.lt_read_status(ws)[0] == 0
+    status = lt.lt_read_status(ws)
+    assert status[0] == 0 and (status[3] > 0) == (tun is not None)
     assert torch.equal(got_idx, idx) and np.array_equal(_bits(got_score), _bits(score))

@@ -65,11 +65,12 @@ def test_dense_scores_match_oracle(T, N, D):
         assert np.array_equal(part.view(np.uint32), got[2:T - 1].view(np.uint32))
 
 
+@pytest.mark.parametrize("tun", [None, lt.Tunables(path=lt.LT_PATH_FUSED)], ids=["dense", "sampled"])
 @pytest.mark.parametrize("T,N,D,topk", [(64, 40000, 768, 512), (9, 20000, 128, 64), (100, 30001, 256, 1024), (64, 9000, 768, 4096)])
-def test_topk_matches_oracle_and_own_scores(T, N, D, topk):
+def test_topk_matches_oracle_and_own_scores(T, N, D, topk, tun):
     inp = make_knn(T=T, N=N, D=D, topk=topk)
-    idx, score, st = gpu_topk(inp)
-    assert st[0] & lt.LT_STATUS_TIMEOUT == 0
+    idx, score, st = gpu_topk(inp, tun)
+    assert st[0] & lt.LT_STATUS_TIMEOUT == 0 and (st[3] > 0) == (tun is not None)
     dumped = gpu_scores(inp, 0, T)
     check(inp, idx, score, list(range(0, T, max(1, T // 9))), dumped)
     for t in range(T):  # own-scores rule for every row
@@ -97,6 +98,7 @@ def test_fallback_and_tunables_keep_every_bit():
     base_idx, base_score, st0 = gpu_topk(inp)
     assert st0[1] == 0
     for tun in (lt.Tunables(cap_mult=1), lt.Tunables(sample_rank=1), lt.Tunables(sample_rank=-1), lt.Tunables(segment_tiles=3, grid=7),
+                lt.Tunables(path=lt.LT_PATH_FUSED, segment_tiles=3, grid=7), lt.Tunables(path=lt.LT_PATH_FUSED, segment_tiles=1000),
                 lt.Tunables(sample_mult=1), lt.Tunables(segment_tiles=1000)):
         idx, score, st = gpu_topk(inp, tun)
         assert st[0] & lt.LT_STATUS_TIMEOUT == 0
@@ -142,6 +144,8 @@ def test_random_shapes():
         inp = make_knn(T=T, N=N, D=D, topk=topk)
         idx, score, st = gpu_topk(inp)
         assert st[0] & lt.LT_STATUS_TIMEOUT == 0, (T, N, D, topk)
+        f_idx, f_score, st = gpu_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED))
+        assert st[3] > 0 and np.array_equal(idx, f_idx) and np.array_equal(score.view(np.uint32), f_score.view(np.uint32)), (T, N, D, topk)
         dumped = gpu_scores(inp, 0, T)
         rows = sorted(set(int(r) for r in rng.integers(0, T, size=3)))
         check(inp, idx, score, rows, dumped)
