@@ -126,8 +126,9 @@ constexpr long long kDenseShortPairs = 1ll << 20;
 bool use_direct(const Tun& tun, int T, int N, int topk, bool paged, int knn_dim) {
   // an explicit path or a tunable of the sampled form asks for that form
   if (tun.path != LT_PATH_AUTO || tun.sample_mult_given || tun.cap_mult_given || tun.sample_rank != 0) return false;
-  // over a paged cache only up to one query block: larger chunks report the survivor counts of the sampled form, which
-  // equal those over dense keys and which callers compare
+  // Over a paged cache only up to one query block.  Larger chunks stay with the sampled form, whose survivor counts their callers
+  // read from the status block; the dense form would filter nothing and report none.  That is not for speed: measured sampled /
+  // dense over paged e4m3 keys, 4096 x 4 K 309 / 179 us, 256 x 16 K 91 / 64, 64 x 64 K 77 / 73, 32 x 128 K 77 / 78.
   if (paged && T > kRowsPerBlock) return false;
   if (N <= kDenseKeys / 2 || (N <= kDenseKeys && topk >= 512)) return true;
   const long long pairs = static_cast<long long>(T) * N;

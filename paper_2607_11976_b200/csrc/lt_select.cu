@@ -556,13 +556,11 @@ __global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const Fi
 }
 
 // ---------------------------------------------------------------------------------------------
-// The kk (<= vis) best of row[0 .. vis), by one CTA, whatever bits the row holds: 4-pass MSB radix select for the kk-th score, then everything above it and
-// the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.  Out of line: it is the rare way of
-// kernels that live for a few microseconds, whose usual way is shorter without it (1 x 32 K dense, topk 2048, 20.9 -> 20.4 us
-// together with the tied slices below).
+// The kk (<= vis) best of row[0 .. vis), by one CTA, whatever bits the row holds: 4-pass MSB radix select for the kk-th score, then
+// everything above it and the lowest indices among its equals, as packed keys in sel[0 .. kk), in no particular order.
 // ---------------------------------------------------------------------------------------------
 template <int kThreads>
-__device__ __noinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel, bool nan_last) {
+__device__ __forceinline__ void radix_select_row(const float* row, int vis, int kk, uint64_t* sel, bool nan_last) {
   constexpr int kWarps = kThreads / 32;
   __shared__ unsigned int hist[256];
   __shared__ unsigned int s_prefix, s_remaining, s_gt;
@@ -818,7 +816,13 @@ __device__ __forceinline__ unsigned int warp_inclusive_sum(unsigned int v, int l
   return v;
 }
 
-// The rare case of a threshold bin of one value, out of line.  A CTA's slice in pieces of four: the first n_held from shared memory.
+// The rare ways of the cluster select are out of line: it lives for a few microseconds, and its usual way is shorter without them (1 x
+// 32 K dense, topk 2048, 20.9 -> 20.4 us).  (Inlined into the select by one CTA, the radix select costs nothing.)
+__device__ __noinline__ void radix_select_row_rare(const float* row, int vis, int kk, uint64_t* sel, bool nan_last) {
+  radix_select_row<kClThreads>(row, vis, kk, sel, nan_last);
+}
+
+// A threshold bin of one value.  A CTA's slice in pieces of four: the first n_held from shared memory.
 __device__ __forceinline__ int tied_shift(int vis) { return 32 - __clz(static_cast<unsigned int>(vis - 1) / kClBins); }
 struct TiedSlice {
   const float4* held;
@@ -1099,7 +1103,7 @@ __global__ void __launch_bounds__(kClThreads, kPerSm) select_cluster_kernel(cons
     if (fine_select_sort<kClThreads>(entry, first, total, kk, p.topk, sorted, cap, bins, out_idx, out_score, p.N, p.ctl)) return;
     if (total > static_cast<unsigned int>(kk)) keep_top_keys(list, static_cast<int>(total), kk, bins, &s_count);
   } else {
-    radix_select_row<kClThreads>(row, vis, kk, list, p.nan_last != 0);
+    radix_select_row_rare(row, vis, kk, list, p.nan_last != 0);
   }
   __syncthreads();
   // room for next_pow2(kk) keys: the list, the bins and the slice lie one behind the other
