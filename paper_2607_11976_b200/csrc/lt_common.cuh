@@ -92,6 +92,23 @@ __device__ __forceinline__ int bin_of(float s, float smin, float width, float in
   while (b > 1 && s < bin_edge(b, smin, width)) --b;
   return b;
 }
+// The bins of two scores side by side: the guesses are right but for scores within rounding of an edge, and only those take bin_of.
+__device__ __forceinline__ void bins_of2(float s0, float s1, float smin, float width, float inv_width, int& b0, int& b1) {
+  auto guess = [&](float s) {
+    const float g = fminf(fmaxf((s - smin) * inv_width, 0.f), static_cast<float>(kBins - 1));
+    return static_cast<int>(g);
+  };
+  // (bin 0 has no lower edge, the last bin no upper one; a zero width leaves every score but those below s_min outside its guess)
+  auto off = [&](float s, int b) {
+    const float f = static_cast<float>(b);
+    return (b > 0 && s < __fmaf_rn(f, width, smin)) || (b < kBins - 1 && s >= __fmaf_rn(f + 1.f, width, smin));
+  };
+  b0 = guess(s0);
+  b1 = guess(s1);
+  const bool off0 = off(s0, b0), off1 = off(s1, b1);
+  if (off0) b0 = bin_of(s0, smin, width, inv_width);
+  if (off1) b1 = bin_of(s1, smin, width, inv_width);
+}
 __device__ __forceinline__ int bin_of(float s, float smin, float width) {
   return bin_of(s, smin, width, width > 0.f ? 1.f / width : 0.f);
 }
