@@ -297,9 +297,29 @@ int sm_count() {
   return cached[dev];
 }
 
-int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid) {
+// causal_offset: of the mask under which tiles that no row of a block can see are skipped
+int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causal_offset = INT_MAX) {
   if (tun.segment_tiles > 0) return tun.segment_tiles;
   int n_tiles = (n_keys + kTileKeys - 1) / kTileKeys;
+  constexpr int kItemOverheadTiles = 4;
+  // A triangular mask: blocks see from `first` tiles to all of them, their items are dealt out longest first, and what matters is the
+  // number of items (each starts up) and how evenly they fill the CTAs: whole rows of up to 256 tiles for many blocks.
+  const long long first = (static_cast<long long>(causal_offset) + kRowsPerBlock + kTileKeys - 1) / kTileKeys;
+  if (2 * first < n_tiles && n_blocks >= 2 * grid) {
+    double best_cost = 0.0;
+    int best = 0;
+    for (int s = 256; s >= 16; s >>= 1) {
+      const double lo = first > 0 ? static_cast<double>(first) : 0.0, hi = static_cast<double>(n_tiles);
+      double items = 0.0;  // blocks that reach into each segment, tiles per block growing evenly from lo to hi
+      for (int at = 0; at < n_tiles; at += s) items += n_blocks * (at <= lo ? 1.0 : (hi - at) / (hi - lo));
+      const double cost = kItemOverheadTiles * items / grid + (s < n_tiles ? 0.5 * s : 0.0);
+      if (best == 0 || cost < best_cost) {
+        best_cost = cost;
+        best = s;
+      }
+    }
+    return best;
+  }
   int seg = 256;
   // at least two items per CTA, so that rows of different visible length even out; one per CTA for a chunk of one
   // or two row blocks, whose items all have the same length (measured: 84 instead of 102 us for 1 row over 2^20 keys)
@@ -312,7 +332,6 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid) {
   // Matters for short chunks: 128 rows over 8192 tiles are 512 items of 256 tiles (4 rounds on 148 CTAs, the last
   // one half empty) or 592 items of 222 tiles.  Also for the sample phase, whose 64 tiles x 10 blocks (77 rows) are 40 items
   // of 16 tiles or 130 of 5: one round either way, 29 or 15 us.
-  constexpr int kItemOverheadTiles = 4;
   long long best_cost = -1;
   int best = seg;
   for (int s = seg; s >= 1; --s) {
@@ -449,7 +468,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     p.n_keys = N;
     p.causal_offset = causal_offset;
     p.skip_masked_tiles = 1;  // the select reads visible keys only
-    p.seg_tiles = pick_seg_tiles(tun, N, (T + kRowsPerBlock - 1) / kRowsPerBlock, grid);
+    p.seg_tiles = pick_seg_tiles(tun, N, (T + kRowsPerBlock - 1) / kRowsPerBlock, grid, causal_offset);
     p.topk = topk;
     p.dump = reinterpret_cast<float*>(ws + L.scratch);
     p.dump_ld = L.direct_ld;
@@ -535,7 +554,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     p.n_keys = N;
     p.causal_offset = causal_offset;
     p.skip_masked_tiles = 1;
-    p.seg_tiles = pick_seg_tiles(tun, N, L.n_blocks, grid);
+    p.seg_tiles = abs_form ? pick_seg_tiles(tun, N, L.n_blocks, grid) : pick_seg_tiles(tun, N, L.n_blocks, grid, causal_offset);
     p.topk = topk;
     p.thr = thr;
     p.smin = smin;
