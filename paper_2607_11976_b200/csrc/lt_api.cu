@@ -346,6 +346,16 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causa
   return best;
 }
 
+// Whether a call's kernels open its status block and clear its counters on the way (lt_common.cuh); else launch_zero does ahead of them.
+bool opens_itself(int grid) {
+#if defined(LT_DEBUG_BOUNDS)
+  return false;
+#else
+  return grid <= kStatusSlots;
+#endif
+}
+unsigned char* status_slots(Control* ctl) { return reinterpret_cast<unsigned char*>(ctl + 1); }
+
 // the default scan kernels, or the alternative fp8 scan, behind the same parameter block
 cudaError_t launch_scan(bool abs_form, int dtype, int mode, const void* q, int T, const void* k, long long n_keys_view,
                         long long key_pitch_elems, const ScanParams& p, int grid, cudaStream_t stream) {
@@ -431,14 +441,16 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     return LT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   Control* ctl = reinterpret_cast<Control*>(ws + L.ctl);
-  if (fused) LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
+  const int grid = tun.grid > 0 ? tun.grid : sm_count();
+  const bool own = fused && !abs_form && opens_itself(grid);
+  unsigned char* slots = own ? status_slots(ctl) : nullptr;
+  if (fused && !own) LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
 
   if (!fused) {
     return run_unfused(dtype, false, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score,
                        reinterpret_cast<float*>(ws + L.scratch), L.generic_rows, ctl, tun, stream);
   }
 
-  const int grid = tun.grid > 0 ? tun.grid : sm_count();
   float* smin = reinterpret_cast<float*>(ws + L.smin);
   float* width = reinterpret_cast<float*>(ws + L.width);
   float* thr = reinterpret_cast<float*>(ws + L.thr);
@@ -477,6 +489,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     p.pool_pages = pool_rows / kPageKeys;
     p.debug_flags = tun.debug_flags;
     p.ctl = ctl;
+    p.status_slots = slots;
     LT_LAUNCH(launch_scan_mma(dtype, kModeDump, q, T, k, key_rows, key_pitch, p, grid, stream));
     mark_phase(3, stream);
     SelectRowsParams sp{};
@@ -491,6 +504,8 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     sp.out_score = out_score;
     sp.nan_last = 1;
     sp.ctl = ctl;
+    sp.status_slots = slots;
+    sp.n_slots = grid;
     LT_LAUNCH(launch_select_dense(sp, stream));
     mark_phase(4, stream);
     mark_phase(5, stream);
@@ -535,10 +550,12 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     p.lin_q = lin_q;
     p.lin_scale = lin_scale;
     p.ctl = ctl;
+    p.status_slots = slots;
     LT_LAUNCH(launch_scan(abs_form, dtype, kModeDump, q, T, sample_keys, L.n_sample, sample_pitch, p, grid, stream));
   }
   mark_phase(1, stream);
-  LT_LAUNCH(launch_sample_stats(sample, T, L.n_sample, L.sample_rank, smin, width, thr, stream));
+  const OpenParams open{ctl, slots, L.n_sample > 0 ? grid : 0, tail, hist, row_flag, block_flag, L.rpb};
+  LT_LAUNCH(launch_sample_stats(sample, T, L.n_sample, L.sample_rank, smin, width, thr, own ? &open : nullptr, stream));
   mark_phase(2, stream);
 
   // 2. fused scan: score, gate, compact, count
@@ -960,8 +977,10 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     return LT_ERR_WORKSPACE;
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   Control* ctl = reinterpret_cast<Control*>(ws + L.ctl);
-  LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
   const int grid = tun.grid > 0 ? tun.grid : sm_count();
+  const bool own = opens_itself(grid);
+  unsigned char* slots = own ? status_slots(ctl) : nullptr;
+  if (!own) LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
   if (L.direct) {  // small problem: dense scores and a select over them (see use_direct)
     mark_phase(0, stream);
     mark_phase(1, stream);
@@ -977,6 +996,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     p.dump = reinterpret_cast<float*>(ws + L.scratch);
     p.dump_ld = L.direct_ld;
     p.ctl = ctl;
+    p.status_slots = slots;
     LT_LAUNCH(launch_scan_knn(kModeDump, q, T, x, N, D, p, grid, stream));
     mark_phase(3, stream);
     SelectRowsParams sp{};
@@ -991,6 +1011,8 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     sp.out_score = out_score;
     sp.nan_last = 1;
     sp.ctl = ctl;
+    sp.status_slots = slots;
+    sp.n_slots = grid;
     LT_LAUNCH(launch_select_dense(sp, stream));
     mark_phase(4, stream);
     mark_phase(5, stream);
@@ -1023,10 +1045,12 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     p.dump = sample;
     p.dump_ld = L.n_sample;
     p.ctl = ctl;
+    p.status_slots = slots;
     LT_LAUNCH(launch_scan_knn(kModeDump, q, T, x, L.n_sample, static_cast<long long>(L.sample_stride) * D, p, grid, stream));
   }
   mark_phase(1, stream);
-  LT_LAUNCH(launch_sample_stats(sample, T, L.n_sample, L.sample_rank, smin, width, thr, stream));
+  const OpenParams open{ctl, slots, L.n_sample > 0 ? grid : 0, tail, hist, row_flag, block_flag, L.rpb};
+  LT_LAUNCH(launch_sample_stats(sample, T, L.n_sample, L.sample_rank, smin, width, thr, own ? &open : nullptr, stream));
   mark_phase(2, stream);
 
   // 2. fused scan: one pass over the corpus

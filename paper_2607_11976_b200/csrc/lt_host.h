@@ -131,6 +131,7 @@ struct ScanParams {
   const void* lin_q;       // [T][kLinTerms][128] e4m3 codes
   const float* lin_scale;  // [T][kLinScaleStride], the first kLinTerms entries of a row are used
   Control* ctl;
+  unsigned char* status_slots;  // null: status bits are OR-ed into ctl; else ctl is cleared and every CTA leaves its bits here (lt_common.cuh)
 };
 constexpr int kPageKeys = 64;  // keys per page of a paged key cache
 
@@ -178,6 +179,7 @@ struct KnnScanParams {
   const unsigned int* fb_flag;  // fallback rounds: flag per block of 8 rows; the launch is a no-op if no block of its row range is flagged
   unsigned int wait_limit_us;   // bound of every device-side wait (0 is replaced by the default at launch)
   Control* ctl;
+  unsigned char* status_slots;  // as in ScanParams
 };
 bool scan_knn_supported(int D);
 cudaError_t launch_scan_knn(int mode, const void* q, int T, const void* x, long long n_keys_view, long long key_pitch_elems,
@@ -195,8 +197,19 @@ cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const v
 
 // Sample statistics (paper Sec. 3.2 "Sampling"): per row min / max of the sampled scores, bin
 // width, and the threshold edge of the bin holding the rank-th largest sampled score.
+// open (or null): what the call's later kernels want cleared; the row's CTA does it on the way.
+struct OpenParams {
+  Control* ctl;
+  const unsigned char* status_slots;  // n_slots of them were written by the scan of the sample; 0: there was none, and ctl is cleared here
+  int n_slots;
+  unsigned int* tail;        // [T]
+  unsigned int* hist;        // [T][kBins]
+  unsigned char* row_flag;   // [T]
+  unsigned int* block_flag;  // [ceil(T / rows_per_block)]
+  int rows_per_block;
+};
 cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int rank, float* smin, float* width, float* thr,
-                                cudaStream_t stream);
+                                const OpenParams* open, cudaStream_t stream);
 
 // Final selection from the candidate buffers (paper Sec. 3.2 "Top-k Selection"); rows that cannot
 // be finished exactly are flagged and their block appended to the fallback list.
@@ -234,6 +247,8 @@ struct SelectRowsParams {
   int rows_per_block;
   const unsigned char* row_flag;
   Control* ctl;
+  const unsigned char* status_slots;  // not null: the scan's n_slots status bytes (dense form)
+  int n_slots;
   // NaN scores rank as their bit patterns do, above +inf.  nan_last != 0: they are selected only where a row has too few others,
   // which is what becomes of them in the sampled form (its gate lets none pass; a row that is then short of keys is redone)
   int nan_last;

@@ -204,6 +204,10 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   const uint32_t tmem_base = st->tmem_base;
   volatile int* abort_flag = &st->abort_flag;
   chain_wait();  // barriers, TMEM and tensor maps are ready by now
+  if (kMode == kModeDump && p.status_slots != nullptr) {
+    if (blockIdx.x == 0) clear_control(p.ctl, threadIdx.x);
+    if (threadIdx.x == 0) p.status_slots[blockIdx.x] = 0;
+  }
 
   const int qb_lo = p.row_begin / kQB;
   const int n_qb = (p.row_end - 1) / kQB - qb_lo + 1;
@@ -466,7 +470,13 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   if (st->abort_flag) {
-    if (threadIdx.x == 0) atomicOr(&p.ctl->status, LT_STATUS_TIMEOUT);
+    if (threadIdx.x == 0) {
+      if (p.status_slots != nullptr) {
+        p.status_slots[blockIdx.x] = LT_STATUS_TIMEOUT;
+      } else {
+        atomicOr(&p.ctl->status, LT_STATUS_TIMEOUT);
+      }
+    }
     uint64_t t0 = globaltimer_ns();
     while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
     __syncthreads();

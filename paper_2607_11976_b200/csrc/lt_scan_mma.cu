@@ -309,6 +309,10 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const uint32_t tmem_base = st->tmem_base;
   volatile int* abort_flag = &st->abort_flag;
   chain_wait();  // barriers, TMEM and tensor maps are ready by now
+  if (kMode == kModeDump && p.status_slots != nullptr) {
+    if (blockIdx.x == 0) clear_control(p.ctl, threadIdx.x);
+    if (threadIdx.x == 0) p.status_slots[blockIdx.x] = 0;
+  }
 
   // number of query blocks / items of this launch
   int n_blocks;
@@ -640,7 +644,13 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   tc_fence_before();
   __syncthreads();
   if (st->abort_flag) {
-    if (threadIdx.x == 0) atomicOr(&p.ctl->status, LT_STATUS_TIMEOUT);
+    if (threadIdx.x == 0) {
+      if (p.status_slots != nullptr) {
+        p.status_slots[blockIdx.x] = LT_STATUS_TIMEOUT;
+      } else {
+        atomicOr(&p.ctl->status, LT_STATUS_TIMEOUT);
+      }
+    }
     // give copies and UMMAs still in flight time to land before TMEM and shared memory go away
     uint64_t t0 = globaltimer_ns();
     while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);

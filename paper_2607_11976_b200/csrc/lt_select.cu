@@ -154,7 +154,7 @@ constexpr int kStatsMaxThreads = 1024;
 constexpr int kStatsBatch = 8;   // loads in flight per thread, first sweep
 __global__ void __launch_bounds__(kStatsMaxThreads) sample_stats_kernel(const float* __restrict__ sample, int n_sample, int rank,
                                                                      float* __restrict__ smin_out, float* __restrict__ width_out,
-                                                                     float* __restrict__ thr_out) {
+                                                                     float* __restrict__ thr_out, const OpenParams open) {
   constexpr int kMaxWarps = kStatsMaxThreads / 32;
   const int n_threads = blockDim.x, n_warps = n_threads >> 5;
   __shared__ unsigned int red_min[kMaxWarps], red_max[kMaxWarps];
@@ -163,6 +163,16 @@ __global__ void __launch_bounds__(kStatsMaxThreads) sample_stats_kernel(const fl
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* row = sample + static_cast<size_t>(t) * n_sample;
   chain_wait();
+  const int slot = load_status_slot(open.status_slots, open.n_slots, tid);
+  if (open.ctl != nullptr) {
+    for (int i = tid; i < kBins; i += n_threads) open.hist[static_cast<size_t>(t) * kBins + i] = 0u;
+    if (tid == 0) {
+      open.tail[t] = 0u;
+      open.row_flag[t] = 0;
+      if (t % open.rows_per_block == 0) open.block_flag[t / open.rows_per_block] = 0u;
+    }
+    if (open.n_slots == 0 && t == 0) clear_control(open.ctl, tid);
+  }
   // minimum and maximum in ordered bit patterns (integer warp reductions)
   unsigned int mn = 0xffffffffu, mx = 0u;
   for (int base = tid; base < n_sample; base += n_threads * kStatsBatch) {
@@ -177,6 +187,7 @@ __global__ void __launch_bounds__(kStatsMaxThreads) sample_stats_kernel(const fl
       mx = max(mx, k);
     }
   }
+  add_status(open.ctl, slot);
   mn = __reduce_min_sync(0xffffffffu, mn);
   mx = __reduce_max_sync(0xffffffffu, mx);
   if (lane == 0) {
@@ -735,6 +746,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
   uint64_t* sel = sel_smem + kFineBins * 4 / 8;
   int t;
   chain_wait();
+  const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x);
   if (p.fb_list != nullptr) {
     int j = p.fb_round_base + blockIdx.x / p.rows_per_block;
     if (j >= *p.fb_blocks) return;
@@ -752,6 +764,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
   const int tid = threadIdx.x;
 
   if (vis == 0) {
+    add_status(p.ctl, slot);
     sort_and_write(sel, 0, p.topk, out_idx, out_score, p.N, p.ctl);
     return;
   }
@@ -762,12 +775,14 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
       const int i = j * kThreads + tid;
       if (i < vis) first[j] = make_uint2(__float_as_uint(row[i]), static_cast<unsigned int>(i));
     }
+    add_status(p.ctl, slot);
     if (fine_select_sort<kThreads>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
                                       static_cast<unsigned int>(vis), kk, p.topk, sel, 2u * p.sel_slots, bins, out_idx, out_score,
                                       p.N, p.ctl, p.nan_last != 0 && vis > p.topk))
       return;
   }
   if (vis <= p.topk) {
+    if (vis > kSelDirect) add_status(p.ctl, slot);
     // every visible key is selected, and they did not spread over the bins
     for (int i = tid; i < vis; i += kThreads) sel[i] = pack_key(row[i], i);
     __syncthreads();
@@ -775,6 +790,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
     return;
   }
 
+  if (vis > kSelDirect) add_status(p.ctl, slot);
   radix_select_row<kThreads>(row, vis, kk, sel, p.nan_last != 0);
   __syncthreads();
   auto winner = [&](unsigned int i) { return make_uint2(key_to_score_bits(static_cast<unsigned int>(sel[i] >> 32)), static_cast<unsigned int>(key_index(sel[i]))); };
@@ -878,7 +894,9 @@ __global__ void __launch_bounds__(kClThreads, kPerSm) select_cluster_kernel(cons
   int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
   float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
   chain_wait();
+  const int slot = load_status_slot(p.status_slots, p.n_slots, tid);
   if (kk == 0) {  // the whole cluster
+    add_status(p.ctl, slot);
     if (rank == 0) sort_and_write(list, 0, p.topk, out_idx, out_score, p.N, p.ctl);
     return;
   }
@@ -928,6 +946,7 @@ __global__ void __launch_bounds__(kClThreads, kPerSm) select_cluster_kernel(cons
     vmin = fminf(vmin, fminf(fminf(m.x, m.y), fminf(m.z, m.w)));
     vmax = fmaxf(vmax, fmaxf(fmaxf(m.x, m.y), fmaxf(m.z, m.w)));
   });
+  add_status(p.ctl, slot);
   if (tid == 0) s_fill = 0u;
 
   float scale = 0.f, limit = 0.f;
@@ -1156,10 +1175,11 @@ cudaError_t launch_simt_scores(int dtype, const void* q, const float* w, const v
 }
 
 cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int rank, float* smin, float* width, float* thr,
-                                cudaStream_t stream) {
+                                const OpenParams* open, cudaStream_t stream) {
   // few rows leave the chip idle: a large CTA then shortens the sweeps; with many rows small CTAs overlap better
   const int threads = T <= 296 ? 1024 : 256;
-  return launch_chained(sample_stats_kernel, T, threads, 0, stream, 1, sample, n_sample, rank, smin, width, thr);
+  return launch_chained(sample_stats_kernel, T, threads, 0, stream, 1, sample, n_sample, rank, smin, width, thr,
+                        open != nullptr ? *open : OpenParams{});
 }
 
 cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream) {
