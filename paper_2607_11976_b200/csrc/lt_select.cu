@@ -740,23 +740,10 @@ __device__ __forceinline__ void radix_select_row(const float* row, int vis, int 
 // indices first), and a sort of the k winners.
 // ---------------------------------------------------------------------------------------------
 template <int kThreads>
-__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const SelectRowsParams p) {
+__device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t, const float* row, int slot) {
   extern __shared__ __align__(16) uint64_t sel_smem[];  // the distribution sort's bins, then two buffers of p.sel_slots keys
   unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
   uint64_t* sel = sel_smem + kFineBins * 4 / 8;
-  int t;
-  chain_wait();
-  const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x);
-  if (p.fb_list != nullptr) {
-    int j = p.fb_round_base + blockIdx.x / p.rows_per_block;
-    if (j >= *p.fb_blocks) return;
-    t = p.fb_list[j] * p.rows_per_block + blockIdx.x % p.rows_per_block;
-    if (t >= p.T || !p.row_flag[t]) return;
-  } else {
-    t = p.row_begin + blockIdx.x;
-    if (p.row_flag != nullptr && !p.row_flag[t]) return;  // only flagged rows are redone
-  }
-  const float* row = p.scores + static_cast<size_t>(blockIdx.x) * p.ld;
   const int vis = visible_keys(t, p.N, p.causal_offset);
   const int kk = p.topk < vis ? p.topk : vis;
   int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
@@ -801,6 +788,27 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
                                  out_idx, out_score, p.N, p.ctl))
     return;
   sort_and_write(sel, kk, p.topk, out_idx, out_score, p.N, p.ctl);
+}
+
+// kFlagged: the rows that row_flag marks (the exact fallback).  They are few or none, and only the device knows: a grid of at most
+// kFlaggedCtas goes through all of them.  (A CTA per
+// row took 21 us, with the scan ahead of it, to find nothing to do among 4096 rows and 39 us, in two rounds, among 8192; now 9 and 12.)
+constexpr int kFlaggedCtas = 296;
+template <int kThreads, bool kFlagged>
+__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const SelectRowsParams p) {
+  chain_wait();
+  if (!kFlagged) {  // a CTA for every row
+    const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x);
+    select_one_row<kThreads>(p, p.row_begin + blockIdx.x, p.scores + static_cast<size_t>(blockIdx.x) * p.ld, slot);
+    return;
+  }
+  const int n = p.fb_list != nullptr ? min(p.n_blocks, (*p.fb_blocks - p.fb_round_base) * p.rows_per_block) : p.n_blocks;
+  for (int b = blockIdx.x; b < n; b += gridDim.x) {
+    const int t = p.fb_list != nullptr ? p.fb_list[p.fb_round_base + b / p.rows_per_block] * p.rows_per_block + b % p.rows_per_block : p.row_begin + b;
+    if (t >= p.T || !p.row_flag[t]) continue;
+    __syncthreads();  // the row before is done with the shared memory
+    select_one_row<kThreads>(p, t, p.scores + static_cast<size_t>(b) * p.ld, 0);
+  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1219,12 +1227,13 @@ cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t str
 }
 
 namespace {
-template <int kThreads>
+template <int kThreads, bool kFlagged>
 cudaError_t launch_select_rows_n(const SelectRowsParams& p, int smem, cudaStream_t stream) {
   static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_rows_kernel<kThreads>), done);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_rows_kernel<kThreads, kFlagged>), done);
   if (e != cudaSuccess) return e;
-  return launch_chained(select_rows_kernel<kThreads>, p.n_blocks, kThreads, smem, stream, 1, p);
+  const int ctas = kFlagged && p.n_blocks > kFlaggedCtas ? kFlaggedCtas : p.n_blocks;
+  return launch_chained(select_rows_kernel<kThreads, kFlagged>, ctas, kThreads, smem, stream, 1, p);
 }
 }  // namespace
 
@@ -1234,8 +1243,9 @@ cudaError_t launch_select_rows(const SelectRowsParams& params, cudaStream_t stre
   p.sel_slots = static_cast<unsigned int>(next_pow2(p.topk < 2048 ? 2048 : p.topk));
   const int smem = kFineBins * 4 + 2 * static_cast<int>(p.sel_slots) * static_cast<int>(sizeof(uint64_t));
   // many short rows: three small CTAs an SM hide one another's barriers; otherwise a row gets all the threads it can use
-  if (p.fb_list == nullptr && p.n_blocks > 296 && p.N <= kSelDirect) return launch_select_rows_n<512>(p, smem, stream);
-  return launch_select_rows_n<1024>(p, smem, stream);
+  if (p.row_flag != nullptr) return launch_select_rows_n<1024, true>(p, smem, stream);
+  if (p.n_blocks > 296 && p.N <= kSelDirect) return launch_select_rows_n<512, false>(p, smem, stream);
+  return launch_select_rows_n<1024, false>(p, smem, stream);
 }
 
 }  // namespace lt
