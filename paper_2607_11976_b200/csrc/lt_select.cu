@@ -392,9 +392,8 @@ __device__ __forceinline__ void keep_top_keys(uint64_t* sel, int count, int keep
 // every candidate at or above its lower edge is pulled into shared memory (the bins above hold fewer than k of
 // them), cut to k by a radix select, sorted, and written out.
 // ---------------------------------------------------------------------------------------------
-constexpr int kFinalThreads = 512;
-
-__global__ void __launch_bounds__(kFinalThreads, 3) final_select_kernel(const FinalSelectParams p, int sel_cap) {
+template <int kFinalThreads>
+__global__ void __launch_bounds__(kFinalThreads, kFinalThreads == 512 ? 3 : 1) final_select_kernel(const FinalSelectParams p, int sel_cap) {
   extern __shared__ __align__(16) uint64_t sel[];  // sel_cap keys; the distribution sort's bins are the last of them
   __shared__ unsigned int hist[kBins];
   __shared__ int s_tb;
@@ -1241,10 +1240,14 @@ cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream)
   if (sel_cap < 8192) sel_cap = 8192;
   if (sel_cap > kSelCap) sel_cap = kSelCap;
   const int smem = sel_cap * static_cast<int>(sizeof(uint64_t));
-  static std::atomic<unsigned long long> done{0};
-  cudaError_t e = allow_smem(reinterpret_cast<const void*>(final_select_kernel), done);
+  // a row to an SM gets all the threads it can use (4 rows of 6.4 k candidates 16.4 -> 10.2 us, 77 of 3.5 k 14.3 -> 10.2); more rows share
+  // SMs, and small CTAs hide one another's barriers
+  static std::atomic<unsigned long long> done[2];
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(final_select_kernel<512>), done[0]);
+  if (e == cudaSuccess) e = allow_smem(reinterpret_cast<const void*>(final_select_kernel<1024>), done[1]);
   if (e != cudaSuccess) return e;
-  return launch_chained(final_select_kernel, p.T, kFinalThreads, smem, stream, 1, p, sel_cap);
+  if (p.T <= 148) return launch_chained(final_select_kernel<1024>, p.T, 1024, smem, stream, 1, p, sel_cap);
+  return launch_chained(final_select_kernel<512>, p.T, 512, smem, stream, 1, p, sel_cap);
 }
 
 cudaError_t launch_select_dense(const SelectRowsParams& params, cudaStream_t stream) {
