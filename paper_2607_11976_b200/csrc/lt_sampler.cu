@@ -35,39 +35,70 @@ __global__ void __launch_bounds__(256) count_positions_kernel(const int32_t* __r
 // ---- ranking the counts: top n_out of the N distinct keys (count, position) ---------------------------------------
 // A key packs the count above the complemented position, (count << pos_bits) | (2^pos_bits - 1 - position), so that
 // larger keys mean (count descending, position ascending) and only count_bits + pos_bits bits carry information.
-// A grid-wide MSB radix select, one launch per 8-bit digit of those bits: every CTA histograms the digit of the
+// A grid-wide MSB radix select, one launch per 11-bit digit of those bits: every CTA histograms the digit of the
 // keys that still match the prefix found so far (per-thread run-length aggregation: neighbouring positions mostly
-// share the digit), adds its 256 counters to the global histogram, and the last CTA to finish picks the digit in
+// share the digit), adds its counters to the global histogram, and the last CTA to finish picks the digit in
 // which the count from the top reaches the number of keys still wanted.  The keys are distinct (the position is
-// part of them), so after the last digit the prefix IS the n_out-th largest key and no tie needs ranking.
+// part of them), so after the last digit the prefix IS the n_out-th largest key and no tie needs ranking.  A pass over a few MB is a
+// chain of latencies (loads, merge, pick), so there are as few passes as shared memory counts cheaply, and the pick is a
+// prefix sum by the whole CTA.  Whole call, 1024 x 2048
+// entries over 262,144 positions, 6144 wanted, 76 -> 48 us; 512 x 512 over 1,000,003, 1536 wanted, 66 -> 35 (8-bit digits, picked by one
+// thread, and two launches for the order).
+constexpr int kRankBits = 11;
+constexpr int kRankDigits = 1 << kRankBits;
+constexpr int kRankThreads = 512;
+constexpr int kOrderKeys = 256;  // keys ranked by one CTA
 struct RankState {
-  unsigned int hist[256];
   unsigned long long prefix;
   unsigned int remaining;
   unsigned int done;
   unsigned int n_written;
-  unsigned int pad[3];
+  unsigned int slices_done[(LT_MAX_TOPK + kOrderKeys - 1) / kOrderKeys];
 };
+// Scratch: the state, then the passes' histogram, over which the keys are written once the passes are through, then the keys' ranks.
+constexpr size_t kRankStateBytes = 1280;
+constexpr size_t kRankHistBytes = kRankDigits * 4;
+static_assert(sizeof(RankState) <= kRankStateBytes, "state block");
+__host__ __device__ inline unsigned int* rank_hist(RankState* st) { return reinterpret_cast<unsigned int*>(reinterpret_cast<uint8_t*>(st) + kRankStateBytes); }
+size_t rank_keys_bytes(int n_out) { return static_cast<size_t>(n_out) * 8 > kRankHistBytes ? static_cast<size_t>(n_out) * 8 : kRankHistBytes; }
 
 constexpr int kRankBatch = 8;  // loads a thread keeps in flight (one CTA-wide load per batch entry)
 
 __device__ __forceinline__ unsigned long long rank_key(unsigned int count, unsigned int pos, int pos_bits) {
   return (static_cast<unsigned long long>(count) << pos_bits) | ((1ull << pos_bits) - 1ull - pos);
 }
+// inclusive prefix sum over the CTA (kRankThreads threads); the barrier inside separates what precedes it from what follows
+__device__ __forceinline__ unsigned int cta_inclusive_sum(unsigned int v, unsigned int* warp_sum) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned int incl = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned int o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) warp_sum[warp] = incl;
+  __syncthreads();
+  return incl + __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum[lane] : 0u);
+}
 
-__global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __restrict__ counts, int N, RankState* st, int shift,
-                                                         int first_pass, int pos_bits, int want) {
-  __shared__ unsigned int hist[256];
+__global__ void __launch_bounds__(kRankThreads) rank_pass_kernel(const unsigned int* __restrict__ counts, int N, RankState* st, int shift,
+                                                                 int first_pass, int pos_bits, int want) {
+  __shared__ __align__(16) unsigned int hist[kRankDigits];
+  __shared__ unsigned int warp_sum[kRankThreads / 32];
   __shared__ bool last;
-  const unsigned long long mask = first_pass ? 0ull : (~0ull << (shift + 8));
+  constexpr int kPer = kRankDigits / kRankThreads;
+  static_assert(kPer == 4, "a thread's digits are one 16-byte piece");
+  const int tid = threadIdx.x;
+  const unsigned long long mask = first_pass ? 0ull : (~0ull << (shift + kRankBits));
+  unsigned int* const total = rank_hist(st);
+  reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u);
   chain_wait();
   const unsigned long long prefix = st->prefix;
-  hist[threadIdx.x] = 0;
   __syncthreads();
-  unsigned int run_digit = 0x100u, run_len = 0;
+  unsigned int run_digit = kRankDigits, run_len = 0;
   // each CTA walks one contiguous range of positions with coalesced loads, kRankBatch of them in flight per
   // thread (one load at a time is latency-bound: 16 dependent DRAM round trips per pass); a thread's consecutive
-  // keys are 256 positions apart, which still share their leading digits (the count's high bytes)
+  // keys are a CTA's width apart, which still share their leading digits (the count's high bits)
   const int per_thread = (N + gridDim.x * blockDim.x - 1) / (gridDim.x * blockDim.x);
   const long long first = static_cast<long long>(blockIdx.x) * blockDim.x * per_thread + threadIdx.x;
   for (int j0 = 0; j0 < per_thread; j0 += kRankBatch) {
@@ -83,7 +114,7 @@ __global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __re
       if (j0 + u >= per_thread || i >= N) continue;
       const unsigned long long key = rank_key(c[u], static_cast<unsigned int>(i), pos_bits);
       if ((key & mask) != prefix) continue;
-      const unsigned int digit = static_cast<unsigned int>(key >> shift) & 255u;
+      const unsigned int digit = static_cast<unsigned int>(key >> shift) & (kRankDigits - 1u);
       if (digit == run_digit) {
         ++run_len;
       } else {
@@ -95,43 +126,47 @@ __global__ void __launch_bounds__(256) rank_pass_kernel(const unsigned int* __re
   }
   if (run_len > 0) atomicAdd(&hist[run_digit], run_len);
   __syncthreads();
-  if (hist[threadIdx.x] != 0) atomicAdd(&st->hist[threadIdx.x], hist[threadIdx.x]);
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    const unsigned int n = hist[tid + j * kRankThreads];
+    if (n != 0u) atomicAdd(total + tid + j * kRankThreads, n);
+  }
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
+  if (tid == 0) last = atomicAdd(&st->done, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();
-  // the complete histogram comes back with one load per thread (a single thread walking it in global memory
-  // would pay 256 dependent L2 round trips)
-  hist[threadIdx.x] = __ldcg(&st->hist[threadIdx.x]);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned int remaining = first_pass ? static_cast<unsigned int>(want) : st->remaining;
-    unsigned int cum = 0;
-    int digit = 0;
-    for (int d = 255; d >= 0; --d) {
-      const unsigned int c = hist[d];
-      if (cum + c >= remaining) {
-        digit = d;
-        break;
-      }
-      cum += c;
+  // digits from the top down, four per thread: the one in which the count reaches what is still wanted
+  const int low = kRankDigits - kPer * (tid + 1);  // this thread's lowest digit
+  const uint4 h = __ldcg(reinterpret_cast<const uint4*>(total + low));
+  const unsigned int remaining = first_pass ? static_cast<unsigned int>(want) : st->remaining;
+  const unsigned int mine = h.x + h.y + h.z + h.w;
+  const unsigned int incl = cta_inclusive_sum(mine, warp_sum);
+  unsigned int cum = incl - mine;
+  if (cum < remaining && incl >= remaining) {  // exactly one thread: there are N >= want keys
+    const unsigned int c[kPer] = {h.w, h.z, h.y, h.x};
+    int digit = -1;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      if (digit < 0 && cum + c[j] >= remaining) digit = low + kPer - 1 - j;
+      if (digit < 0) cum += c[j];
     }
     st->remaining = remaining - cum;
     st->prefix = prefix | (static_cast<unsigned long long>(digit) << shift);
     st->done = 0;
   }
-  __syncthreads();
-  st->hist[threadIdx.x] = 0;
+  *reinterpret_cast<uint4*>(total + low) = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// every key at or above the n_out-th largest goes to the list (any order; exactly n_out of them)
-__global__ void __launch_bounds__(256) rank_collect_kernel(const unsigned int* __restrict__ counts, int N, RankState* st,
-                                                            unsigned long long* __restrict__ keys, int n_out, int pos_bits) {
+// every key at or above the n_out-th largest goes to the list (any order; exactly n_out of them): places are reserved once for each CTA
+// and round of kRankBatch keys per thread (a reservation per warp and key, all on one address, took twice as long)
+__global__ void __launch_bounds__(kRankThreads) rank_collect_kernel(const unsigned int* __restrict__ counts, int N, RankState* st,
+                                                                    unsigned long long* __restrict__ keys, int n_out, int pos_bits) {
+  __shared__ unsigned int warp_sum[kRankThreads / 32];
+  __shared__ unsigned int s_base;
   chain_wait();
   const unsigned long long kth = st->prefix;
-  const int lane = threadIdx.x & 31;
   const int per_thread = (N + gridDim.x * blockDim.x - 1) / (gridDim.x * blockDim.x);
   const long long first = static_cast<long long>(blockIdx.x) * blockDim.x * per_thread + threadIdx.x;
   for (int j0 = 0; j0 < per_thread; j0 += kRankBatch) {
@@ -141,61 +176,64 @@ __global__ void __launch_bounds__(256) rank_collect_kernel(const unsigned int* _
       const long long i = first + static_cast<long long>(j0 + u) * blockDim.x;
       c[u] = (j0 + u < per_thread && i < N) ? __ldg(counts + i) : 0u;
     }
+    unsigned int take = 0;
 #pragma unroll
     for (int u = 0; u < kRankBatch; ++u) {
       const long long i = first + static_cast<long long>(j0 + u) * blockDim.x;
-      unsigned long long key = 0;
-      bool take = false;
-      if (j0 + u < per_thread && i < N) {
-        key = rank_key(c[u], static_cast<unsigned int>(i), pos_bits);
-        take = key >= kth;
-      }
-      const unsigned int ballot = __ballot_sync(0xffffffffu, take);
-      if (ballot != 0) {
-        unsigned int base = 0;
-        if (lane == 0) base = atomicAdd(&st->n_written, static_cast<unsigned int>(__popc(ballot)));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        const unsigned int pos = base + __popc(ballot & ((1u << lane) - 1u));
-        if (take && pos < static_cast<unsigned int>(n_out)) keys[pos] = key;
+      if (j0 + u < per_thread && i < N && rank_key(c[u], static_cast<unsigned int>(i), pos_bits) >= kth) take |= 1u << u;
+    }
+    const unsigned int mine = __popc(take);
+    const unsigned int incl = cta_inclusive_sum(mine, warp_sum);
+    if (threadIdx.x == kRankThreads - 1) s_base = incl != 0u ? atomicAdd(&st->n_written, incl) : 0u;
+    __syncthreads();
+    unsigned int pos = s_base + incl - mine;
+#pragma unroll
+    for (int u = 0; u < kRankBatch; ++u) {
+      const long long i = first + static_cast<long long>(j0 + u) * blockDim.x;
+      if ((take >> u) & 1u) {
+        if (pos < static_cast<unsigned int>(n_out)) keys[pos] = rank_key(c[u], static_cast<unsigned int>(i), pos_bits);
+        ++pos;
       }
     }
+    __syncthreads();  // the sums have been read
   }
 }
 
 // Order of the n_out winners (count descending, position ascending) by counting: the keys are distinct, so the
-// number of larger keys IS a key's place in the output.  CTA (x, y) ranks 256 keys against slice y of the list
-// held in shared memory; the slices' partial ranks meet in `rank` (zeroed by the caller).  n_out^2 comparisons
-// spread over the whole GPU take a few microseconds where a one-CTA sort of the list took 80.
-constexpr int kOrderSlice = 1024;
+// number of larger keys IS a key's place in the output.  CTA (x, y) ranks kOrderKeys keys against slice y of the list
+// held in shared memory; the slices' partial ranks meet in `rank` (zeroed by the caller), and the last CTA of a block of keys writes them
+// out.  n_out^2 comparisons spread over the whole GPU take a few microseconds where a one-CTA sort of the list took 80; slices of 256 keys
+// fill it from a few thousand keys on.
+constexpr int kOrderSlice = 256;
 
-__global__ void __launch_bounds__(256) rank_count_larger_kernel(const unsigned long long* __restrict__ keys, int n_out,
-                                                                 unsigned int* __restrict__ rank) {
-  __shared__ unsigned long long slice[kOrderSlice];
+__global__ void __launch_bounds__(kOrderKeys) rank_order_kernel(const unsigned long long* __restrict__ keys, int n_out, RankState* st,
+                                                                unsigned int* __restrict__ rank, int pos_bits, int32_t* __restrict__ out_pos,
+                                                                int32_t* __restrict__ out_count) {
+  __shared__ __align__(16) unsigned long long slice[kOrderSlice];
+  __shared__ bool last;
+  static_assert(kOrderSlice == kOrderKeys, "a thread fetches one key of the slice");
   chain_wait();
-  const int s0 = blockIdx.y * kOrderSlice;
-  const int len = min(kOrderSlice, n_out - s0);
-  for (int i = threadIdx.x; i < len; i += blockDim.x) slice[i] = keys[s0 + i];
+  const int me = blockIdx.x * kOrderKeys + threadIdx.x, other = blockIdx.y * kOrderSlice + threadIdx.x;
+  const unsigned long long mine = me < n_out ? keys[me] : ~0ull;
+  slice[threadIdx.x] = other < n_out ? keys[other] : 0ull;  // (zero is larger than nothing)
   __syncthreads();
-  const int me = blockIdx.x * blockDim.x + threadIdx.x;
-  if (me >= n_out) return;
-  const unsigned long long mine = keys[me];
   unsigned int larger = 0;
-#pragma unroll 8
-  for (int i = 0; i < len; ++i) larger += slice[i] > mine ? 1u : 0u;
-  if (larger != 0) atomicAdd(rank + me, larger);
-}
-
-__global__ void __launch_bounds__(256) rank_write_kernel(const unsigned long long* __restrict__ keys, int n_out,
-                                                          const unsigned int* __restrict__ rank, int pos_bits,
-                                                          int32_t* __restrict__ out_pos, int32_t* __restrict__ out_count) {
-  chain_wait();
-  const int me = blockIdx.x * blockDim.x + threadIdx.x;
-  if (me >= n_out) return;
-  const unsigned long long key = keys[me];
-  const unsigned int r = rank[me];
+#pragma unroll 16
+  for (int i = 0; i < kOrderSlice; i += 2) {
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(slice + i);
+    larger += (v.x > mine ? 1u : 0u) + (v.y > mine ? 1u : 0u);
+  }
+  if (larger != 0u) atomicAdd(rank + me, larger);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(&st->slices_done[blockIdx.x], 1u) == gridDim.y - 1;
+  __syncthreads();
+  if (!last || me >= n_out) return;
+  __threadfence();
+  const unsigned int r = __ldcg(rank + me);
   if (r >= static_cast<unsigned int>(n_out)) return;  // cannot happen for distinct keys
-  out_pos[r] = static_cast<int32_t>((1ull << pos_bits) - 1ull - (key & ((1ull << pos_bits) - 1ull)));
-  if (out_count != nullptr) out_count[r] = static_cast<int32_t>(key >> pos_bits);
+  out_pos[r] = static_cast<int32_t>((1ull << pos_bits) - 1ull - (mine & ((1ull << pos_bits) - 1ull)));
+  if (out_count != nullptr) out_count[r] = static_cast<int32_t>(mine >> pos_bits);
 }
 
 // out_k[j] = key row at position sample_idx[j] (or j * stride when no list is given), row_bytes bytes (a
@@ -234,7 +272,8 @@ cudaError_t launch_count_positions(const int32_t* idx, long long n, int N, unsig
   return launch_chained(count_positions_kernel, static_cast<unsigned int>(blocks), 256, 0, stream, 1, idx, n, N, counts);
 }
 
-size_t rank_scratch_bytes(int n_out) { return 1280 + static_cast<size_t>(n_out) * 12; }
+// (for LT_MAX_TOPK keys, which every workspace is sized for, what it was with a smaller histogram inside the state)
+size_t rank_scratch_bytes(int n_out) { return kRankStateBytes + rank_keys_bytes(n_out) + static_cast<size_t>(n_out) * 4; }
 
 namespace {
 int bits_for(unsigned long long max_value) {
@@ -248,25 +287,22 @@ int bits_for(unsigned long long max_value) {
 // 256-byte aligned.  max_count: an upper bound of any count (it fixes how many digits the select has to visit).
 cudaError_t launch_rank_counts(const unsigned int* counts, int N, int n_out, unsigned long long max_count, void* scratch,
                                int32_t* out_pos, int32_t* out_count, cudaStream_t stream) {
-  static_assert(sizeof(RankState) <= 1088, "state block");
   RankState* st = static_cast<RankState*>(scratch);
-  unsigned long long* keys = reinterpret_cast<unsigned long long*>(static_cast<uint8_t*>(scratch) + 1280);
-  unsigned int* rank = reinterpret_cast<unsigned int*>(keys + n_out);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(rank_hist(st));
+  unsigned int* rank = reinterpret_cast<unsigned int*>(reinterpret_cast<uint8_t*>(keys) + rank_keys_bytes(n_out));
   if (max_count > 0xffffffffull) max_count = 0xffffffffull;
   const int pos_bits = bits_for(static_cast<unsigned long long>(N - 1));
-  const int passes = (bits_for(max_count) + pos_bits + 7) / 8;
-  int blocks = (N + 256 * kRankBatch - 1) / (256 * kRankBatch);
+  const int passes = (bits_for(max_count) + pos_bits + kRankBits - 1) / kRankBits;
+  int blocks = (N + kRankThreads * kRankBatch - 1) / (kRankThreads * kRankBatch);
   if (blocks < 1) blocks = 1;
-  if (blocks > 148 * 4) blocks = 148 * 4;
+  if (blocks > 148 * 2) blocks = 148 * 2;
   cudaError_t e = cudaSuccess;
   for (int pass = 0; pass < passes && e == cudaSuccess; ++pass)
-    e = launch_chained(rank_pass_kernel, blocks, 256, 0, stream, 1, counts, N, st, 8 * (passes - 1 - pass), pass == 0 ? 1 : 0, pos_bits, n_out);
-  if (e == cudaSuccess) e = launch_chained(rank_collect_kernel, blocks, 256, 0, stream, 1, counts, N, st, keys, n_out, pos_bits);
-  const int key_blocks = (n_out + 255) / 256;
+    e = launch_chained(rank_pass_kernel, blocks, kRankThreads, 0, stream, 1, counts, N, st, kRankBits * (passes - 1 - pass), pass == 0 ? 1 : 0, pos_bits, n_out);
+  if (e == cudaSuccess) e = launch_chained(rank_collect_kernel, blocks, kRankThreads, 0, stream, 1, counts, N, st, keys, n_out, pos_bits);
   if (e == cudaSuccess)
-    e = launch_chained(rank_count_larger_kernel, dim3(key_blocks, (n_out + kOrderSlice - 1) / kOrderSlice), 256, 0, stream, 1, keys, n_out, rank);
-  if (e == cudaSuccess)
-    e = launch_chained(rank_write_kernel, key_blocks, 256, 0, stream, 1, keys, n_out, rank, pos_bits, out_pos, out_count);
+    e = launch_chained(rank_order_kernel, dim3((n_out + kOrderKeys - 1) / kOrderKeys, (n_out + kOrderSlice - 1) / kOrderSlice), kOrderKeys, 0, stream, 1,
+                       keys, n_out, st, rank, pos_bits, out_pos, out_count);
   return e;
 }
 
