@@ -6,10 +6,13 @@ namespace lt {
 constexpr int kSelDirect = 16384;  // rows up to this length are selected by one CTA (a few batches of registers)
 
 // CTAs that share a row of n_keys > kSelDirect keys: as many as the row is long, no more than `widest`, the widest cluster the device
-// can place.  Clusters of 16 need a whole GPC, and are asked for only while few are wanted.
+// can place.  While few CTAs are wanted a share is half as long (1 x 20 K keys, whole call, width 2 / 4: 18.1 / 16.7 us; 7 x 40 K, 4 / 8: 24.0 /
+// 22.9), but not beyond clusters of 8 (1 x 128 K, 8 / 16: 22.2 / 22.6).  Clusters of 16 need a whole GPC, and are asked for only while few are wanted.
+constexpr int kSelFewCtas = 32;
 inline int select_cluster_width(int n_keys, int n_rows, int widest) {
   int width = 2;
-  while (width < 16 && static_cast<long long>(width) * kSelDirect < n_keys) width <<= 1;
+  auto share = [&](int w) { return w < 8 && static_cast<long long>(n_rows) * w <= kSelFewCtas ? kSelDirect / 2 : kSelDirect; };
+  while (width < 16 && static_cast<long long>(width) * share(width) < n_keys) width <<= 1;
   if (width > 8 && static_cast<long long>(n_rows) * width > 128) width = 8;
   return width < widest ? width : widest;
 }
