@@ -62,11 +62,14 @@ __device__ __forceinline__ bool lt_in_bounds(bool cond, Control* ctl) {
 // memory flush.  chain_wait() returns once everything ahead in the stream has completed and its writes are visible.
 // EVERY thread of every kernel launched that way that touches global memory calls chain_wait() before it does, on every
 // path: a grid that ended without waiting would let the kernel behind it run ahead of the kernel before it.
-// No kernel lets its successor start earlier than that (griddepcontrol.launch_dependents): tried at the top of every
-// kernel, it slowed what ran beside the waiting grid, 4096 rows over 2^20 keys 40.0 -> 42.5 ms, 4 rows 73 -> 80 us, 77 rows
-// over 300 K keys 238 -> 248 us.
+// Only the scans of the exact fallback let their successor start earlier than that (chain_trigger): nearly always they have nothing to do,
+// and neither has the select behind them (4 rows over 2^20 keys 67.5 -> 64.9 us, 1 row 48.0 -> 45.3).  At the top of every kernel the
+// trigger slowed what ran beside the waiting grid, 4096 rows over 2^20 keys 40.0 -> 42.5 ms, 4 rows 73 -> 80 us, 77 rows over 300 K keys
+// 238 -> 248 us.  A kernel triggers behind its own chain_wait(), so that what its successor waits for is all that is ahead of it.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel of the stream start already.
+__device__ __forceinline__ void chain_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------------------------
 // total order on (score, index): larger key = better.  Scores are canonicalised (-0 -> +0)

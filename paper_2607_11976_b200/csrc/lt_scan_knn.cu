@@ -170,6 +170,7 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // (uniform across the grid)
   if (p.fb_flag != nullptr) {
     chain_wait();
+    chain_trigger();
     unsigned int any = 0u;
     for (int b = p.row_begin / kRowsPerBlock; b * kRowsPerBlock < p.row_end; ++b) any |= p.fb_flag[b];
     if (any == 0u) return;

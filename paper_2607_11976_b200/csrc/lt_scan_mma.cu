@@ -277,6 +277,7 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   // a fallback round with no flagged block left has nothing to do (uniform across the CTA)
   if (p.fb_list != nullptr) {
     chain_wait();
+    chain_trigger();
     if (*p.fb_blocks <= p.fb_round_base) return;
   }
 
