@@ -25,9 +25,9 @@ struct Control {
 };
 
 // The status block opens without a launch of its own: the call's first scan clears it and leaves each CTA's status bits in a byte of its
-// own behind it, and the kernel after that, a byte per thread of its first CTA, adds them to the status word.  (A kernel that only cleared the block and the counters cost a 1-row call 0.9 of 22.9 us, a first chunk of 4096 rows 2 of 184.)  In the
-// bounds-checking build, whose checks write the status word from every kernel, and with more CTAs than bytes, everything
-// is cleared ahead of the call.
+// own behind it, and the kernel after that, a byte per thread of its first CTA, adds them to the status word.  (A kernel that only
+// cleared the block and the counters cost a 1-row call 0.9 of 22.9 us, a first chunk of 4096 rows 2 of 184.)  In the bounds-checking
+// build, whose checks write the status word from every kernel, and with more CTAs than bytes, everything is cleared ahead of the call.
 constexpr int kStatusSlots = 256 - static_cast<int>(sizeof(Control));  // what the block leaves of its 256 bytes
 __device__ __forceinline__ void clear_control(Control* ctl, int tid) {
   if (tid < static_cast<int>(sizeof(Control) / 4)) reinterpret_cast<int*>(ctl)[tid] = 0;
