@@ -835,9 +835,14 @@ __device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t,
 // kFlagged: the rows that row_flag marks (the exact fallback).  They are few or none, and only the device knows: a grid of at most
 // kFlaggedCtas goes through all of them.  (A CTA per
 // row took 21 us, with the scan ahead of it, to find nothing to do among 4096 rows and 39 us, in two rounds, among 8192; now 9 and 12.)
+// (The row's select is out of line there: inlined into the loop, 4 rows of 2^20 keys through the fallback took 1.51 ms, so 1.09; a CTA per row 1.14.)
 constexpr int kFlaggedCtas = 296;
+template <int kThreads>
+__device__ __noinline__ void select_flagged_row(const SelectRowsParams& p, int t, const float* row) {
+  select_one_row<kThreads>(p, t, row, 0);
+}
 template <int kThreads, bool kFlagged>
-__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const SelectRowsParams p) {
+__global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const __grid_constant__ SelectRowsParams p) {
   chain_wait();
   if (!kFlagged) {  // a CTA for every row
     const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x);
@@ -849,7 +854,7 @@ __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows
     const int t = p.fb_list != nullptr ? p.fb_list[p.fb_round_base + b / p.rows_per_block] * p.rows_per_block + b % p.rows_per_block : p.row_begin + b;
     if (t >= p.T || !p.row_flag[t]) continue;
     __syncthreads();  // the row before is done with the shared memory
-    select_one_row<kThreads>(p, t, p.scores + static_cast<size_t>(b) * p.ld, 0);
+    select_flagged_row<kThreads>(p, t, p.scores + static_cast<size_t>(b) * p.ld);
   }
 }
 
