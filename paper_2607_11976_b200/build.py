@@ -11,7 +11,7 @@ LIB_DIR = os.path.join(HERE, "lib")
 LIB_PATH = os.path.join(LIB_DIR, "liblt_indexer.so")
 DEBUG_LIB_PATH = os.path.join(LIB_DIR, "liblt_indexer_dbg.so")  # bounds-checking build (-DLT_DEBUG_BOUNDS)
 SOURCES = ["lt_api.cu", "lt_scan_mma.cu", "lt_scan_fp8.cu", "lt_select.cu", "lt_sampler.cu", "lt_dsa_union.cu", "lt_scan_knn.cu", "lt_umma_stream.cu"]
-HEADERS = ["lt_cluster_width.h", "lt_common.cuh", "lt_fine_select.cuh", "lt_host.h", "lt_ptx.cuh", os.path.join("..", "..", "include", "lt_indexer.h")]
+HEADERS = ["lt_cluster_width.h", "lt_common.cuh", "lt_fine_select.cuh", "lt_host.h", "lt_ptx.cuh", "lt_work_items.h", os.path.join("..", "..", "include", "lt_indexer.h")]
 
 
 def _nvcc() -> str:

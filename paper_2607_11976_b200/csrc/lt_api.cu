@@ -12,6 +12,7 @@
 #include "../../include/lt_indexer.h"
 #include "lt_common.cuh"
 #include "lt_host.h"
+#include "lt_work_items.h"
 
 namespace lt {
 namespace {
@@ -299,8 +300,8 @@ int sm_count() {
 
 // causal_offset: of the mask under which tiles that no row of a block can see are skipped
 int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causal_offset = INT_MAX) {
-  if (tun.segment_tiles > 0) return tun.segment_tiles;
   int n_tiles = (n_keys + kTileKeys - 1) / kTileKeys;
+  if (tun.segment_tiles > 0) return clamp_segment(tun.segment_tiles, n_tiles);
   constexpr int kItemOverheadTiles = 4;
   // A triangular mask: blocks see from `first` tiles to all of them, their items are dealt out longest first, and what matters is the
   // number of items (each starts up) and how evenly they fill the CTAs: whole rows of up to 256 tiles for many blocks.
@@ -927,8 +928,8 @@ int knn_check(int dtype, const void* q, const void* x, int T, int N, int D) {
 }
 
 int knn_seg_tiles(const Tun& tun, int n_keys, int grid) {
-  if (tun.segment_tiles > 0) return tun.segment_tiles;
   const int n_tiles = (n_keys + kTileKeys - 1) / kTileKeys;
+  if (tun.segment_tiles > 0) return clamp_segment(tun.segment_tiles, n_tiles);
   int seg = 32;
   while (seg > 2 && (n_tiles + seg - 1) / seg < 4 * grid) seg >>= 1;
   // too few tiles to go round (the sample of 64 queries over 2^20 vectors, 64 tiles on 148 SMs: 17 -> 15 us, whole call 287 -> 283)

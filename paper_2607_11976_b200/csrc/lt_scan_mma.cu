@@ -33,6 +33,7 @@
 #include "lt_common.cuh"
 #include "lt_host.h"
 #include "lt_ptx.cuh"
+#include "lt_work_items.h"
 
 namespace lt {
 
@@ -115,16 +116,11 @@ struct Item {
 
 // Work items are (key segment, query block) pairs, segment-major, so that CTAs running side by
 // side stream the same part of K (L2 reuse) for different query blocks.  Within a segment the last rows come first: under a triangular
-// mask they are the longest.  The items are dealt out to and fro (CTA 0 .. G - 1, then G - 1 .. 0), so that the CTA with the longest item
-// of a round gets the shortest of the next (4096 rows over their own 4096 keys, scan 117 -> 107 us).
-__device__ __forceinline__ int item_of_round(int round) {
-  const int b = static_cast<int>(blockIdx.x), g = static_cast<int>(gridDim.x);
-  return round * g + ((round & 1) ? g - 1 - b : b);
-}
-// (false also for numbers past the last item: their segment has no tiles)
-__device__ __forceinline__ bool resolve_item(const ScanParams& p, int n_blocks, int item, Item& it) {
-  int seg = item / n_blocks;
-  int qb = n_blocks - 1 - (item - seg * n_blocks);
+// mask they are the longest.  Dealt out to and fro, 4096 rows over their own 4096 keys, scan 117 -> 107 us (lt_work_items.h).
+// (false also for numbers past the last item: nothing of the chunk is looked up for them)
+__device__ __forceinline__ bool resolve_item(const ScanParams& p, int n_blocks, unsigned int n_items, unsigned int item, Item& it) {
+  int qb;
+  if (!split_item(item, n_items, n_blocks, p.seg_tiles, qb, it.tile_lo)) return false;
   int last_row;
   if (p.fb_list != nullptr) {
     it.t0 = p.fb_list[p.fb_round_base + qb] * kBlockQ;
@@ -140,7 +136,6 @@ __device__ __forceinline__ bool resolve_item(const ScanParams& p, int n_blocks, 
     int vis = visible_keys(last_row, p.n_keys, p.causal_offset);
     n_tiles = (vis + kTileKeys - 1) / kTileKeys;
   }
-  it.tile_lo = seg * p.seg_tiles;
   it.tile_hi = min(it.tile_lo + p.seg_tiles, n_tiles);
   return it.tile_lo < it.tile_hi;
 }
@@ -323,9 +318,8 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   } else {
     n_blocks = (p.row_end - p.row_begin + kBlockQ - 1) / kBlockQ;
   }
-  const int n_tiles_all = (p.n_keys + kTileKeys - 1) / kTileKeys;
-  const int n_seg = (n_tiles_all + p.seg_tiles - 1) / p.seg_tiles;
-  const int n_rounds = (n_blocks * n_seg + static_cast<int>(gridDim.x) - 1) / static_cast<int>(gridDim.x);
+  const unsigned int n_items = count_items((p.n_keys + kTileKeys - 1) / kTileKeys, p.seg_tiles, n_blocks);
+  const unsigned int n_rounds = count_rounds(n_items, gridDim.x);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -334,9 +328,9 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       uint32_t phase = 0;
       uint32_t n_done = 0;  // items issued so far (parity of the Q-block handshake)
       bool ok = true;
-      for (int round = 0; round < n_rounds && ok; ++round) {
+      for (unsigned int round = 0; round < n_rounds && ok; ++round) {
         Item it;
-        if (!resolve_item(p, n_blocks, item_of_round(round), it)) continue;
+        if (!resolve_item(p, n_blocks, n_items, item_of_round(round, blockIdx.x, gridDim.x), it)) continue;
         // query block: wait until the UMMAs of the previous item no longer read it
         ok = mbar_wait<40>(smem_u32(&st->bar_q_empty), (n_done & 1) ^ 1, abort_flag);
         if (!ok) break;
@@ -389,9 +383,9 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       uint32_t useq = 0;       // one unit: tiles issued so far
       uint32_t n_done = 0;
       bool ok = true;
-      for (int round = 0; round < n_rounds && ok; ++round) {
+      for (unsigned int round = 0; round < n_rounds && ok; ++round) {
         Item it;
-        if (!resolve_item(p, n_blocks, item_of_round(round), it)) continue;
+        if (!resolve_item(p, n_blocks, n_items, item_of_round(round, blockIdx.x, gridDim.x), it)) continue;
         ok = mbar_wait<40>(smem_u32(&st->bar_q_full), n_done & 1, abort_flag);
         if (!ok) break;
         ++n_done;
@@ -441,9 +435,9 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       uint32_t acc_phase = 0;
       uint32_t useq = 0;  // one unit: tiles gone through so far
       int seq = 0;
-      for (int round = 0; round < n_rounds; ++round) {
+      for (unsigned int round = 0; round < n_rounds; ++round) {
         Item it;
-        if (!resolve_item(p, n_blocks, item_of_round(round), it)) continue;
+        if (!resolve_item(p, n_blocks, n_items, item_of_round(round, blockIdx.x, gridDim.x), it)) continue;
         ++seq;
         named_bar_sync(1, n_sync);  // A: everybody is done with the previous item's shared state
         if (!is_refresh) {

@@ -110,3 +110,30 @@ def test_triangular_mask(name, offset, path):
     idx, score, status = run_topk(inp, lt.Tunables(path=path))
     assert status[0] & lt.LT_STATUS_TIMEOUT == 0
     assert np.array_equal(idx, want[0]) and np.array_equal(score.view(np.uint32), want[1].view(np.uint32))
+
+
+# "do not split": a segment longer than any row, in the forms that scan with one unit, two units, a sample, vectors, and through the fallback
+@pytest.mark.parametrize("segment_tiles", [1 << 24, 1 << 30, 2 ** 31 - 1])
+@pytest.mark.parametrize("T,N,tun", [(1, 40000, {}), (64, 9000, {}), (70, 9000, dict(path=lt.LT_PATH_FUSED)), (9, 40000, dict(path=lt.LT_PATH_FUSED, grid=296)),
+                                     (40, 9000, dict(path=lt.LT_PATH_FUSED, cap_mult=1, sample_rank=1)), (20, 9000, dict(path=lt.LT_PATH_FUSED_ABS))])
+def test_segments_longer_than_the_context(segment_tiles, T, N, tun):
+    inp = make_config("fp8_ar1", T=T, N=N, topk=128)
+    want = run_topk(inp, lt.Tunables(**tun))
+    idx, score, status = run_topk(inp, lt.Tunables(segment_tiles=segment_tiles, **tun))
+    assert status[0] & lt.LT_STATUS_TIMEOUT == 0 and (status[1] > 0) == (want[2][1] > 0)
+    assert np.array_equal(idx, want[0]) and np.array_equal(score.view(np.uint32), want[1].view(np.uint32))
+
+
+@pytest.mark.parametrize("segment_tiles", [1 << 24, 2 ** 31 - 1])
+@pytest.mark.parametrize("path", [lt.LT_PATH_AUTO, lt.LT_PATH_FUSED])
+def test_segments_longer_than_the_corpus(segment_tiles, path):
+    inp = make_knn(T=70, N=9000, D=64, topk=100)
+    q, x = (torch.from_numpy(a.view(np.int16)).view(torch.bfloat16).cuda() for a in (inp.q, inp.x))
+    bits = []
+    for tun in (lt.Tunables(path=path), lt.Tunables(path=path, segment_tiles=segment_tiles)):
+        ws = torch.empty(lt.lt_knn_topk_workspace_bytes(70, 9000, 64, 100, tun), dtype=torch.uint8, device="cuda")
+        idx, score = torch.empty((70, 100), dtype=torch.int32, device="cuda"), torch.empty((70, 100), device="cuda")
+        lt.lt_knn_topk(q, x, 100, idx, score, ws, tun)
+        assert lt.lt_read_status(ws)[0] & lt.LT_STATUS_TIMEOUT == 0
+        bits.append((idx.cpu().numpy(), score.cpu().numpy().view(np.uint32)))
+    assert np.array_equal(bits[0][0], bits[1][0]) and np.array_equal(bits[0][1], bits[1][1])
