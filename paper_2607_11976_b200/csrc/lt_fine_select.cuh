@@ -38,15 +38,19 @@ namespace lt {
 constexpr int kFineBins = 4096;
 constexpr int kFineBatch = 8;
 
-// visits every key of this thread from number `from` on
-template <int kThreads, class Load, class Visit>
+// visits every key of this thread from number `from` on.  kInLoop: the caller goes through several rows.  Registers that only some paths
+// set then count as held from one row to the next - those of every sweep together, half a kilobyte a thread went to memory - so
+// that the keys past the end are set too.  (Where a CTA selects one row it costs a few instructions: 8 x 16 K dense 13.4 -> 13.6 us.)
+template <int kThreads, bool kInLoop, class Load, class Visit>
 __device__ __forceinline__ void fine_sweep(const Load& load, unsigned int from, unsigned int n, Visit&& visit) {
   const unsigned int tid = threadIdx.x;
   for (unsigned int at = from; at < n; at += kFineBatch * kThreads) {
     uint2 e[kFineBatch];
 #pragma unroll
-    for (int j = 0; j < kFineBatch; ++j)
+    for (int j = 0; j < kFineBatch; ++j) {
       if (at + j * kThreads + tid < n) e[j] = load(at + j * kThreads + tid);
+      else if (kInLoop) e[j] = make_uint2(0u, 0u);
+    }
 #pragma unroll
     for (int j = 0; j < kFineBatch; ++j)
       if (at + j * kThreads + tid < n) visit(e[j]);
@@ -54,13 +58,13 @@ __device__ __forceinline__ void fine_sweep(const Load& load, unsigned int from, 
 }
 
 // ... and all of them, the first batch from registers
-template <int kThreads, class Load, class Visit>
+template <int kThreads, bool kInLoop, class Load, class Visit>
 __device__ __forceinline__ void fine_sweep(const Load& load, const uint2 (&c)[kFineBatch], unsigned int n, Visit&& visit) {
   const unsigned int tid = threadIdx.x;
 #pragma unroll
   for (int j = 0; j < kFineBatch; ++j)
     if (j * kThreads + tid < n) visit(c[j]);
-  fine_sweep<kThreads>(load, kFineBatch * kThreads, n, visit);
+  fine_sweep<kThreads, kInLoop>(load, kFineBatch * kThreads, n, visit);
 }
 
 // One attempt: sweep(visit) visits every key of the thread, bin_of(score bits) maps monotonically, the best keys to bin 0; the bins are
@@ -151,7 +155,7 @@ __device__ __forceinline__ bool fine_attempt(const Sweep& sweep, int kk, int top
   return true;
 }
 
-template <int kThreads, class Load>
+template <int kThreads, bool kInLoop = false, class Load>
 __device__ __forceinline__ bool fine_select_sort(const Load& load, const uint2 (&c)[kFineBatch], unsigned int n, int kk, int topk,
                                                  uint64_t* keys, unsigned int key_cap, unsigned int* bins, int32_t* out_idx,
                                                  float* out_score, int n_keys, Control* ctl, bool leave_nan = false) {
@@ -164,7 +168,7 @@ __device__ __forceinline__ bool fine_select_sort(const Load& load, const uint2 (
   // range of the scores; a warp with a NaN among its own says so in place of its maximum
   float fmin = INFINITY, fmax = -INFINITY;
   bool nan = false;
-  fine_sweep<kThreads>(load, c, n, [&](uint2 e) {
+  fine_sweep<kThreads, kInLoop>(load, c, n, [&](uint2 e) {
     const float v = __uint_as_float(e.x);
     fmin = fminf(fmin, v);
     fmax = fmaxf(fmax, v);
@@ -194,7 +198,7 @@ __device__ __forceinline__ bool fine_select_sort(const Load& load, const uint2 (
     fmin = __uint_as_float(key_to_score_bits(kmin));
     fmax = __uint_as_float(key_to_score_bits(kmax));
     const float scale = static_cast<float>(kFineBins) / (fmax - fmin);
-    if (fine_attempt<kThreads>([&](auto&& visit) { fine_sweep<kThreads>(load, c, n, visit); }, kk, topk, keys, key_cap, bins, out_idx, out_score, n_keys, ctl, [&](uint32_t bits) {
+    if (fine_attempt<kThreads>([&](auto&& visit) { fine_sweep<kThreads, kInLoop>(load, c, n, visit); }, kk, topk, keys, key_cap, bins, out_idx, out_score, n_keys, ctl, [&](uint32_t bits) {
           const float d = fmax - __uint_as_float(bits);
           const float b = __fmaf_rn(d, scale, kOne);
           return min(__float_as_uint(b), kOneBits + kFineBins - 1u) - kOneBits;
@@ -207,7 +211,7 @@ __device__ __forceinline__ bool fine_select_sort(const Load& load, const uint2 (
   if (nan) {
     kmin = 0xffffffffu;
     kmax = 0u;
-    fine_sweep<kThreads>(load, 0u, n, [&](uint2 e) {
+    fine_sweep<kThreads, kInLoop>(load, 0u, n, [&](uint2 e) {
       kmin = min(kmin, score_to_key(e.x));
       kmax = max(kmax, score_to_key(e.x));
     });
@@ -226,7 +230,7 @@ __device__ __forceinline__ bool fine_select_sort(const Load& load, const uint2 (
   }
   const unsigned int span = kmax - kmin;
   const unsigned int kscale = span >= kFineBins ? static_cast<unsigned int>((static_cast<unsigned long long>(kFineBins) << 32) / (static_cast<unsigned long long>(span) + 1ull)) : 0u;
-  return fine_attempt<kThreads>([&](auto&& visit) { fine_sweep<kThreads>(load, 0u, n, visit); }, kk, topk, keys, key_cap, bins, out_idx, out_score, n_keys, ctl, [&](uint32_t bits) {
+  return fine_attempt<kThreads>([&](auto&& visit) { fine_sweep<kThreads, kInLoop>(load, 0u, n, visit); }, kk, topk, keys, key_cap, bins, out_idx, out_score, n_keys, ctl, [&](uint32_t bits) {
     const unsigned int k = score_to_key(bits);
     return kscale != 0u ? __umulhi(kmax - k, kscale) : min(kmax - k, static_cast<unsigned int>(kFineBins - 1));
   });

@@ -781,7 +781,7 @@ __device__ __forceinline__ void radix_select_row(const float* row, int vis, int 
 // one (or one with mass ties) takes a 4-pass MSB radix select for the k-th key, ordered collection of ties (lowest
 // indices first), and a sort of the k winners.
 // ---------------------------------------------------------------------------------------------
-template <int kThreads>
+template <int kThreads, bool kInLoop>
 __device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t, const float* row, int slot) {
   extern __shared__ __align__(16) uint64_t sel_smem[];  // the distribution sort's bins, then two buffers of p.sel_slots keys
   unsigned int* bins = reinterpret_cast<unsigned int*>(sel_smem);
@@ -805,7 +805,7 @@ __device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t,
       if (i < vis) first[j] = make_uint2(__float_as_uint(row[i]), static_cast<unsigned int>(i));
     }
     add_status(p.ctl, slot);
-    if (fine_select_sort<kThreads>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
+    if (fine_select_sort<kThreads, kInLoop>([&](unsigned int i) { return make_uint2(__float_as_uint(row[i]), i); }, first,
                                       static_cast<unsigned int>(vis), kk, p.topk, sel, 2u * p.sel_slots, bins, out_idx, out_score,
                                       p.N, p.ctl, p.nan_last != 0 && vis > p.topk))
       return;
@@ -826,7 +826,7 @@ __device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t,
 #pragma unroll
   for (int j = 0; j < kFineBatch; ++j)
     if (j * kThreads + tid < kk) first[j] = winner(j * kThreads + tid);
-  if (fine_select_sort<kThreads>(winner, first, static_cast<unsigned int>(kk), kk, p.topk, sel + p.sel_slots, p.sel_slots, bins,
+  if (fine_select_sort<kThreads, kInLoop>(winner, first, static_cast<unsigned int>(kk), kk, p.topk, sel + p.sel_slots, p.sel_slots, bins,
                                  out_idx, out_score, p.N, p.ctl))
     return;
   sort_and_write(sel, kk, p.topk, out_idx, out_score, p.N, p.ctl);
@@ -835,18 +835,19 @@ __device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t,
 // kFlagged: the rows that row_flag marks (the exact fallback).  They are few or none, and only the device knows: a grid of at most
 // kFlaggedCtas goes through all of them.  (A CTA per
 // row took 21 us, with the scan ahead of it, to find nothing to do among 4096 rows and 39 us, in two rounds, among 8192; now 9 and 12.)
-// (The row's select is out of line there: inlined into the loop, 4 rows of 2^20 keys through the fallback took 1.51 ms, so 1.09; a CTA per row 1.14.)
+// (The row's select is out of line there: inlined into the loop, 4 rows of 2^20 keys through the fallback 1.20 ms, so 1.08; a CTA per row 1.17.
+// Whole calls with every row flagged, a CTA per row / now: 8 x 16 K 36.0 / 35.1 us, 148 x 8 K 64.8 / 64.2, 4096 x 8 K 939 / 886.)
 constexpr int kFlaggedCtas = 296;
 template <int kThreads>
 __device__ __noinline__ void select_flagged_row(const SelectRowsParams& p, int t, const float* row) {
-  select_one_row<kThreads>(p, t, row, 0);
+  select_one_row<kThreads, true>(p, t, row, 0);
 }
 template <int kThreads, bool kFlagged>
 __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const __grid_constant__ SelectRowsParams p) {
   chain_wait();
   if (!kFlagged) {  // a CTA for every row
     const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x);
-    select_one_row<kThreads>(p, p.row_begin + blockIdx.x, p.scores + static_cast<size_t>(blockIdx.x) * p.ld, slot);
+    select_one_row<kThreads, false>(p, p.row_begin + blockIdx.x, p.scores + static_cast<size_t>(blockIdx.x) * p.ld, slot);
     return;
   }
   const int n = p.fb_list != nullptr ? min(p.n_blocks, (*p.fb_blocks - p.fb_round_base) * p.rows_per_block) : p.n_blocks;
