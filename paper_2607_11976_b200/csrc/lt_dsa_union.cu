@@ -9,7 +9,7 @@
 // distributed shared memory (a CTA combines one slice and hands it to all), and from then on every CTA can turn a
 // position into its slot on its own: it writes its slice of the list and builds its rows' masks in shared memory.
 // With one CTA per group, outputs cleared by memsets and masks built by global atomics, 4096 rows x 2048 over 128 K
-// positions in groups of 64 took 201 us; now 50 us, with 25 us the time of
+// positions in groups of 64 took 201 us; now 46 us, with 25 us the time of
 // moving the bytes.  What is left is the chain of phases of a CTA (mark 5 us, combine 5, prefix 2, list 4, then the masks) and
 // clusters that fill some GPCs' SMs with four CTAs and others' with three.
 #include <cooperative_groups.h>
@@ -62,8 +62,29 @@ __device__ __forceinline__ unsigned int warp_inclusive_sum(unsigned int v, int l
   return v;
 }
 
+// the slot of position q of the window, whose first slot is `slot`
+template <int kUnit>
+__device__ __forceinline__ unsigned int slot_of(const uint32_t* bitmap, const uint32_t* prefix, unsigned int q, unsigned int slot) {
+  const uint4* bitmap4 = reinterpret_cast<const uint4*>(bitmap);
+  const unsigned int below = (1u << (q & 31)) - 1u;
+  if (kUnit == 1) {
+    slot += prefix[q >> 5] + __popc(bitmap[q >> 5] & below);
+  } else {
+    const uint4 v = bitmap4[q >> 7];
+    const unsigned int k = (q >> 5) & 3u;
+    const uint32_t word = k == 0u ? v.x : k == 1u ? v.y : k == 2u ? v.z : v.w;
+    if (kUnit == 8 && ((q >> 7) & 1u) != 0u) slot += popc4(bitmap4[(q >> 7) - 1u]);
+    slot += prefix[(q >> 5) / kUnit] + __popc(word & below) + (k > 0u ? __popc(v.x) : 0) + (k > 1u ? __popc(v.y) : 0) + (k > 2u ? __popc(v.z) : 0);
+  }
+  return slot;
+}
+
 // kUnit: words to a stored prefix (1, 4 or 8).  512 threads while several CTAs share an SM, 1024 where one has it to itself.
-template <int kUnit, int kUnionThreads>
+// kWholeRows: one window, and rows whose masks come one at a time and whole, four positions to a thread, in 16-byte pieces.  Kernels of
+// their own: beside that loop the general one was slower (4096 x 2048 in 32 groups over 65,536 positions 76.2 -> 78.3 us).
+// Where four CTAs share an SM a thread has 32 registers, and it counts what holds them: copies of the masks are not unrolled (the same 73.3, in 64
+// groups, whole rows, 41.9 -> 40.1).
+template <int kUnit, int kUnionThreads, bool kWholeRows>
 __global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUnit == 1 ? 4 : 2) dsa_union_kernel(const UnionParams p) {
   constexpr int kUnionWarps = kUnionThreads / 32;
   namespace cg = cooperative_groups;
@@ -85,12 +106,12 @@ __global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUn
 
   for (int i = tid; i < p.buf_words; i += kUnionThreads) masks[i] = 0u;
   chain_wait();
-  for (long long wbase = 0; wbase < p.N; wbase += static_cast<long long>(p.window_words) * 32) {
+  for (long long wbase = 0; kWholeRows || wbase < p.N; wbase += static_cast<long long>(p.window_words) * 32) {
     const long long left = p.N - wbase;
-    const int span = static_cast<int>(left < static_cast<long long>(p.window_words) * 32 ? left : static_cast<long long>(p.window_words) * 32);
+    const int span = kWholeRows ? p.N : static_cast<int>(left < static_cast<long long>(p.window_words) * 32 ? left : static_cast<long long>(p.window_words) * 32);
     const bool last = left <= static_cast<long long>(p.window_words) * 32;
     const int words = ((span + 31) / 32 + 7) / 8 * 8;
-    const int base = static_cast<int>(wbase);  // positions are below N < 2^31
+    const int base = kWholeRows ? 0 : static_cast<int>(wbase);  // positions are below N < 2^31
     for (int i = tid; i < words / 4; i += kUnionThreads) reinterpret_cast<uint4*>(bitmap)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     // 1. mark this CTA's rows: the atomic OR deduplicates
@@ -174,7 +195,7 @@ __global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUn
       const uint32_t own = w + lane < s1 ? bitmap[w + lane] : 0u;
       const unsigned int in_all = __reduce_add_sync(0xffffffffu, static_cast<unsigned int>(__popc(own)));
       if (in_all == 0u) continue;
-      int32_t* dst = out + list_len;
+      int32_t* dst = kWholeRows ? out : out + list_len;
       if (in_all >= 96u) {
         dst += prefix[w / kUnit];  // (w is a multiple of eight)
 #pragma unroll 8
@@ -204,28 +225,16 @@ __global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUn
     const unsigned int end_slot = list_len + total;
     const int w_end = last ? p.mask_words : static_cast<int>((end_slot + 31u) >> 5);
     const int batch = p.mask_words <= p.buf_words ? p.buf_words / p.mask_words : 1;
-    // list slots before position q of the window
-    auto slots_before = [&](unsigned int q) {
-      const unsigned int below = (1u << (q & 31)) - 1u;
-      if (kUnit == 1) return prefix[q >> 5] + __popc(bitmap[q >> 5] & below);
-      const uint4 v = bitmap4[q >> 7];
-      const unsigned int k = (q >> 5) & 3u;
-      const uint32_t word = k == 0u ? v.x : k == 1u ? v.y : k == 2u ? v.z : v.w;
-      unsigned int n = prefix[(q >> 5) / kUnit] + __popc(word & below) + (k > 0u ? __popc(v.x) : 0) + (k > 1u ? __popc(v.y) : 0) + (k > 2u ? __popc(v.z) : 0);
-      if (kUnit == 8 && ((q >> 7) & 1u) != 0u) n += popc4(bitmap4[(q >> 7) - 1u]);
-      return n;
-    };
-    // Rows that come one at a time, whole, four positions to a thread: a row's positions are fetched while the mask of the row before it
-    // is written out.  (4096 x 2048 in 64 groups over 131,072 positions 67 -> 50 us.)
-    if (last && wbase == 0 && batch == 1 && p.mask_words <= p.buf_words && (p.topk & 3) == 0 && p.topk <= 4 * kUnionThreads &&
-        ((reinterpret_cast<uintptr_t>(p.idx) | reinterpret_cast<uintptr_t>(p.mask)) & 15u) == 0 && (p.mask_words & 3) == 0) {
+    if constexpr (kWholeRows) {
+      // a row's positions are fetched while the mask of the row before it is written out (4096 x 2048 in 64 groups over 131,072 positions
+      // 63.0 -> 46.0 us)
       const bool mine = 4 * tid < p.topk;
       const int4* src = reinterpret_cast<const int4*>(my_idx) + tid;
       uint4* dst = reinterpret_cast<uint4*>(p.mask + static_cast<size_t>(row_lo) * p.mask_words);
       uint4* masks4 = reinterpret_cast<uint4*>(masks);
       auto member = [&](int pos) {
         if (static_cast<unsigned int>(pos) < static_cast<unsigned int>(span)) {
-          const unsigned int slot = slots_before(static_cast<unsigned int>(pos));
+          const unsigned int slot = slot_of<kUnit>(bitmap, prefix, static_cast<unsigned int>(pos), 0u);
           atomicOr(&masks[slot >> 5], 1u << (slot & 31));
         }
       };
@@ -241,6 +250,7 @@ __global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUn
         member(pos.w);
         __syncthreads();
         // written and cleared by the same thread
+#pragma unroll 1
         for (int i = tid; i < p.mask_words / 4; i += kUnionThreads) {
           dst[i] = masks4[i];
           masks4[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -250,61 +260,63 @@ __global__ void __launch_bounds__(kUnionThreads, kUnionThreads == 1024 ? 1 : kUn
       }
       list_len = total;
       break;
-    }
-    for (int w0 = w_first; w0 < w_end; w0 += p.buf_words) {
-      const int n_words = min(w_end - w0, p.buf_words);
-      const bool has_bits = (static_cast<unsigned int>(w0) << 5) < end_slot;
-      for (int row = row_lo; row < row_hi; row += batch) {
-        uint32_t* buf = masks;
-        const int rows = min(batch, row_hi - row);
-        __syncthreads();  // the batch before has been written out
-        if (has_bits) {
-          const int32_t* e = p.idx + static_cast<size_t>(row) * p.topk;
-          const int n = rows * p.topk;
-          for (int i = tid; i < n; i += 4 * kUnionThreads) {
-            int pos[4];
+    } else {
+      for (int w0 = w_first; w0 < w_end; w0 += p.buf_words) {
+        const int n_words = min(w_end - w0, p.buf_words);
+        const bool has_bits = (static_cast<unsigned int>(w0) << 5) < end_slot;
+        for (int row = row_lo; row < row_hi; row += batch) {
+          uint32_t* buf = masks;
+          const int rows = min(batch, row_hi - row);
+          __syncthreads();  // the batch before has been written out
+          if (has_bits) {
+            const int32_t* e = p.idx + static_cast<size_t>(row) * p.topk;
+            const int n = rows * p.topk;
+            for (int i = tid; i < n; i += 4 * kUnionThreads) {
+              int pos[4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) pos[j] = __ldg(e + min(i + j * kUnionThreads, n - 1));  // (the last entry again: harmless)
+              for (int j = 0; j < 4; ++j) pos[j] = __ldg(e + min(i + j * kUnionThreads, n - 1));  // (the last entry again: harmless)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const unsigned int q = static_cast<unsigned int>(pos[j] - base);
-              if (pos[j] < base || q >= static_cast<unsigned int>(span)) continue;
-              const unsigned int slot = list_len + slots_before(q);
-              const int mw = static_cast<int>(slot >> 5) - w0;
-              const int r = rows == 1 ? 0 : min(i + j * kUnionThreads, n - 1) / p.topk;
-              if (mw >= 0 && mw < n_words) atomicOr(&buf[r * n_words + mw], 1u << (slot & 31));
+              for (int j = 0; j < 4; ++j) {
+                const unsigned int q = static_cast<unsigned int>(pos[j] - base);
+                if (pos[j] < base || q >= static_cast<unsigned int>(span)) continue;
+                const unsigned int slot = slot_of<kUnit>(bitmap, prefix, q, list_len);
+                const int mw = static_cast<int>(slot >> 5) - w0;
+                const int r = rows == 1 ? 0 : min(i + j * kUnionThreads, n - 1) / p.topk;
+                if (mw >= 0 && mw < n_words) atomicOr(&buf[r * n_words + mw], 1u << (slot & 31));
+              }
             }
+            if (w0 == w_first && (list_len & 31u) != 0u && tid < rows)
+              atomicOr(&buf[tid * n_words], __ldcg(p.mask + static_cast<size_t>(row + tid) * p.mask_words + w0));
           }
-          if (w0 == w_first && (list_len & 31u) != 0u && tid < rows)
-            atomicOr(&buf[tid * n_words], __ldcg(p.mask + static_cast<size_t>(row + tid) * p.mask_words + w0));
-        }
-        __syncthreads();
-        // written and cleared by the same thread
-        uint32_t* dst = p.mask + static_cast<size_t>(row) * p.mask_words + w0;
-        if (rows == 1 || n_words == p.mask_words) {  // one run of words
-          const int n = rows * n_words;
-          if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0 && (n & 3) == 0) {
-            for (int i = tid; i < n / 4; i += kUnionThreads) {
-              reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(buf)[i];
-              reinterpret_cast<uint4*>(buf)[i] = make_uint4(0u, 0u, 0u, 0u);
+          __syncthreads();
+          // written and cleared by the same thread
+          uint32_t* dst = p.mask + static_cast<size_t>(row) * p.mask_words + w0;
+          if (rows == 1 || n_words == p.mask_words) {  // one run of words
+            const int n = rows * n_words;
+            if ((reinterpret_cast<uintptr_t>(dst) & 15u) == 0 && (n & 3) == 0) {
+#pragma unroll 1
+              for (int i = tid; i < n / 4; i += kUnionThreads) {
+                reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(buf)[i];
+                reinterpret_cast<uint4*>(buf)[i] = make_uint4(0u, 0u, 0u, 0u);
+              }
+            } else {
+              for (int i = tid; i < n; i += kUnionThreads) {
+                dst[i] = buf[i];
+                buf[i] = 0u;
+              }
             }
           } else {
-            for (int i = tid; i < n; i += kUnionThreads) {
-              dst[i] = buf[i];
-              buf[i] = 0u;
-            }
+            for (int r = 0; r < rows; ++r)
+              for (int i = tid; i < n_words; i += kUnionThreads) {
+                dst[static_cast<size_t>(r) * p.mask_words + i] = buf[r * n_words + i];
+                buf[r * n_words + i] = 0u;
+              }
           }
-        } else {
-          for (int r = 0; r < rows; ++r)
-            for (int i = tid; i < n_words; i += kUnionThreads) {
-              dst[static_cast<size_t>(r) * p.mask_words + i] = buf[r * n_words + i];
-              buf[r * n_words + i] = 0u;
-            }
         }
       }
+      list_len = end_slot;
+      __syncthreads();
     }
-    list_len = end_slot;
-    __syncthreads();
   }
   for (unsigned int i = list_len + static_cast<unsigned int>(rank * kUnionThreads + tid); i < static_cast<unsigned int>(p.cap);
        i += static_cast<unsigned int>(n_cta * kUnionThreads))
@@ -342,13 +354,14 @@ cudaError_t launch_dsa_union(const int32_t* idx, int T, int topk, int N, int gro
   };
 
   // by unit and threads
-  static std::atomic<unsigned long long> done[5];
+  static std::atomic<unsigned long long> done[2][5];
   using Kernel = void (*)(UnionParams);
-  const Kernel kernels[5] = {dsa_union_kernel<1, 512>, dsa_union_kernel<1, 1024>, dsa_union_kernel<4, 512>, dsa_union_kernel<4, 1024>,
-                             dsa_union_kernel<8, 1024>};
+  const Kernel kernels[2][5] = {{dsa_union_kernel<1, 512, false>, dsa_union_kernel<1, 1024, false>, dsa_union_kernel<4, 512, false>,
+                                 dsa_union_kernel<4, 1024, false>, dsa_union_kernel<8, 1024, false>},
+                                {dsa_union_kernel<1, 512, true>, dsa_union_kernel<1, 1024, true>, dsa_union_kernel<4, 512, true>,
+                                 dsa_union_kernel<4, 1024, true>, dsa_union_kernel<8, 1024, true>}};
   const int first = unit == 1 ? 0 : unit == 4 ? 2 : 4;
-  cudaError_t e = cudaSuccess;
-  for (int k = first; k < (unit == 8 ? 5 : first + 2) && e == cudaSuccess; ++k) e = allow_smem(reinterpret_cast<const void*>(kernels[k]), done[k], true);
+  cudaError_t e = allow_smem(reinterpret_cast<const void*>(kernels[0][first]), done[0][first], true);
   if (e != cudaSuccess) return e;
   // how many clusters of a width run at once: asked for once for each device, unit, CTAs of that size to an SM, and width (with the
   // largest mask buffer, of one CTA for all rows)
@@ -367,7 +380,7 @@ cudaError_t launch_dsa_union(const int32_t* idx, int T, int topk, int N, int gro
     std::atomic<short>& known = at_once_cache[dev & 63][first / 2][per_sm > 0 ? per_sm - 1 : 0][log2];
     int n = known.load(std::memory_order_relaxed);
     if (n == 0) {
-      n = 1 + clusters_at_once(kernels[first], unit == 8 ? 1024 : 512, smem_max, width);
+      n = 1 + clusters_at_once(kernels[0][first], unit == 8 ? 1024 : 512, smem_max, width);
       known.store(static_cast<short>(n), std::memory_order_relaxed);
     }
     return n - 1;
@@ -382,8 +395,14 @@ cudaError_t launch_dsa_union(const int32_t* idx, int T, int topk, int N, int gro
   const bool wide = unit == 8 ||
                     (static_cast<long long>(n_groups) * width <= (width == 1 ? sms : unit == 1 ? sms / 2 : 0) &&
                      static_cast<long long>(p.rows_per_cta) * topk <= kUnionWideEntries);
-  const Kernel kernel = kernels[unit == 8 || !wide ? first : first + 1];
-  return launch_chained(kernel, n_groups * width, wide ? 1024 : 512, smem, stream, width, p);
+  const int threads = wide ? 1024 : 512;
+  // (what the loop over whole rows takes.  Rows that come several at a time wait for their positions at each batch; prefetching them was not tried)
+  const bool whole = words <= p.window_words && p.mask_words <= p.buf_words && p.buf_words / p.mask_words == 1 && topk % 4 == 0 && topk <= 4 * threads &&
+                     p.mask_words % 4 == 0 && ((reinterpret_cast<uintptr_t>(idx) | reinterpret_cast<uintptr_t>(mask)) & 15u) == 0;
+  const int k = unit == 8 || !wide ? first : first + 1;
+  e = allow_smem(reinterpret_cast<const void*>(kernels[whole][k]), done[whole][k], true);
+  if (e != cudaSuccess) return e;
+  return launch_chained(kernels[whole][k], n_groups * width, threads, smem, stream, width, p);
 }
 
 }  // namespace lt
