@@ -146,21 +146,28 @@ __global__ void __launch_bounds__(kSimtThreads, 2) simt_scores_kernel(const void
 }
 
 // ---------------------------------------------------------------------------------------------
-// sample statistics: one CTA per row.  A row's scores stay in registers between the sweep for the range and the one for the histogram
-// (longer rows are read again).  The threshold is nearly always in the upper bins - the rank is a twentieth of the sample - so
-// only scores from kStatsCutBin up are looked at first; they are compacted per warp, because a bin search is long and nearly every 32
-// scores hold one.  Rows whose rank-th score lies below the cut count the others too.  One B200, 8192 rows of
-// 4064 scores 91 -> 54 us, 4096 of 2048 30 -> 25, 1024 of 6144 22 -> 19, against a bin search for every score.
+// sample statistics: one CTA per row.  With the default rank, a twentieth of the sample or less, the threshold is nearly always in the upper
+// bins: a row's scores stay in registers between the sweep for the range and the one for the histogram (longer rows are
+// read again), and only scores from bin kStatsCutBin up are looked at; they are compacted per warp, because a bin search is long and nearly
+// every 32 scores hold one.  Rows whose rank-th score lies below the cut - a few outliers stretch their range - count the others too.
+// One B200, 8192 rows of 4064 scores 91 -> 54 us, 4096 of 2048 30 -> 25, 1024 of 6144 22 -> 19, against a bin search for every score;
+// 4096 of 2048 with outliers 27 -> 35.
+// Where the rank is topk - a caller's sample of usually 3 topk positions, sample_rank = -1 - nearly every row would take both sweeps, and a
+// short sample is counted before it is sorted out: all scores are counted at once there, and read again for it.  Cut / all, us: 4096
+// rows of 6144, rank 2048, 90 / 62; 2048 of 12288, rank 2048 79 / 62, 1024 60 / 62, 512 54 / 62; of 2048, rank 256 19 / 17; 8192 of 1024, rank
+// 109, 44 / 35, of 1664 44 / 42, of 2048 46 / 48.
 // ---------------------------------------------------------------------------------------------
-constexpr int kStatsCutBin = 160;  // of kBins: for bell-shaped scores about a fifth of them, three times the usual rank
-template <int kThreads, int kKeep>  // kKeep: scores a thread holds
+constexpr int kStatsCutBin = 160;    // of kBins: for bell-shaped scores about a fifth of them, three times the usual rank
+constexpr int kStatsHighShare = 8;   // the cut is used for ranks below an eighth of the sample
+constexpr int kStatsShort = 2048;    // ... of at least so many scores
+template <int kThreads, int kKeep>  // kKeep: scores a thread holds; 0: all scores are counted at once
 __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const float* __restrict__ sample, int n_sample, int rank,
                                                                 float* __restrict__ smin_out, float* __restrict__ width_out,
                                                                 float* __restrict__ thr_out, const OpenParams open) {
   constexpr int kWarps = kThreads / 32;
   __shared__ float red_min[kWarps], red_max[kWarps];
   __shared__ __align__(16) unsigned int hist[kBins];
-  __shared__ float high[kWarps][kKeep * 32];  // per warp: its scores from the cut up
+  __shared__ float high[kWarps][(kKeep > 0 ? kKeep : 1) * 32];  // per warp: its scores from the cut up
   __shared__ int s_more;
   const int t = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -179,7 +186,7 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const float* __r
   // NaN scores (sums that overflowed) would leave the row without bins; neither the minimum nor the maximum takes them, they
   // are in no bin above 0, and the gate lets none pass
   const float kNan = __uint_as_float(0x7fffffffu);
-  float v[kKeep];
+  float v[kKeep > 0 ? kKeep : 1];
 #pragma unroll
   for (int j = 0; j < kKeep; ++j) v[j] = tid + j * kThreads < n_sample ? row[tid + j * kThreads] : kNan;
   add_status(open.ctl, slot);
@@ -189,11 +196,24 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const float* __r
     mn = fminf(mn, v[j]);
     mx = fmaxf(mx, v[j]);
   }
+  if (kKeep == 0) {
+    for (int base = tid; base < n_sample; base += 8 * kThreads) {
+      float x[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) x[j] = base + j * kThreads < n_sample ? row[base + j * kThreads] : kNan;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        mn = fminf(mn, x[j]);
+        mx = fmaxf(mx, x[j]);
+      }
+    }
+  } else {
 #pragma unroll 8
-  for (int i = tid + kKeep * kThreads; i < n_sample; i += kThreads) {
-    const float x = row[i];
-    mn = fminf(mn, x);
-    mx = fmaxf(mx, x);
+    for (int i = tid + kKeep * kThreads; i < n_sample; i += kThreads) {
+      const float x = row[i];
+      mn = fminf(mn, x);
+      mx = fmaxf(mx, x);
+    }
   }
   auto warp_range = [&]() {
 #pragma unroll
@@ -215,7 +235,7 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const float* __r
   const float smin = n_sample > 0 ? mn : 0.f;
   const float width = n_sample > 0 ? (mx - smin) / static_cast<float>(kBins) : 0.f;
   const float inv_width = width > 0.f ? 1.f / width : 0.f;
-  const float cut = bin_edge(kStatsCutBin, smin, width);
+  const float cut = bin_edge(kKeep > 0 ? kStatsCutBin : 0, smin, width);
   auto count = [&](float x) { atomicAdd(&hist[bin_of(x, smin, width, inv_width)], 1u); };
   int n_high = 0;
 #pragma unroll
@@ -1234,9 +1254,12 @@ cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int ra
                                 const OpenParams* open, cudaStream_t stream) {
   const OpenParams o = open != nullptr ? *open : OpenParams{};
   // few rows leave the chip idle: a large CTA then shortens the sweeps; with many rows small CTAs overlap better
-  if (T <= 296) return launch_chained(sample_stats_kernel<1024, 8>, T, 1024, 0, stream, 1, sample, n_sample, rank, smin, width, thr, o);
-  if (n_sample > 4096) return launch_chained(sample_stats_kernel<512, 16>, T, 512, 0, stream, 1, sample, n_sample, rank, smin, width, thr, o);
-  return launch_chained(sample_stats_kernel<256, 16>, T, 256, 0, stream, 1, sample, n_sample, rank, smin, width, thr, o);
+  const bool few = T <= 296;
+  auto launch = [&](auto kernel, int threads) { return launch_chained(kernel, T, threads, 0, stream, 1, sample, n_sample, rank, smin, width, thr, o); };
+  if (n_sample < kStatsShort || static_cast<long long>(rank) * kStatsHighShare >= n_sample) return few ? launch(sample_stats_kernel<1024, 0>, 1024) : launch(sample_stats_kernel<256, 0>, 256);
+  if (few) return launch(sample_stats_kernel<1024, 8>, 1024);
+  if (n_sample > 4096) return launch(sample_stats_kernel<512, 16>, 512);
+  return launch(sample_stats_kernel<256, 16>, 256);
 }
 
 cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream) {

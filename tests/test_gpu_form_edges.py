@@ -69,6 +69,27 @@ def test_any_sample_gives_the_same_bits(T, tun):
     assert np.array_equal(idx, want[0]) and np.array_equal(score.view(np.uint32), want[1].view(np.uint32))
 
 
+# either side of the rank and the size from which a sample is cut before it is counted (an eighth, 2048 scores), in one batch of loads and
+# in several, in a sample smaller than its rank, and with keys that stretch every row's range
+@pytest.mark.parametrize("T", [5, 300])
+@pytest.mark.parametrize("outliers", [False, True])
+@pytest.mark.parametrize("topk,offset,tun", [(256, 19000, dict(sample_mult=8, sample_rank=-1)), (256, 19000, dict(sample_mult=8, sample_rank=255)),
+                                             (255, 19000, dict(sample_mult=8, sample_rank=200)), (256, 19000, dict(sample_mult=70, sample_rank=-1)),
+                                             (2048, 19000, dict(sample_mult=8, sample_rank=-1)),
+                                             (256, 100, dict(sample_rank=-1)), (1, 19000, dict(sample_mult=1, sample_rank=-1))])
+def test_sample_ranks_around_the_cut(T, outliers, topk, offset, tun):
+    inp = make_config("fp8_ar1", T=T, N=20000, topk=topk)
+    inp = dataclasses.replace(inp, causal_offset=offset)
+    if outliers:
+        scale = inp.k_scale.copy()
+        scale[::911] *= np.float32(50.0)
+        inp = dataclasses.replace(inp, k_scale=scale)
+    want = run_unfused(inp, rows_per_pass=304)
+    idx, score, status = run_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED, **tun))
+    assert status[0] & lt.LT_STATUS_TIMEOUT == 0
+    assert np.array_equal(idx, want[0]) and np.array_equal(score.view(np.uint32), want[1].view(np.uint32))
+
+
 # dense form (one CTA per row, clusters), sampled form, no common prefix to sample, more CTAs than status bytes
 @pytest.mark.parametrize("T,N,offset,tun", [(3, 5000, 4997, None), (2, 40000, 39998, None), (40, 9000, 8960, dict(path=lt.LT_PATH_FUSED)),
                                             (40, 9000, -5, dict(path=lt.LT_PATH_FUSED)), (6, 3000, -4, None),
