@@ -348,13 +348,9 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causa
 }
 
 // Whether a call's kernels open its status block and clear its counters on the way (lt_common.cuh); else launch_zero does ahead of them.
-bool opens_itself(int grid) {
-#if defined(LT_DEBUG_BOUNDS)
-  return false;
-#else
-  return grid <= kStatusSlots;
-#endif
-}
+bool opens_itself(int grid) { return grid <= kStatusSlots; }
+// what is cleared ahead of a call
+size_t cleared_ahead(const Layout& L, bool own) { return !own ? L.zero_end : kControlClearedAhead ? sizeof(Control) : 0; }
 unsigned char* status_slots(Control* ctl) { return reinterpret_cast<unsigned char*>(ctl + 1); }
 
 // the default scan kernels, or the alternative fp8 scan, behind the same parameter block
@@ -445,7 +441,8 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
   const int grid = tun.grid > 0 ? tun.grid : sm_count();
   const bool own = fused && !abs_form && opens_itself(grid);
   unsigned char* slots = own ? status_slots(ctl) : nullptr;
-  if (fused && !own) LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
+  const size_t ahead = fused ? cleared_ahead(L, own) : 0;
+  if (ahead > 0) LT_LAUNCH(launch_zero(ws, ahead, stream));
 
   if (!fused) {
     return run_unfused(dtype, false, q, w, k, k_scale, T, N, H, D, topk, causal_offset, out_idx, out_score,
@@ -555,7 +552,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     LT_LAUNCH(launch_scan(abs_form, dtype, kModeDump, q, T, sample_keys, L.n_sample, sample_pitch, p, grid, stream));
   }
   mark_phase(1, stream);
-  const OpenParams open{ctl, slots, L.n_sample > 0 ? grid : 0, tail, hist, row_flag, block_flag, L.rpb};
+  const OpenParams open{ctl, slots, L.n_sample > 0 ? grid : 0, tail, hist, row_flag, block_flag, L.rpb, L.n_blocks};
   LT_LAUNCH(launch_sample_stats(sample, T, L.n_sample, L.sample_rank, smin, width, thr, own ? &open : nullptr, stream));
   mark_phase(2, stream);
 
@@ -983,7 +980,8 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
   const int grid = tun.grid > 0 ? tun.grid : sm_count();
   const bool own = opens_itself(grid);
   unsigned char* slots = own ? status_slots(ctl) : nullptr;
-  if (!own) LT_LAUNCH(launch_zero(ws, L.zero_end, stream));
+  const size_t ahead = cleared_ahead(L, own);
+  if (ahead > 0) LT_LAUNCH(launch_zero(ws, ahead, stream));
   if (L.direct) {  // small problem: dense scores and a select over them (see use_direct)
     mark_phase(0, stream);
     mark_phase(1, stream);
@@ -1052,7 +1050,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     LT_LAUNCH(launch_scan_knn(kModeDump, q, T, x, L.n_sample, static_cast<long long>(L.sample_stride) * D, p, grid, stream));
   }
   mark_phase(1, stream);
-  const OpenParams open{ctl, slots, L.n_sample > 0 ? grid : 0, tail, hist, row_flag, block_flag, L.rpb};
+  const OpenParams open{ctl, slots, L.n_sample > 0 ? grid : 0, tail, hist, row_flag, block_flag, L.rpb, L.n_blocks};
   LT_LAUNCH(launch_sample_stats(sample, T, L.n_sample, L.sample_rank, smin, width, thr, own ? &open : nullptr, stream));
   mark_phase(2, stream);
 

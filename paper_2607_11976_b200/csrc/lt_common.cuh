@@ -26,20 +26,18 @@ struct Control {
 
 // The status block opens without a launch of its own: the call's first scan clears it and leaves each CTA's status bits in a byte of its
 // own behind it, and the kernel after that, a byte per thread of its first CTA, adds them to the status word.  (A kernel that only
-// cleared the block and the counters cost a 1-row call 0.9 of 22.9 us, a first chunk of 4096 rows 2 of 184.)  In the bounds-checking
-// build, whose checks write the status word from every kernel, and with more CTAs than bytes, everything is cleared ahead of the call.
+// cleared the block and the counters cost a 1-row call 0.9 of 22.9 us, a first chunk of 4096 rows 2 of 184.)  With more CTAs than bytes,
+// everything is cleared ahead of the call.  The bounds-checking build, whose checks write the status word from every kernel, clears the
+// block, and nothing else, ahead of the call, and then goes the same way.
 constexpr int kStatusSlots = 256 - static_cast<int>(sizeof(Control));  // what the block leaves of its 256 bytes
+#if defined(LT_DEBUG_BOUNDS)
+constexpr bool kControlClearedAhead = true;
+#else
+constexpr bool kControlClearedAhead = false;
+#endif
 __device__ __forceinline__ void clear_control(Control* ctl, int tid) {
-  if (tid < static_cast<int>(sizeof(Control) / 4)) reinterpret_cast<int*>(ctl)[tid] = 0;
+  if (!kControlClearedAhead && tid < static_cast<int>(sizeof(Control) / 4)) reinterpret_cast<int*>(ctl)[tid] = 0;
 }
-// The byte is fetched beside a kernel's first loads and looked at with them.
-__device__ __forceinline__ int load_status_slot(const unsigned char* slots, int n_slots, int tid) {
-  return slots != nullptr && blockIdx.x == 0 && tid < n_slots ? slots[tid] : 0;
-}
-__device__ __forceinline__ void add_status(Control* ctl, int slot) {
-  if (slot != 0) atomicOr(&ctl->status, slot);
-}
-
 // ---------------------------------------------------------------------------------------------
 // Index checks of the bounds-checking build (compiled with -DLT_DEBUG_BOUNDS; it stands in for a memory
 // checker): LT_IN_BOUNDS(cond, ctl) is `cond`, and where it is false it records LT_STATUS_BOUNDS in the
@@ -55,6 +53,17 @@ __device__ __forceinline__ bool lt_in_bounds(bool cond, Control* ctl) {
 #else
 #define LT_IN_BOUNDS(cond, ctl) (true)
 #endif
+
+// A scan's CTA leaves its status bits; the kernel behind it fetches them beside its first loads, and looks at them with those.
+__device__ __forceinline__ void store_status_slot(unsigned char* slots, Control* ctl, int bits) {
+  if (LT_IN_BOUNDS(static_cast<int>(blockIdx.x) < kStatusSlots, ctl)) slots[blockIdx.x] = static_cast<unsigned char>(bits);
+}
+__device__ __forceinline__ int load_status_slot(const unsigned char* slots, int n_slots, int tid, Control* ctl) {
+  return slots != nullptr && blockIdx.x == 0 && tid < n_slots && LT_IN_BOUNDS(n_slots <= kStatusSlots, ctl) ? slots[tid] : 0;
+}
+__device__ __forceinline__ void add_status(Control* ctl, int slot) {
+  if (slot != 0) atomicOr(&ctl->status, slot);
+}
 
 // ---------------------------------------------------------------------------------------------
 // Chained launches.  Every kernel of a call is launched so that it may start when the kernel ahead of it in the stream has no

@@ -205,8 +205,9 @@ struct OpenParams {
   unsigned int* tail;        // [T]
   unsigned int* hist;        // [T][kBins]
   unsigned char* row_flag;   // [T]
-  unsigned int* block_flag;  // [ceil(T / rows_per_block)]
+  unsigned int* block_flag;  // [n_blocks]
   int rows_per_block;
+  int n_blocks;
 };
 cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int rank, float* smin, float* width, float* thr,
                                 const OpenParams* open, cudaStream_t stream);

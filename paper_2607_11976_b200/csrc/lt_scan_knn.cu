@@ -207,7 +207,7 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   chain_wait();  // barriers, TMEM and tensor maps are ready by now
   if (kMode == kModeDump && p.status_slots != nullptr) {
     if (blockIdx.x == 0) clear_control(p.ctl, threadIdx.x);
-    if (threadIdx.x == 0) p.status_slots[blockIdx.x] = 0;
+    if (threadIdx.x == 0) store_status_slot(p.status_slots, p.ctl, 0);
   }
 
   const int qb_lo = p.row_begin / kQB;
@@ -473,7 +473,7 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   if (st->abort_flag) {
     if (threadIdx.x == 0) {
       if (p.status_slots != nullptr) {
-        p.status_slots[blockIdx.x] = LT_STATUS_TIMEOUT;
+        store_status_slot(p.status_slots, p.ctl, LT_STATUS_TIMEOUT);
       } else {
         atomicOr(&p.ctl->status, LT_STATUS_TIMEOUT);
       }

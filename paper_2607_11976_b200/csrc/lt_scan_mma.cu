@@ -307,7 +307,7 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   chain_wait();  // barriers, TMEM and tensor maps are ready by now
   if (kMode == kModeDump && p.status_slots != nullptr) {
     if (blockIdx.x == 0) clear_control(p.ctl, threadIdx.x);
-    if (threadIdx.x == 0) p.status_slots[blockIdx.x] = 0;
+    if (threadIdx.x == 0) store_status_slot(p.status_slots, p.ctl, 0);
   }
 
   // number of query blocks / items of this launch
@@ -641,7 +641,7 @@ scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   if (st->abort_flag) {
     if (threadIdx.x == 0) {
       if (p.status_slots != nullptr) {
-        p.status_slots[blockIdx.x] = LT_STATUS_TIMEOUT;
+        store_status_slot(p.status_slots, p.ctl, LT_STATUS_TIMEOUT);
       } else {
         atomicOr(&p.ctl->status, LT_STATUS_TIMEOUT);
       }

@@ -173,13 +173,14 @@ __global__ void __launch_bounds__(kThreads) sample_stats_kernel(const float* __r
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float* row = sample + static_cast<size_t>(t) * n_sample;
   chain_wait();
-  const int slot = load_status_slot(open.status_slots, open.n_slots, tid);
+  const int slot = load_status_slot(open.status_slots, open.n_slots, tid, open.ctl);
   if (open.ctl != nullptr) {
     for (int i = tid; i < kBins; i += kThreads) open.hist[static_cast<size_t>(t) * kBins + i] = 0u;
     if (tid == 0) {
       open.tail[t] = 0u;
       open.row_flag[t] = 0;
-      if (t % open.rows_per_block == 0) open.block_flag[t / open.rows_per_block] = 0u;
+      const int block = t / open.rows_per_block;
+      if (t == block * open.rows_per_block && LT_IN_BOUNDS(block < open.n_blocks, open.ctl)) open.block_flag[block] = 0u;
     }
     if (open.n_slots == 0 && t == 0) clear_control(open.ctl, tid);
   }
@@ -866,7 +867,7 @@ template <int kThreads, bool kFlagged>
 __global__ void __launch_bounds__(kThreads, kThreads <= 512 ? 3 : 1) select_rows_kernel(const __grid_constant__ SelectRowsParams p) {
   chain_wait();
   if (!kFlagged) {  // a CTA for every row
-    const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x);
+    const int slot = load_status_slot(p.status_slots, p.n_slots, threadIdx.x, p.ctl);
     select_one_row<kThreads, false>(p, p.row_begin + blockIdx.x, p.scores + static_cast<size_t>(blockIdx.x) * p.ld, slot);
     return;
   }
@@ -970,7 +971,7 @@ __global__ void __launch_bounds__(kClThreads, kPerSm) select_cluster_kernel(cons
   int32_t* out_idx = p.out_idx + static_cast<size_t>(t) * p.topk;
   float* out_score = p.out_score ? p.out_score + static_cast<size_t>(t) * p.topk : nullptr;
   chain_wait();
-  const int slot = load_status_slot(p.status_slots, p.n_slots, tid);
+  const int slot = load_status_slot(p.status_slots, p.n_slots, tid, p.ctl);
   if (kk == 0) {  // the whole cluster
     add_status(p.ctl, slot);
     if (rank == 0) sort_and_write(list, 0, p.topk, out_idx, out_score, p.N, p.ctl);

@@ -71,3 +71,31 @@ def test_knn_is_clean(tun, debug_library):
     got = gpu_topk(inp, tun)
     assert got[2][0] & lt.LT_STATUS_BOUNDS == 0 and (got[2][3] > 0) == (tun is not None)
     assert np.array_equal(got[0], want[0]) and np.array_equal(got[1].view(np.uint32), want[1].view(np.uint32))
+
+
+@pytest.mark.parametrize("T,N,tun", [(3, 5000, {}), (2, 40000, {}), (70, 9000, dict(path=lt.LT_PATH_FUSED)), (40, 9000, dict(path=lt.LT_PATH_FUSED, grid=296)),
+                                     (40, 9000, dict(path=lt.LT_PATH_FUSED, cap_mult=1, sample_rank=1))])
+def test_status_block_opens_as_in_the_release_build(T, N, tun, debug_library):
+    """A workspace full of ones: the status bytes and counters are cleared by the call's own kernels in this build too, and checked."""
+    inp = make_config("fp8_ar1", T=T, N=N, topk=64)
+    lt.use_library(None)
+    want = run_topk(inp)
+    lt.use_library(debug_library)
+    tun = lt.Tunables(**tun)
+    q, w, k, ks = lt.to_device(inp)
+    ws = lt.alloc_workspace(inp.dtype, T, N, inp.H, inp.D, 64, tun).fill_(0xff)
+    idx, score = torch.empty((T, 64), dtype=torch.int32, device="cuda"), torch.empty((T, 64), device="cuda")
+    lt.lt_indexer_topk_ex(inp.dtype, q, w, k, ks, 64, inp.causal_offset, idx, score, ws, tun)
+    status = lt.lt_read_status(ws)
+    assert status[0] & ~lt.LT_STATUS_FALLBACK == 0 and 0 <= status[4] <= T and status[6] == 0 and status[7] == 0, status
+    assert np.array_equal(idx.cpu().numpy(), want[0]) and np.array_equal(score.cpu().numpy().view(np.uint32), want[1].view(np.uint32))
+
+
+def test_status_block_opens_as_in_the_release_build_knn(debug_library):
+    inp = make_knn(T=70, N=30000, D=64, topk=10)
+    q, x = (torch.from_numpy(a.view(np.int16)).view(torch.bfloat16).cuda() for a in (inp.q, inp.x))
+    ws = torch.full((lt.lt_knn_topk_workspace_bytes(70, 30000, 64, 10),), 0xff, dtype=torch.uint8, device="cuda")
+    idx = torch.empty((70, 10), dtype=torch.int32, device="cuda")
+    lt.lt_knn_topk(q, x, 10, idx, None, ws)
+    status = lt.lt_read_status(ws)
+    assert status[0] & ~lt.LT_STATUS_FALLBACK == 0 and status[6] == 0 and status[7] == 0, status
