@@ -117,9 +117,10 @@ typedef struct lt_tunables {
 
 /* lt_tunables.debug_flags (no counterpart in the paper; used by the library's own tests) */
 #define LT_DEBUG_SKIP_ONE_KTILE 1 /* the first CTA of the fused scan (of the scoring scan where LT_PATH_AUTO takes
-                                     the dense form) never loads its first key tile: with a short
-                                     wait_limit_us this exercises the bounded-wait timeout path without
+                                     the dense form; of lt_knn_topk's alike) never loads its first key tile: with a
+                                     short wait_limit_us this exercises the bounded-wait timeout path without
                                      any fault (the call returns, status has LT_STATUS_TIMEOUT)        */
+#define LT_DEBUG_SKIP_SAMPLE_KTILE 2 /* the same in the scan of the sample                          */
 
 /*
  * Fused indexer top-k (paper Sec. 3.2; Eq. 1 + Eq. 2), 13-argument form.

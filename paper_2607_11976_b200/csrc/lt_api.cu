@@ -78,6 +78,9 @@ Tun resolve_tunables(const lt_tunables* t) {
   return r;
 }
 
+// the test hook of the sample's scan
+int sample_hooks(const Tun& tun) { return (tun.debug_flags & LT_DEBUG_SKIP_SAMPLE_KTILE) != 0 ? LT_DEBUG_SKIP_ONE_KTILE : 0; }
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 int check_problem(int dtype, const void* q, const float* w, const void* k, const float* k_scale, int T, int N, int H, int D) {
@@ -538,6 +541,7 @@ int topk_impl(int dtype, const void* q, const float* w, const void* k, const flo
     p.T = T;
     p.row_begin = 0;
     p.row_end = T;
+    p.debug_flags = sample_hooks(tun);
     p.n_keys = L.n_sample;
     p.causal_offset = INT_MAX / 2;
     p.skip_masked_tiles = 0;
@@ -993,6 +997,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     p.row_end = T;
     p.n_keys = N;
     p.D = D;
+    p.debug_flags = tun.debug_flags;
     p.seg_tiles = knn_seg_tiles(tun, N, grid);
     p.dump = reinterpret_cast<float*>(ws + L.scratch);
     p.dump_ld = L.direct_ld;
@@ -1042,6 +1047,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     p.row_end = T;
     p.n_keys = L.n_sample;
     p.D = D;
+    p.debug_flags = sample_hooks(tun);
     p.seg_tiles = knn_seg_tiles(tun, L.n_sample, grid);
     p.dump = sample;
     p.dump_ld = L.n_sample;
@@ -1063,6 +1069,7 @@ int lt_knn_topk(int dtype, const void* q, const void* x, int T, int N, int D, in
     p.row_end = T;
     p.n_keys = N;
     p.D = D;
+    p.debug_flags = tun.debug_flags;
     p.seg_tiles = knn_seg_tiles(tun, N, grid);
     p.topk = topk;
     p.thr = thr;

@@ -180,6 +180,7 @@ struct KnnScanParams {
   unsigned int wait_limit_us;   // bound of every device-side wait (0 is replaced by the default at launch)
   Control* ctl;
   unsigned char* status_slots;  // as in ScanParams
+  int debug_flags;              // LT_DEBUG_* test hooks
 };
 bool scan_knn_supported(int D);
 cudaError_t launch_scan_knn(int mode, const void* q, int T, const void* x, long long n_keys_view, long long key_pitch_elems,

@@ -235,6 +235,9 @@ knn_scan_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           ++n_done;
           cur_qb = it.qb;
         }
+        // test hook (lt_tunables.debug_flags): CTA 0 loads its first query block and no vectors, so that the UMMA warp's wait for them
+        // runs out and the whole CTA unwinds through the timeout path
+        if ((p.debug_flags & LT_DEBUG_SKIP_ONE_KTILE) && item == 0) break;
         for (int tile = it.tile_lo; tile < it.tile_hi && ok; ++tile) {
           for (int sl = 0; sl < n_slices; ++sl) {
             ok = mbar_wait<40>(smem_u32(&st->bar_empty[stage]), phase ^ 1, abort_flag);

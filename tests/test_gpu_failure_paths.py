@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from paper_2607_11976_b200 import binding as lt
-from workloads import make_config
+from workloads import make_config, make_knn
 
 from gpu_util import assert_matches_oracle, run_topk
 
@@ -54,6 +54,39 @@ def test_dense_form_times_out_and_the_next_call_is_clean(name, T, N):
     idx, score, status = run_topk(inp)
     assert status[0] == 0 and status[3] == 0
     assert_matches_oracle(inp, idx, score, [0, T - 1])
+
+
+# status bits through a byte per CTA to the statistics, and (more CTAs than bytes) straight into the status word
+@pytest.mark.parametrize("grid", [0, 296])
+def test_sample_scan_times_out_and_the_next_call_is_clean(grid):
+    """The same in the scan of the sample, whose status bits another kernel collects."""
+    inp = make_config("fp8_ar1", T=40, N=9000, topk=64)
+    tun = lt.Tunables(path=lt.LT_PATH_FUSED, grid=grid, wait_limit_us=1000, debug_flags=lt.LT_DEBUG_SKIP_SAMPLE_KTILE)
+    idx, _, status = run_topk(inp, tun)
+    assert status[0] & lt.LT_STATUS_TIMEOUT, "the skipped tile of the sample should have made a wait run out"
+    assert idx.min() >= -1 and idx.max() < inp.N
+    idx, score, status = run_topk(inp, lt.Tunables(path=lt.LT_PATH_FUSED, grid=grid))
+    assert status[0] & lt.LT_STATUS_TIMEOUT == 0
+    assert_matches_oracle(inp, idx, score, [0, inp.T - 1])
+
+
+# dense form; fused scan and sample of the sampled form; one query block and several
+@pytest.mark.parametrize("T,path,hook", [(9, lt.LT_PATH_AUTO, lt.LT_DEBUG_SKIP_ONE_KTILE), (9, lt.LT_PATH_FUSED, lt.LT_DEBUG_SKIP_ONE_KTILE),
+                                         (9, lt.LT_PATH_FUSED, lt.LT_DEBUG_SKIP_SAMPLE_KTILE), (150, lt.LT_PATH_FUSED, lt.LT_DEBUG_SKIP_ONE_KTILE),
+                                         (150, lt.LT_PATH_FUSED, lt.LT_DEBUG_SKIP_SAMPLE_KTILE)])
+def test_knn_times_out_and_the_next_call_is_clean(T, path, hook):
+    inp = make_knn(T=T, N=9000, D=128, topk=50)
+    q, x = (torch.from_numpy(a.view(np.int16)).view(torch.bfloat16).cuda() for a in (inp.q, inp.x))
+    ws = torch.full((lt.lt_knn_topk_workspace_bytes(T, 9000, 128, 50),), 0xff, dtype=torch.uint8, device="cuda")
+    bits = []
+    for tun in (lt.Tunables(path=path), lt.Tunables(path=path, wait_limit_us=1000, debug_flags=hook), lt.Tunables(path=path)):
+        idx, score = torch.empty((T, 50), dtype=torch.int32, device="cuda"), torch.empty((T, 50), device="cuda")
+        lt.lt_knn_topk(q, x, 50, idx, score, ws, tun)
+        status = lt.lt_read_status(ws)
+        assert (status[0] & lt.LT_STATUS_TIMEOUT != 0) == (tun.debug_flags != 0)
+        assert idx.min().item() >= -1 and idx.max().item() < 9000
+        bits.append((idx.cpu().numpy(), score.cpu().numpy().view(np.uint32)))
+    assert np.array_equal(bits[0][0], bits[2][0]) and np.array_equal(bits[0][1], bits[2][1])
 
 
 def test_wait_limit_is_not_a_result_tunable():
