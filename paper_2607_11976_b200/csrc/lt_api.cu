@@ -289,18 +289,6 @@ size_t workspace_for(bool fused, int T, int N, int topk, const Tun& tun, int n_g
   return own > other ? own : other;
 }
 
-int sm_count() {
-  static int cached[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-  if (cached[dev] == 0) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-    cached[dev] = n;
-  }
-  return cached[dev];
-}
-
 // causal_offset: of the mask under which tiles that no row of a block can see are skipped
 int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causal_offset = INT_MAX) {
   int n_tiles = (n_keys + kTileKeys - 1) / kTileKeys;

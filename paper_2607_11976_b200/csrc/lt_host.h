@@ -29,6 +29,19 @@ inline cudaError_t allow_smem(const void* kernel, std::atomic<unsigned long long
   return e;
 }
 
+// SMs of the current device, asked for once
+inline int sm_count() {
+  static std::atomic<int> cached[64];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
+    cached[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 // Clusters of `cluster` CTAs of a kernel that the current device (or the part of it that this process may use) holds at once; 0 where
 // it can place none.
 template <typename... Params>

@@ -268,7 +268,7 @@ cudaError_t launch_count_positions(const int32_t* idx, long long n, int N, unsig
   if (n <= 0) return cudaSuccess;
   long long blocks = (n / 4 + 255) / 256;
   if (blocks < 1) blocks = 1;
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  if (blocks > 16 * sm_count()) blocks = 16 * sm_count();
   return launch_chained(count_positions_kernel, static_cast<unsigned int>(blocks), 256, 0, stream, 1, idx, n, N, counts);
 }
 
@@ -295,7 +295,7 @@ cudaError_t launch_rank_counts(const unsigned int* counts, int N, int n_out, uns
   const int passes = (bits_for(max_count) + pos_bits + kRankBits - 1) / kRankBits;
   int blocks = (N + kRankThreads * kRankBatch - 1) / (kRankThreads * kRankBatch);
   if (blocks < 1) blocks = 1;
-  if (blocks > 148 * 2) blocks = 148 * 2;
+  if (blocks > 2 * sm_count()) blocks = 2 * sm_count();
   cudaError_t e = cudaSuccess;
   for (int pass = 0; pass < passes && e == cudaSuccess; ++pass)
     e = launch_chained(rank_pass_kernel, blocks, kRankThreads, 0, stream, 1, counts, N, st, kRankBits * (passes - 1 - pass), pass == 0 ? 1 : 0, pos_bits, n_out);

@@ -854,11 +854,9 @@ __device__ __forceinline__ void select_one_row(const SelectRowsParams& p, int t,
 }
 
 // kFlagged: the rows that row_flag marks (the exact fallback).  They are few or none, and only the device knows: a grid of at most
-// kFlaggedCtas goes through all of them.  (A CTA per
-// row took 21 us, with the scan ahead of it, to find nothing to do among 4096 rows and 39 us, in two rounds, among 8192; now 9 and 12.)
+// two CTAs for every SM goes through all of them.  (A CTA per row took 21 us, with the scan ahead of it, to find nothing to do among 4096 rows and 39 us, in two rounds, among 8192; now 9 and 12.)
 // (The row's select is out of line there: inlined into the loop, 4 rows of 2^20 keys through the fallback 1.20 ms, so 1.08; a CTA per row 1.17.
 // Whole calls with every row flagged, a CTA per row / now: 8 x 16 K 36.0 / 35.1 us, 148 x 8 K 64.8 / 64.2, 4096 x 8 K 939 / 886.)
-constexpr int kFlaggedCtas = 296;
 template <int kThreads>
 __device__ __noinline__ void select_flagged_row(const SelectRowsParams& p, int t, const float* row) {
   select_one_row<kThreads, true>(p, t, row, 0);
@@ -1255,7 +1253,7 @@ cudaError_t launch_sample_stats(const float* sample, int T, int n_sample, int ra
                                 const OpenParams* open, cudaStream_t stream) {
   const OpenParams o = open != nullptr ? *open : OpenParams{};
   // few rows leave the chip idle: a large CTA then shortens the sweeps; with many rows small CTAs overlap better
-  const bool few = T <= 296;
+  const bool few = T <= 2 * sm_count();
   auto launch = [&](auto kernel, int threads) { return launch_chained(kernel, T, threads, 0, stream, 1, sample, n_sample, rank, smin, width, thr, o); };
   if (n_sample < kStatsShort || static_cast<long long>(rank) * kStatsHighShare >= n_sample) return few ? launch(sample_stats_kernel<1024, 0>, 1024) : launch(sample_stats_kernel<256, 0>, 256);
   if (few) return launch(sample_stats_kernel<1024, 8>, 1024);
@@ -1276,7 +1274,7 @@ cudaError_t launch_final_select(const FinalSelectParams& p, cudaStream_t stream)
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(final_select_kernel<512>), done[0]);
   if (e == cudaSuccess) e = allow_smem(reinterpret_cast<const void*>(final_select_kernel<1024>), done[1]);
   if (e != cudaSuccess) return e;
-  if (p.T <= 148) return launch_chained(final_select_kernel<1024>, p.T, 1024, smem, stream, 1, p, sel_cap);
+  if (p.T <= sm_count()) return launch_chained(final_select_kernel<1024>, p.T, 1024, smem, stream, 1, p, sel_cap);
   return launch_chained(final_select_kernel<512>, p.T, 512, smem, stream, 1, p, sel_cap);
 }
 
@@ -1309,7 +1307,8 @@ cudaError_t launch_select_rows_n(const SelectRowsParams& p, int smem, cudaStream
   static std::atomic<unsigned long long> done{0};
   cudaError_t e = allow_smem(reinterpret_cast<const void*>(select_rows_kernel<kThreads, kFlagged>), done);
   if (e != cudaSuccess) return e;
-  const int ctas = kFlagged && p.n_blocks > kFlaggedCtas ? kFlaggedCtas : p.n_blocks;
+  const int most = 2 * sm_count();
+  const int ctas = kFlagged && p.n_blocks > most ? most : p.n_blocks;
   return launch_chained(select_rows_kernel<kThreads, kFlagged>, ctas, kThreads, smem, stream, 1, p);
 }
 }  // namespace
@@ -1321,7 +1320,7 @@ cudaError_t launch_select_rows(const SelectRowsParams& params, cudaStream_t stre
   const int smem = kFineBins * 4 + 2 * static_cast<int>(p.sel_slots) * static_cast<int>(sizeof(uint64_t));
   // many short rows: three small CTAs an SM hide one another's barriers; otherwise a row gets all the threads it can use
   if (p.row_flag != nullptr) return launch_select_rows_n<1024, true>(p, smem, stream);
-  if (p.n_blocks > 296 && p.N <= kSelDirect) return launch_select_rows_n<512, false>(p, smem, stream);
+  if (p.n_blocks > 2 * sm_count() && p.N <= kSelDirect) return launch_select_rows_n<512, false>(p, smem, stream);
   return launch_select_rows_n<1024, false>(p, smem, stream);
 }
 
