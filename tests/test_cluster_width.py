@@ -40,6 +40,16 @@ def test_select_never_asks_for_more_than_the_device_places(rules, widest):
     assert wide == widest
 
 
+def test_select_widths_at_measured_points(rules):
+    """(keys, rows) -> the width that measured best; below, both sides of the line between shares of 8192 and of 16384 keys (32 CTAs of the
+    row count times the width before it is doubled) and of the widths beyond which a share is never short."""
+    for n_keys, n_rows, best in ((20000, 1, 4), (40000, 7, 8), (131072, 1, 8), (131073, 8, 16), (131073, 9, 8)):
+        assert rules.select_width(n_keys, n_rows, 16) == best
+    for n_keys, n_rows, width in ((16385, 16, 4), (16385, 17, 2), (32768, 8, 4), (32769, 8, 8), (32769, 9, 4), (32768, 17, 2), (65536, 8, 8), (65536, 9, 4),
+                                  (65537, 9, 8), (131072, 2, 8)):
+        assert rules.select_width(n_keys, n_rows, 16) == width
+
+
 @pytest.mark.parametrize("widest", [1, 2, 4, 8, 16])
 @pytest.mark.parametrize("ctas_at_once", [16, 148, 592])
 def test_union_runs_in_one_wave(rules, widest, ctas_at_once):
