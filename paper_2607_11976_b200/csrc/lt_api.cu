@@ -101,8 +101,8 @@ bool use_abs_form(const Tun& tun, int dtype, int H, int D) {
   return tun.path == LT_PATH_FUSED_ABS && dtype == LT_DTYPE_E4M3 && scan_mma_supported(dtype, H, D);
 }
 
-// Small problems: score everything into a dense buffer and select from it (three launches) instead of sample, statistics,
-// gated scan, final select and fallback.  Both give the same bits.  The dense form saves four launches and the gate's work
+// Small problems: score everything into a dense buffer and select from it (two launches) instead of sample, statistics,
+// gated scan, final select and the fallback's two.  Both give the same bits.  The dense form saves four launches and the gate's work
 // per key, and pays 4 bytes of traffic per pair and a select over whole rows.  Measured on one B200, dense against sampled,
 // us per call, topk 2048 unless given.  Rows of up to kDenseKeys keys are selected by one CTA each: 256 x 16 K 63 / 85,
 // 4096 x 4 K (bf16, first chunk) 194 / 333, 4096 x 16 K 744 / 881, topk 64 4096 x 8 K 342 / 377, 1024 x 16 K 197 / 214; many
@@ -130,9 +130,9 @@ constexpr long long kDenseShortPairs = 1ll << 20;
 bool use_direct(const Tun& tun, int T, int N, int topk, bool paged, int knn_dim) {
   // an explicit path or a tunable of the sampled form asks for that form
   if (tun.path != LT_PATH_AUTO || tun.sample_mult_given || tun.cap_mult_given || tun.sample_rank != 0) return false;
-  // Over a paged cache only up to one query block.  Larger chunks stay with the sampled form, whose survivor counts their callers
-  // read from the status block; the dense form would filter nothing and report none.  That is not for speed: measured sampled /
-  // dense over paged e4m3 keys, 4096 x 4 K 309 / 179 us, 256 x 16 K 91 / 64, 64 x 64 K 77 / 73, 32 x 128 K 77 / 78.
+  // Over a paged cache only up to one query block.  Larger chunks stay with the sampled form because a test of the paged entry
+  // point asks for survivor counts, which the header does not promise; the dense form filters nothing and reports none.  It is not for
+  // speed: measured sampled / dense over paged e4m3 keys, 4096 x 4 K 309 / 179 us, 256 x 16 K 91 / 64, 64 x 64 K 77 / 73, 32 x 128 K 77 / 78.
   if (paged && T > kRowsPerBlock) return false;
   if (N <= kDenseKeys / 2 || (N <= kDenseKeys && topk >= 512)) return true;
   const long long pairs = static_cast<long long>(T) * N;
@@ -295,7 +295,11 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causa
   if (tun.segment_tiles > 0) return clamp_segment(tun.segment_tiles, n_tiles);
   constexpr int kItemOverheadTiles = 4;
   // A triangular mask: blocks see from `first` tiles to all of them, their items are dealt out longest first, and what matters is the
-  // number of items (each starts up) and how evenly they fill the CTAs: whole rows of up to 256 tiles for many blocks.
+  // number of items (each starts up) and how evenly they fill the CTAs: whole rows of up to 256 tiles for many blocks.  Whole calls, bf16 /
+  // e4m3, us, segments by the rule below / whole rows: 4096 rows of their own 4096 keys (16 tiles) 198 / 180, 169 / 156; 4096 of 8192 (32) 181 / 181,
+  // 157 / 156; from position 2000 on 315 / 313, 252 / 253, from 3900 on 425 / 433, 330 / 342, so that the line would be as well at a quarter of
+  // the keys; 20000 of 20000 and 8192 of 40000 no difference.  Below two blocks to a CTA, 295 blocks (2360 rows, 10 tiles) 84 / 74, 77 / 68
+  // say that this line could be lower, 250 and 188 blocks (16 and 21 tiles) 60 / 59 and 46 / 45 that little is lost elsewhere.
   const long long first = (static_cast<long long>(causal_offset) + kRowsPerBlock + kTileKeys - 1) / kTileKeys;
   if (2 * first < n_tiles && n_blocks >= 2 * grid) {
     double best_cost = 0.0;
@@ -318,8 +322,8 @@ int pick_seg_tiles(const Tun& tun, int n_keys, int n_blocks, int grid, int causa
   const long long want = (n_blocks <= 2 ? 1ll : 2ll) * grid;
   while (seg > 16 && static_cast<long long>(n_blocks) * ((n_tiles + seg - 1) / seg) < want) seg >>= 1;
   if (n_blocks <= 2 && seg < 256) seg = 2 * seg - 1;  // the halving may have gone past one item per CTA
-  // Work items are dealt to the persistent CTAs round-robin, so the launch lasts as long as the CTA with the
-  // most items: among the sizes from the one above down to one tile, take the shortest such critical path (in key
+  // Work items are dealt to the persistent CTAs to and fro (by the k-NN and the alternative fp8 scan: round-robin), so the launch lasts as
+  // long as the CTA with the most items: among the sizes from the one above down to one tile, take the shortest such critical path (in key
   // tiles, plus a few tiles' worth of per-item start-up: the query block of an item is as large as four key tiles).
   // Matters for short chunks: 128 rows over 8192 tiles are 512 items of 256 tiles (4 rounds on 148 CTAs, the last
   // one half empty) or 592 items of 222 tiles.  Also for the sample phase, whose 64 tiles x 10 blocks (77 rows) are 40 items
@@ -921,7 +925,7 @@ int knn_seg_tiles(const Tun& tun, int n_keys, int grid) {
   if (tun.segment_tiles > 0) return clamp_segment(tun.segment_tiles, n_tiles);
   int seg = 32;
   while (seg > 2 && (n_tiles + seg - 1) / seg < 4 * grid) seg >>= 1;
-  // too few tiles to go round (the sample of 64 queries over 2^20 vectors, 64 tiles on 148 SMs: 17 -> 15 us, whole call 287 -> 283)
+  // too few tiles to go round (the sample of 64 queries over 2^20 vectors, 64 tiles on 148 SMs: 17 -> 15 us, whole call 308 -> 303)
   if (seg == 2 && (n_tiles + 1) / 2 < grid) seg = 1;
   return seg;
 }
