@@ -99,7 +99,8 @@ typedef struct lt_tunables {
                         min(8192, keys the sample is drawn from / 32)), but no more than 64 * (keys the
                         sample is drawn from) / topk, which is what the default sample_rank needs; an
                         explicit value is taken as given                                           */
-  int segment_tiles; /* key tiles (128 keys each) per work item (default 256)            */
+  int segment_tiles; /* key tiles (128 keys each) per work item (default: by the sizes, at most 256);
+                        more than the context has means all of them                          */
   int grid;          /* CTAs of the scan kernel (default: number of SMs)                 */
   int sample_rank;   /* initial gate = lower edge of the bin holding the sample's r-th largest
                         score.  0 (default): r = ceil(m + 5 sqrt(m) + 5) capped at topk, where
