@@ -42,6 +42,13 @@ def test_union_masks_by_whole_rows(T, topk, N, group, shift):
         assert np.array_equal(mask[t], pack_mask_words(masks[t], words)), t
 
 
+# whole rows beside every size of bitmap, by CTAs of both sizes, around the longest single window, and one position to a row
+@pytest.mark.parametrize("T,topk,N,group", [(32, 2048, 1200000, 32), (32, 2048, 1572864, 32), (32, 2048, 1572865, 32), (8, 2048, 200000, 8), (8, 2048, 400000, 8),
+                                            (130, 1024, 262145, 128), (33, 2044, 90000, 32), (5, 4, 40, 5), (1, 4096, 131072, 1)])
+def test_union_masks_by_whole_rows_everywhere(T, topk, N, group):
+    test_union_masks_by_whole_rows(T, topk, N, group, 0)
+
+
 # around a digit of 2048 positions, a CTA's 4096, one block of 256 keys more or less, and as many keys as a workspace holds
 @pytest.mark.parametrize("N,n_out", [(2047, 256), (2048, 257), (2049, 255), (4096, 4096), (4097, 1), (8193, 8192), (1 << 18, 6144)])
 def test_frequent_positions_around_digits(N, n_out):
